@@ -7,18 +7,18 @@
 // alignment a traceback from the end selects when it prefers the diagonal, then F,
 // then E, and a gap open over an extension (its begin, identities, columns).
 //
-// Pass 1 (the whole matrix, every pair): score and end only.  A warp takes two pairs
-//   that share the query (candidate lists are grouped by i; within a run of pairs of
-//   one query they are taken in order of target length, so the two matrices match)
-//   and holds them in the two 16-bit halves of each register, so one 16x2 maximum or
-//   one 32-bit add advances both.  Lane l owns up to 16 consecutive query rows and at
-//   step s computes column j = s - l, taking H/F of the row above from lane l-1
+// Pass 1 (the whole matrix, every pair): score and end only.  A group of 8, 16 or 32 lanes
+//   takes two pairs that share the query (candidate lists are grouped by i; within a run
+//   of pairs of one query they are taken in order of target length, so the matrices of a
+//   warp match) and holds them in the two 16-bit halves of each register, so one 16x2
+//   maximum or add advances both.  Lane l owns up to 32 consecutive query rows and at step
+//   s computes column j = s - l, taking H/F of the row above from lane l-1
 //   (__shfl_up_sync).  Scores come from a biased query profile in shared memory
-//   (one byte per [target residue][query row]) shared by every warp of the CTA.  Each row
-//   keeps a key (H << 16 | 65535 - j) of its first maximum; the end is the first row
-//   with the best score, at that row's first maximum: the row-major first maximum.
+//   (one byte per [target residue][query row]) shared by every warp of the CTA.  Each lane
+//   keeps its best cell (H, row, column) and looks at a column only when it holds a value
+//   that can replace the group's best, so the end is the row-major first maximum.
 //   Pass 1 also stores, per pair of query rows, the largest H it met there.
-//   Queries longer than one stripe of 32 * 16 rows go in stripes whose last row is
+//   Queries longer than one stripe of 32 * 32 rows go in stripes whose last row is
 //   handed on through a per-warp buffer.
 // Pass 2 (its own kernel, one warp per pair; a band around the path): an anchored DP
 //   over the reversed prefixes from the end (ei, ej), row by row with up to 64 columns
@@ -48,9 +48,9 @@ namespace {
 constexpr int NEG = -1000000000;
 constexpr int SW_THREADS = 256;
 constexpr int SW_WARPS = SW_THREADS / 32;
-constexpr int STRIPE1 = 512;               // rows per stripe in pass 1 at 16 rows per lane
+constexpr int STRIPE1 = 512;               // profile bytes per residue come in whole multiples
 constexpr int PAD_SCORE = -30000;
-constexpr int SEG_MAX = 128;               // pairs per scheduling segment
+constexpr int SEG_MAX = 512;               // pairs per scheduling segment, at most
 
 struct sw_score_out {                      // pass 1 result per pair
     int32_t score;
@@ -70,23 +70,70 @@ __device__ __forceinline__ bool cannot_cover(const sw_score_out &r, int lq, int 
 }
 
 // ---------------------------------------------------------------------------------
-// segments: runs of pairs with the same query, at most SEG_MAX long
+// segments: runs of pairs with the same query, at most seg_len(pairs of the call) long
 // ---------------------------------------------------------------------------------
+// A power of two from 16 to SEG_MAX that leaves about 1,024 full segments, three or more for
+// each resident CTA: longer segments share a profile and balance the warps of a CTA, shorter
+// ones the CTAs.
+__device__ __forceinline__ int seg_len(int64_t n) {
+    int len = SEG_MAX;
+    while (len > 16 && n < (int64_t)len * 1024) len >>= 1;
+    return len;
+}
+
 // dn (captured launches): the pair count in device memory, n the capacity; 0 past it.
 __global__ void k_seg_flags(const pastis_cand *pairs, int64_t n, uint32_t *flags, const int64_t *dn) {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const int64_t m = dn ? *dn : n;
-    flags[p] = p < m && (p == 0 || (p % SEG_MAX) == 0 || pairs[p].i != pairs[p - 1].i) ? 1u : 0u;
+    flags[p] = p < m && (p == 0 || (p & (seg_len(m) - 1)) == 0 || pairs[p].i != pairs[p - 1].i) ? 1u : 0u;
 }
 
-__global__ void k_seg_starts(const uint32_t *flags, const uint32_t *off, int64_t n, int64_t *seg_start,
-                             const int64_t *dn) {
+// Segments run in order of query length, longest first (bins of 16 residues): the CTAs at
+// work at one time then run the same few of pass 1's sixteen loop bodies, which together
+// exceed the instruction cache (pass 1 of 10^6 pairs 51.2 ms in input order, 46.9 ms so),
+// and the last segments taken are the shortest.
+constexpr int SEG_BINS = 128;
+__device__ __forceinline__ int seg_bin(int64_t m) { return SEG_BINS - 1 - (int)min((int64_t)SEG_BINS - 1, m >> 4); }
+
+// Also counts the segments of each length bin (hist, zeroed by the caller).
+__global__ void k_seg_starts(const pastis_cand *pairs, const int64_t *qoffsets, const uint32_t *flags,
+                             const uint32_t *off, int64_t n, int64_t *seg_start, uint32_t *hist, const int64_t *dn,
+                             const int *chk) {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const int64_t m = dn ? *dn : n;
-    if (p < m && flags[p]) seg_start[off[p]] = p;
+    if (p < m && flags[p]) {
+        seg_start[off[p]] = p;
+        if (!(chk && (chk[0] | chk[1]))) {       // a refused batch's indexes are not to be followed
+            const int i = pairs[p].i;
+            atomicAdd(&hist[seg_bin(qoffsets[i + 1] - qoffsets[i])], 1u);
+        }
+    }
     if (p == m - 1) seg_start[off[p] + flags[p]] = m;
+}
+
+// order[] = the segments by length bin (any order within a bin); taken: one zeroed counter
+// per bin.
+__global__ void __launch_bounds__(256) k_seg_order(const pastis_cand *pairs, const int64_t *qoffsets,
+                                                   const int64_t *seg_start, int64_t n_seg, const uint32_t *d_nseg,
+                                                   const uint32_t *hist, uint32_t *taken, uint32_t *order,
+                                                   const int *chk) {
+    if (d_nseg) n_seg = *d_nseg;
+    if (chk && (chk[0] | chk[1])) return;
+    if ((int64_t)blockIdx.x * blockDim.x >= n_seg) return;
+    __shared__ uint32_t s_base[SEG_BINS];
+    if (threadIdx.x < SEG_BINS) {
+        uint32_t b = 0;
+        for (int x = 0; x < (int)threadIdx.x; ++x) b += hist[x];
+        s_base[threadIdx.x] = b;
+    }
+    __syncthreads();
+    const int64_t sg = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (sg >= n_seg) return;
+    const int i = pairs[seg_start[sg]].i;
+    const int b = seg_bin(qoffsets[i + 1] - qoffsets[i]);
+    order[s_base[b] + atomicAdd(&taken[b], 1u)] = (uint32_t)sg;
 }
 
 // ---------------------------------------------------------------------------------
@@ -119,194 +166,260 @@ __device__ __forceinline__ uint32_t madd(uint32_t a, uint32_t b, uint32_t c) {
 
 struct end_cell { int h, i, j; };
 
-// Rows per lane: as few stripes as 16 rows per lane allow, plus `extra` stripes (the
-// layout the tuner picked for the query's length bin), then the smallest row count
-// (at least 2) that covers the query in that many stripes.  More stripes pad fewer rows
-// but sweep the target more often; the layout changes no result.
-__device__ __forceinline__ int rows_per_lane(int m, int extra) {
-    const int ns = max(1, (m + 511) / 512) + extra;
-    const int per = (m + 32 * ns - 1) / (32 * ns);
-    return min(16, max(2, per));
+// The profile holds one signed byte per (target residue, query row): score + o, and
+// o - 64 (the lowest score) for the pad residue and past the query.  A group of G lanes
+// holds G * LR query rows (a stripe), lane l the LR consecutive rows l * LR ..; per stripe
+// the bytes lie in planes of 16 rows, lane l's rows 16 p .. 16 p + 15 at p * 16 G + 16 l, so
+// a lane reads its rows of one column with one 16-byte load per plane and the lanes of a
+// group read consecutive words.
+constexpr int SLOT = 16;
+constexpr int LR_MAX = 32;
+
+// The layout of one query of m residues: G lanes a pair, LR (even) rows a lane, ns stripes.
+// A column step costs a lane about 10 cycles of the integer pipe per row (five 16x2
+// instructions at half rate) and STEP_ROWS rows' worth of work that does not depend on
+// LR (shuffles, window, addresses, the test for a new best), and a sweep takes n + G - 1
+// steps; so few lanes with many rows each cost least per cell, but leave more pairs to a
+// grab.  The fewest cycles of the CTA's slowest warp over the cnt pairs of the segment,
+// with nt the longest target, decide.  More than one stripe takes 32 lanes.  `extra` (the
+// layout the tuner picked for the query's length bin): 32 lanes and that many stripes more
+// than needed, which pad fewer rows but sweep the target more often.  A query whose
+// profile would not fit prow_cap bytes per residue so takes stripes of 512 rows, the densest
+// profile.  The layout changes no result.
+constexpr int STEP_ROWS = 3;
+struct sw_tile { int G, lr, ns, prow; };
+
+__device__ __forceinline__ sw_tile make_tile(int m, int G, int ns) {
+    sw_tile t;
+    const int per = (m + G * ns - 1) / (G * ns);
+    t.G = G;
+    t.ns = ns;
+    t.lr = min(LR_MAX, max(2, (per + 1) & ~1));
+    t.prow = ns * G * (t.lr > SLOT ? 2 * SLOT : SLOT);
+    return t;
 }
 
-// The profile holds one signed byte per (target residue, query row): score + o, and
-// o - 64 (the lowest score) for the pad residue and past the query.  Rows are laid out
-// per stripe and lane in 16-byte slots (slot of lane l in stripe st at st * 512 + l * 16,
-// row r of the lane at +r), so a lane reads its rows of one column with one 16-byte load.
-constexpr int SLOT = 16;
-constexpr int STRIPE_BYTES = 32 * SLOT;
+__device__ sw_tile pick_tile(int m, int extra, int cnt, int nt, int prow_cap) {
+    const int need = max(1, (m + 32 * LR_MAX - 1) / (32 * LR_MAX));
+    sw_tile best = make_tile(m, 32, need + extra);
+    if (extra == 0 && need == 1) {
+        int cost = 0x7FFFFFFF;
+        for (int G = 32; G >= 8 && m <= G * LR_MAX; G >>= 1) {
+            const sw_tile t = make_tile(m, G, 1);
+            const int grabs = (cnt * G + 63) / 64;                  // of 64 / G pairs
+            const int c = ((grabs + SW_WARPS - 1) / SW_WARPS) * (nt + G) * (t.lr + STEP_ROWS);
+            if (c < cost) { cost = c; best = t; }
+        }
+    }
+    if (best.prow > prow_cap) {
+        best.G = 32;
+        best.lr = SLOT;
+        best.ns = max(1, (m + 511) / 512);
+        best.prow = best.ns * 512;
+    }
+    return best;
+}
 
 // One column of a lane's LR rows for both pairs.  Ho = H - o is kept per row (it feeds
-// E, F and the keys), so the diagonal term is Ho(i-1, j-1) + (score + o).  The key of a
-// row keeps (Ho << 16 | 65535 - j) of its best column as a signed word: the largest Ho,
-// then the first column, i.e. the first maximum of that row.  Pair A's key is
-// Ho * 2^16 + jt (pair B's half leaves the word), pair B's is (Ho & 0xFFFF0000) | jt.
-template <int LR>
-__device__ __forceinline__ void column2(const uint8_t *__restrict__ pa, const uint8_t *__restrict__ pb,
-                                        uint32_t (&Ho)[LR], uint32_t (&E)[LR], uint32_t (&kA)[LR],
-                                        uint32_t (&kB)[LR], uint32_t hdiag, uint32_t &f, uint32_t &hup, uint32_t jt,
-                                        uint32_t sh16, uint32_t OP, uint32_t nEP) {
-    const uint4 x = *reinterpret_cast<const uint4 *>(pa), y = *reinterpret_cast<const uint4 *>(pb);
-    const uint32_t wa[4] = {x.x, x.y, x.z, x.w}, wb[4] = {y.x, y.y, y.z, y.w};
+// E, F and the maxima), so the diagonal term is Ho(i-1, j-1) + (score + o).  rm keeps the
+// largest Ho of each pair of rows over the columns (pass 2's bound); cm returns the
+// largest Ho of this column, and tm where no row exceeds it.
+template <int LR, int PLANE>
+__device__ __forceinline__ uint32_t column2(const uint8_t *__restrict__ pa, const uint8_t *__restrict__ pb,
+                                            uint32_t (&Ho)[LR], uint32_t (&E)[LR], uint32_t (&rm)[LR / 2],
+                                            uint32_t hdiag, uint32_t &f, uint32_t &hup, uint32_t tm, uint32_t OP,
+                                            uint32_t nEP) {
     // byte r of the two words into the low and high halves, sign-extended
     constexpr uint32_t SEL[4] = {0xc480u, 0xd591u, 0xe6a2u, 0xf7b3u};
+    constexpr int PLANES = (LR + SLOT - 1) / SLOT;
+    uint32_t wa[4 * PLANES], wb[4 * PLANES];
+#pragma unroll
+    for (int p = 0; p < PLANES; ++p) {
+        const uint4 x = *reinterpret_cast<const uint4 *>(pa + p * PLANE);
+        const uint4 y = *reinterpret_cast<const uint4 *>(pb + p * PLANE);
+        wa[4 * p] = x.x; wa[4 * p + 1] = x.y; wa[4 * p + 2] = x.z; wa[4 * p + 3] = x.w;
+        wb[4 * p] = y.x; wb[4 * p + 1] = y.y; wb[4 * p + 2] = y.z; wb[4 * p + 3] = y.w;
+    }
+    uint32_t cm = tm;
+    uint32_t d = __vadd2(hdiag, prmt_sx(wa[0], wb[0], SEL[0]));   // H(i-1, j-1) + score
 #pragma unroll
     for (int r = 0; r < LR; ++r) {
-        const uint32_t s = prmt_sx(wa[r >> 2], wb[r >> 2], SEL[r & 3]);
-        const uint32_t d = __vadd2(hdiag, s);                 // H(i-1, j-1) + score
-        E[r] = __viaddmax_s16x2(E[r], nEP, Ho[r]);            // E(i, j) = max(E(i, j-1) - e, H(i, j-1) - o)
-        f = __viaddmax_s16x2(f, nEP, hup);                    // F(i, j) = max(F(i-1, j) - e, H(i-1, j) - o)
-        const uint32_t h = __vimax3_s16x2_relu(d, E[r], f);   // H = max(0, diagonal, E, F)
-        hdiag = Ho[r];
-        Ho[r] = __vsub2(h, OP);
+        // the next row's diagonal term is formed before this row's Ho is replaced, so each
+        // row keeps its register from column to column
+        uint32_t dn = 0u;
+        if (r + 1 < LR) dn = __vadd2(Ho[r], prmt_sx(wa[(r + 1) >> 2], wb[(r + 1) >> 2], SEL[(r + 1) & 3]));
+        E[r] = __viaddmax_s16x2(E[r], nEP, Ho[r]);                // E(i, j) = max(E(i, j-1) - e, H(i, j-1) - o)
+        f = __viaddmax_s16x2(f, nEP, hup);                        // F(i, j) = max(F(i-1, j) - e, H(i-1, j) - o)
+        Ho[r] = __vsub2(__vimax3_s16x2_relu(d, E[r], f), OP);     // H = max(0, diagonal, E, F)
         hup = Ho[r];
-        kA[r] = (uint32_t)max((int)kA[r], (int)madd(Ho[r], sh16, jt));
-        kB[r] = (uint32_t)max((int)kB[r], (int)((Ho[r] & 0xFFFF0000u) | jt));
+        if (r & 1) {
+            rm[r >> 1] = __vimax3_s16x2(rm[r >> 1], Ho[r - 1], Ho[r]);
+            cm = __vimax3_s16x2(cm, Ho[r - 1], Ho[r]);
+        }
+        d = dn;
     }
+    return cm;
 }
 
-// The registers a pass-1 stripe sweep carries from column to column, and the values
-// that stay fixed over the sweep.
-template <int LR>
-struct pass1_state {
-    uint32_t (&Ho)[LR], (&E)[LR], (&kA)[LR], (&kB)[LR];
-    uint32_t &hd, &out_h, &out_f, &out_t, &twin, &tnext;
+// A column that may hold a new end for one half (HI: the high one): the lane's largest Ho
+// of the column and its first row, merged into the lane's best (larger Ho, then smaller
+// row; a later column of the same row never replaces an earlier one), then the group's:
+// its best and the first lane holding it.  Returns the value a cell of this lane must
+// exceed to matter: the group's best for the lanes behind the holder, whose rows are
+// larger, one less for the holder and the lanes before it.
+template <int G, int LR, bool HI>
+__device__ __forceinline__ int note_best(const uint32_t (&Ho)[LR], bool mine, int row0, int j, int lg, uint32_t sh16,
+                                         int &bv, int &brow, int &bcol) {
+    int kk = (int)0x80000000;
+#pragma unroll
+    for (int r = 0; r < LR; ++r) {
+        const uint32_t k = HI ? (Ho[r] & 0xFFFF0000u) | (uint32_t)(LR - 1 - r) : madd(Ho[r], sh16, (uint32_t)(LR - 1 - r));
+        kk = max(kk, (int)k);
+    }
+    const int v = kk >> 16, row = row0 + LR - 1 - (kk & 0xFFFF);
+    if (mine && (v > bv || (v == bv && row < brow))) { bv = v; brow = row; bcol = j; }
+    int gk = bv * 64 + (63 - lg);
+    for (int d = G >> 1; d > 0; d >>= 1) gk = max(gk, __shfl_xor_sync(0xffffffffu, gk, d));
+    const int holder = 63 - (gk & 63);
+    return (gk >> 6) - (lg > holder ? 0 : 1);
+}
+
+// One group's two pairs in pass 1: targets, columns and the outputs.
+struct pair_io {
+    const uint8_t *tA, *tB;
+    int nA, nB;
+    int16_t *bmA, *bmB;                        // null: the half holds no pair of its own
 };
-struct pass1_consts {
-    const uint8_t *pr;
-    int prow8;
-    const uint8_t *tA;
-    int nA;
-    const uint8_t *tB;
-    int nB, n, lane;
-    bool first_stripe, hand_on;
-    uint32_t INIT, sh16, OP, nEP;
-    const uint2 *in_buf;
-    uint2 *out_buf;
-};
 
-// The target window at step s (a multiple of 32): columns [s, s + 32) move to twin,
-// and lane k loads column s + 32 + k of both targets into tnext.
-template <int LR>
-__device__ __forceinline__ void pass1_window(const int s, const pass1_consts &c, pass1_state<LR> &st) {
-    st.twin = st.tnext;
-    const int x = s + 32 + c.lane;
-    st.tnext = (x < c.nA ? (uint32_t)c.tA[x] : (uint32_t)PAD_RES) |
-               ((x < c.nB ? (uint32_t)c.tB[x] : (uint32_t)PAD_RES) << 16);
-}
-
-// One step s of the wavefront: lane l computes column j = s - l of its rows.  CHECKED
-// tests that j is a column (the ramps); `window` = false when the caller loads the
-// target windows itself.
-template <int LR, bool CHECKED>
-__device__ __forceinline__ void pass1_step(const int s, const pass1_consts &c, pass1_state<LR> &st,
-                                           const bool window = true) {
-    const int lane = c.lane, j = s - lane;
-    if (window && s > 0 && (s & 31) == 0) pass1_window<LR>(s, c, st);
-    const uint32_t tw = __shfl_sync(0xffffffffu, st.twin, s & 31);
-    uint32_t hu = __shfl_up_sync(0xffffffffu, st.out_h, 1);
-    uint32_t fu = __shfl_up_sync(0xffffffffu, st.out_f, 1);
-    uint32_t tt = __shfl_up_sync(0xffffffffu, st.out_t, 1);
-    if (lane == 0) {
-        tt = tw;
-        if (c.first_stripe) { hu = c.INIT; fu = c.INIT; }
-        else if (!CHECKED || j < c.n) { const uint2 v = c.in_buf[j]; hu = v.x; fu = v.y; }
-    }
-    if (!CHECKED || (j >= 0 && j < c.n)) {
-        uint32_t f = fu, hup = hu;
-        column2<LR>(c.pr + (int)(tt & 0xFFFFu) * c.prow8, c.pr + (int)(tt >> 16) * c.prow8, st.Ho, st.E, st.kA,
-                    st.kB, st.hd, f, hup, 65535u - (uint32_t)j, c.sh16, c.OP, c.nEP);
-        st.hd = hu;
-        st.out_h = hup; st.out_f = f; st.out_t = tt;
-        if (lane == 31 && c.hand_on) c.out_buf[j] = make_uint2(hup, f);
-    }
-}
-
-// Pass 1 over the whole matrix of two pairs with the same query: pair A (target tA,
-// nA columns) in the low halves, pair B in the high halves.  Lane l owns LR
-// consecutive query rows and at step s does column j = s - l, taking the row above from
-// lane l-1; a stripe is 32 * LR rows, its last row handed on through buf.  Columns
-// past the shorter target use the pad residue, which scores -64 against every row: a
-// cell there stays below the best score of its own pair, so it never becomes the end.
-// Lane 0 takes the target residues from a window of 32 columns that the warp loads one
-// window ahead.  Returns each pair's best score and its first maximum in row-major
-// order, and writes bm[g] = the largest H on rows 2g and 2g+1 (pass 2's bound).
-template <int LR>
-__device__ void score_pair(const uint8_t *__restrict__ prof, int prow8, const uint8_t *__restrict__ tA, int nA,
-                           const uint8_t *__restrict__ tB, int nB, int m, int o, int e, uint32_t one, uint2 *buf,
-                           int sstride, int16_t *bmA, int16_t *bmB, end_cell *ra, end_cell *rb) {
-    constexpr int STRIPE = 32 * LR;
-    const int lane = threadIdx.x & 31;
-    const int n = max(nA, nB);
+// Pass 1 over the whole matrices of the warp's 32 / G groups, two pairs with the same
+// query each: pair A (target tA, nA columns) in the low halves, pair B in the high halves.
+// Lane l of a group owns LR consecutive query rows and at step s does column j = s - l,
+// taking the row above from lane l-1; with several stripes (G = 32 only) a stripe's last row
+// is handed on through buf.  Columns outside a target (before its first: the wavefront's
+// ramp; past its last) use the pad residue, which scores -64 against every row: before
+// the first column that leaves every state at its initial value, and past the last no cell
+// reaches the best of a smaller row, so no step tests its range.  Every lane holds one
+// column of the group's target window and takes the next window's when the step that
+// needs it comes, so one shuffle per step gives each lane its column's residues.
+// The end (the largest H, then the smallest row, then the smallest column) is kept per
+// lane and looked at only in the steps whose column holds a value that can replace it
+// (note_best): on random pairs 20 of 325 steps a pair; tracking each row's first maximum
+// in a 32-bit key instead cost three integer-pipe and one multiply-add instruction per row.
+// What bounds it is the integer pipe: per register and row prmt, two maxima for E and F, one
+// for H and one for both running maxima, at half rate.  Measured (2.00e11 cells, 10^6
+// pairs of 20,000 proteins with 25 substitutes): 69.6 ms with 32 lanes a pair, at most 16
+// rows a lane and a key per row, 44.2 ms so (4,520 GCUPS); queries of 1,000 residues 43.7
+// -> 25.3 ms.  A function of its own, so that what the caller keeps is saved around it
+// instead of spilled inside its loop (1% faster).
+// Writes bm[g] = the largest H on rows 2g and 2g+1 (pass 2's bound).
+template <int G, int LR, bool MULTI>
+__device__ __noinline__ void score_group(const uint8_t *__restrict__ prof, const sw_tile tl, const pair_io &io, int m, int o, int e,
+                            uint32_t one, uint2 *buf, int sstride, end_cell *ra, end_cell *rb) {
+    const int lg = threadIdx.x & (G - 1);
+    const int n = __reduce_max_sync(0xffffffffu, max(io.nA, io.nB));
+    constexpr int PLANE = G * SLOT, SBYTES = LR > SLOT ? 2 * PLANE : PLANE;
+    const int nstripes = MULTI ? tl.ns : 1;
     const uint32_t INIT = ((uint32_t)(-o) & 0xFFFFu) * P2;  // -o in both halves
     const uint32_t OP = (uint32_t)o * P2, nEP = ((uint32_t)(-e) & 0xFFFFu) * P2;
     const uint32_t sh16 = one << 16;                        // 2^16 at run time (keeps the multiply-add)
-    int bA = -1, iA = 0, jA = 0, bB = -1, iB = 0, jB = 0;
-    const int nstripes = (m + STRIPE - 1) / STRIPE;
+    constexpr uint32_t PADS = (uint32_t)PAD_RES * P2;
+    int vA = -o, iA = 0, jA = 0, vB = -o, iB = 0, jB = 0;   // the lane's best Ho, its row and column
+    uint32_t tm = INIT;                                     // what a column must exceed to matter, per half
     for (int stripe = 0; stripe < nstripes; ++stripe) {
-        const int row0 = stripe * STRIPE + lane * LR;
-        uint32_t Ho[LR], E[LR], kA[LR], kB[LR];
+        const int row0 = (stripe * G + lg) * LR;
+        uint32_t Ho[LR], E[LR], rm[LR / 2];
 #pragma unroll
-        for (int r = 0; r < LR; ++r) { Ho[r] = INIT; E[r] = INIT; kA[r] = 0x80000000u; kB[r] = 0x80000000u; }
+        for (int r = 0; r < LR; ++r) { Ho[r] = INIT; E[r] = INIT; rm[r >> 1] = INIT; }
         uint32_t hd = INIT;                                 // Ho(row0 - 1, j - 1)
-        uint32_t out_h = INIT, out_f = INIT, out_t = 0;
+        uint32_t out_h = INIT, out_f = INIT;
+        const bool take = MULTI && stripe > 0, hand_on = MULTI && stripe + 1 < nstripes;
         const uint2 *in_buf = buf + (size_t)(stripe & 1) * sstride;
         uint2 *out_buf = buf + (size_t)((stripe + 1) & 1) * sstride;
-        const bool last = stripe + 1 == nstripes;
-        const uint8_t *pr = prof + stripe * STRIPE_BYTES + lane * SLOT;
-        // target residues of columns [w, w + 32) (lane k holds column w + k), and the next window
-        uint32_t twin = (lane < nA ? (uint32_t)tA[lane] : (uint32_t)PAD_RES) |
-                        ((lane < nB ? (uint32_t)tB[lane] : (uint32_t)PAD_RES) << 16);
-        uint32_t tnext = (32 + lane < nA ? (uint32_t)tA[32 + lane] : (uint32_t)PAD_RES) |
-                         ((32 + lane < nB ? (uint32_t)tB[32 + lane] : (uint32_t)PAD_RES) << 16);
-        // Steps [0, 31) and [n, n + 31) are the wavefront's ramps, where some lanes have
-        // no column; in [31, n) every lane has one, so those steps skip the range tests
-        // and run in runs that end at the next 32-column window boundary, the window
-        // loaded once per run instead of tested at every step (measured on the 100k
-        // step: pass 1 -7% against one loop with the tests in every step).
-        pass1_state<LR> st{Ho, E, kA, kB, hd, out_h, out_f, out_t, twin, tnext};
-        const pass1_consts pc{pr, prow8, tA, nA, tB, nB, n, lane, stripe == 0, !last, INIT, sh16, OP, nEP,
-                              in_buf, out_buf};
-        int s = 0;
-        for (const int s_up = min(31, n + 31); s < s_up; ++s) pass1_step<LR, true>(s, pc, st);
-        while (s < n) {
-            if ((s & 31) == 0) pass1_window<LR>(s, pc, st);
-            const int ce = min(n, (s | 31) + 1);          // up to the next window boundary
-#pragma unroll 2
-            for (; s < ce; ++s) pass1_step<LR, false>(s, pc, st, false);
+        const uint8_t *pr = prof + stripe * SBYTES + lg * SLOT;
+        if (take) {                                         // later rows must beat the earlier stripes' best
+            int a = vA, b = vB;
+            for (int d = G >> 1; d > 0; d >>= 1) {
+                a = max(a, __shfl_xor_sync(0xffffffffu, a, d));
+                b = max(b, __shfl_xor_sync(0xffffffffu, b, d));
+            }
+            tm = ((uint32_t)a & 0xFFFFu) | ((uint32_t)b << 16);
         }
-        for (; s < n + 31; ++s) pass1_step<LR, true>(s, pc, st);
-        // this lane's rows: first maximum per pair, and the row-pair bounds.  With LR odd
-        // every other lane starts on an odd row, so the pair (2g, 2g+1) may straddle two
-        // lanes: the lane holding row 2g takes row 2g+1's maximum from the next lane.  A
-        // stripe (32 LR rows) starts on an even row, so no pair straddles two stripes.
-        const int nxa = __shfl_down_sync(0xffffffffu, ((int)kA[0] >> 16) + o, 1);
-        const int nxb = __shfl_down_sync(0xffffffffu, ((int)kB[0] >> 16) + o, 1);
-#pragma unroll
-        for (int r = 0; r < LR; ++r) {
-            const int xa0 = ((int)kA[r] >> 16) + o, xb0 = ((int)kB[r] >> 16) + o;
-            const int xa1 = r + 1 < LR ? ((int)kA[(r + 1) % LR] >> 16) + o : nxa;
-            const int xb1 = r + 1 < LR ? ((int)kB[(r + 1) % LR] >> 16) + o : nxb;
-            const int i = row0 + r;
-            if (i < m) {
-                if ((i & 1) == 0) {
-                    bmA[i >> 1] = (int16_t)max(xa0, xa1);
-                    bmB[i >> 1] = (int16_t)max(xb0, xb1);
+        auto residues = [&](int x) {
+            return (x < io.nA ? (uint32_t)io.tA[x] : (uint32_t)PAD_RES) |
+                   ((x < io.nB ? (uint32_t)io.tB[x] : (uint32_t)PAD_RES) << 16);
+        };
+        uint32_t win = PADS, nxt = residues(lg);
+        int j = -lg;
+        const int steps = n + G - 1;
+        for (int w = 0; w < steps; w += G) {
+            const uint32_t cur = nxt;                       // columns [w, w + G)
+            nxt = residues(w + G + lg);
+            const int we = min(G, steps - w);
+#pragma unroll 1
+            for (int x = 0; x < we; ++x, ++j) {
+                win = lg == x ? cur : win;
+                const uint32_t tt = __shfl_sync(0xffffffffu, win, j, G);
+                uint32_t hu = __shfl_up_sync(0xffffffffu, out_h, 1, G);
+                uint32_t fu = __shfl_up_sync(0xffffffffu, out_f, 1, G);
+                if (lg == 0) { hu = INIT; fu = INIT; }
+                if (take && lg == 0 && j < n) { const uint2 v = in_buf[j]; hu = v.x; fu = v.y; }
+                uint32_t f = fu, hup = hu;
+                const uint32_t cm = column2<LR, PLANE>(pr + (int)(tt & 0xFFFFu) * tl.prow,
+                                                       pr + (int)(tt >> 16) * tl.prow, Ho, E, rm, hd, f, hup, tm, OP, nEP);
+                hd = hu;
+                out_h = hup; out_f = f;
+                if (hand_on && lg == G - 1 && (unsigned)j < (unsigned)n) out_buf[j] = make_uint2(hup, f);
+                const uint32_t over = cm ^ tm;
+                if (__builtin_expect(__any_sync(0xffffffffu, over != 0u), 0)) {
+                    if (__any_sync(0xffffffffu, (over & 0xFFFFu) != 0u)) {
+                        const int t = note_best<G, LR, false>(Ho, (over & 0xFFFFu) != 0u, row0, j, lg, sh16, vA, iA, jA);
+                        tm = (tm & 0xFFFF0000u) | ((uint32_t)t & 0xFFFFu);
+                    }
+                    if (__any_sync(0xffffffffu, (over >> 16) != 0u)) {
+                        const int t = note_best<G, LR, true>(Ho, (over >> 16) != 0u, row0, j, lg, sh16, vB, iB, jB);
+                        tm = (tm & 0xFFFFu) | ((uint32_t)t << 16);
+                    }
                 }
-                if (xa0 > bA) { bA = xa0; iA = i; jA = 65535 - (int)(kA[r] & 0xFFFFu); }
-                if (xb0 > bB) { bB = xb0; iB = i; jB = 65535 - (int)(kB[r] & 0xFFFFu); }
+            }
+        }
+        // the row-pair bounds (LR is even, so no pair of rows straddles two lanes)
+#pragma unroll
+        for (int r = 0; r < LR; r += 2) {
+            const int g = (row0 + r) >> 1;
+            if (row0 + r < m) {
+                const uint32_t h = __vadd2(rm[r >> 1], OP);
+                if (io.bmA) io.bmA[g] = (int16_t)(h & 0xFFFFu);
+                if (io.bmB) io.bmB[g] = (int16_t)(h >> 16);
             }
         }
         __syncwarp();
     }
-    // across the warp: the largest score, then the smallest row (rows are unique per lane)
-    const int SA = __reduce_max_sync(0xffffffffu, bA), SB = __reduce_max_sync(0xffffffffu, bB);
-    const int eiA = (int)__reduce_min_sync(0xffffffffu, bA == SA ? (unsigned)iA : 0xFFFFFFFFu);
-    const int eiB = (int)__reduce_min_sync(0xffffffffu, bB == SB ? (unsigned)iB : 0xFFFFFFFFu);
-    const unsigned wa = __ballot_sync(0xffffffffu, bA == SA && iA == eiA);
-    const unsigned wb = __ballot_sync(0xffffffffu, bB == SB && iB == eiB);
-    ra->h = SA; ra->i = eiA; ra->j = __shfl_sync(0xffffffffu, jA, __ffs(wa) - 1);
-    rb->h = SB; rb->i = eiB; rb->j = __shfl_sync(0xffffffffu, jB, __ffs(wb) - 1);
+    // across the group: the largest score, then the smallest row (rows are unique per lane)
+    auto finish = [&](int v, int i, int j, end_cell *r) {
+        int S = v;
+        for (int d = G >> 1; d > 0; d >>= 1) S = max(S, __shfl_xor_sync(0xffffffffu, S, d));
+        int bi = v == S ? i : 0x7FFFFFFF;
+        for (int d = G >> 1; d > 0; d >>= 1) bi = min(bi, __shfl_xor_sync(0xffffffffu, bi, d));
+        int bj = v == S && i == bi ? j : -1;
+        for (int d = G >> 1; d > 0; d >>= 1) bj = max(bj, __shfl_xor_sync(0xffffffffu, bj, d));
+        r->h = S + o; r->i = bi; r->j = bj;
+    };
+    finish(vA, iA, jA, ra);
+    finish(vB, iB, jB, rb);
+}
+
+template <int G, bool MULTI>
+__device__ __forceinline__ void score_rows(const sw_tile &tl, const uint8_t *prof, const pair_io &io, int m, int o,
+                                           int e, uint32_t one, uint2 *buf, int sstride, end_cell *ea, end_cell *eb) {
+#define PASTIS_SW_CASE(L) \
+    case L: score_group<G, L, MULTI>(prof, tl, io, m, o, e, one, buf, sstride, ea, eb); break;
+    switch (tl.lr) {
+        PASTIS_SW_CASE(2) PASTIS_SW_CASE(4) PASTIS_SW_CASE(6) PASTIS_SW_CASE(8) PASTIS_SW_CASE(10)
+        PASTIS_SW_CASE(12) PASTIS_SW_CASE(14) PASTIS_SW_CASE(16) PASTIS_SW_CASE(18) PASTIS_SW_CASE(20)
+        PASTIS_SW_CASE(22) PASTIS_SW_CASE(24) PASTIS_SW_CASE(26) PASTIS_SW_CASE(28) PASTIS_SW_CASE(30)
+        default: score_group<G, LR_MAX, MULTI>(prof, tl, io, m, o, e, one, buf, sstride, ea, eb); break;
+    }
+#undef PASTIS_SW_CASE
 }
 
 // ---------------------------------------------------------------------------------
@@ -585,7 +698,8 @@ __global__ void k_bm_count(const pastis_cand *pairs, int64_t n, const int64_t *q
 __global__ void __launch_bounds__(SW_THREADS, 2) k_sw_score(const uint8_t *qcodes, const int64_t *qoffsets,
                                                          const uint8_t *tcodes, const int64_t *toffsets,
                                                          const pastis_cand *pairs, const int64_t *seg_start,
-                                                         int64_t n_seg, const int8_t *gmat, int o, int e,
+                                                         const uint32_t *seg_order, int64_t n_seg,
+                                                         const int8_t *gmat, int o, int e,
                                                          int max_s, int prow_cap, uint32_t one, char *scratch,
                                                          size_t warp_bytes, int sstride, int *next_seg,
                                                          int16_t *bm_all, const int64_t *bm_off, sw_score_out *out,
@@ -595,10 +709,12 @@ __global__ void __launch_bounds__(SW_THREADS, 2) k_sw_score(const uint8_t *qcode
     // captured launches: the segment count from device memory, nothing on bad input
     if (d_nseg) n_seg = *d_nseg;
     if (chk && (chk[0] | chk[1])) return;
-    // dynamic shared memory: the profile [NRES][prow_cap] bytes (prow_cap a whole number of stripes)
+    // dynamic shared memory: the profile [NRES][prow_cap] bytes (prow_cap a whole number of
+    // 512-row stripes); before it is built, the segment's sort keys
     extern __shared__ __align__(16) uint8_t s_prof[];
     __shared__ int s_seg, s_next;
-    __shared__ uint32_t s_key[SEG_MAX];
+    __shared__ uint16_t s_ord[SEG_MAX];
+    uint32_t *s_key = reinterpret_cast<uint32_t *>(s_prof);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gw = blockIdx.x * SW_WARPS + warp;
     uint2 *my = reinterpret_cast<uint2 *>(scratch + (size_t)gw * warp_bytes);
@@ -607,8 +723,8 @@ __global__ void __launch_bounds__(SW_THREADS, 2) k_sw_score(const uint8_t *qcode
     for (;;) {
         if (threadIdx.x == 0) { s_seg = atomicAdd(next_seg, 1); s_next = 0; }
         __syncthreads();
-        const int64_t sg = s_seg;
-        if (sg >= n_seg) break;
+        if (s_seg >= n_seg) break;
+        const int64_t sg = seg_order[s_seg];
         const long long t_seg = tune ? clock64() : 0;
         const int64_t p0 = seg_start[sg], p1 = seg_start[sg + 1];
         const int cnt = (int)(p1 - p0);
@@ -617,56 +733,62 @@ __global__ void __launch_bounds__(SW_THREADS, 2) k_sw_score(const uint8_t *qcode
         const int m = (int)(qoffsets[qi + 1] - qo);
         const int bin = sw_bin(m);
         const bool int32_bin = extra[bin] == PASTIS_SW_INT32;    // the bin's pairs in 32-bit lanes
-        const int ex = int32_bin ? 0 : extra[bin];
-        int lr = rows_per_lane(m, ex);
-        int prow8 = ((m + 32 * lr - 1) / (32 * lr)) * STRIPE_BYTES;     // profile bytes per residue
-        if (prow8 > prow_cap && ex) {                                  // the extra stripes do not fit
-            lr = rows_per_lane(m, 0);
-            prow8 = ((m + 32 * lr - 1) / (32 * lr)) * STRIPE_BYTES;
-        }
-        // query profile: byte (st * 512 + l * 16 + r) of residue c = M[q_i][c] + o for row
-        // i = st * 32 * lr + l * lr + r of the query; o - 64 for the pad residue, unused
-        // slots and rows past the query
-        if (prow8 <= prow_cap) {
-            for (int x = threadIdx.x; x < NRES * prow8; x += blockDim.x) {
-                const int c = x / prow8, rest = x - c * prow8;
-                const int st = rest / STRIPE_BYTES, l = (rest % STRIPE_BYTES) / SLOT, r = rest % SLOT;
-                const int i = st * 32 * lr + l * lr + r;
-                s_prof[x] = (uint8_t)(int8_t)((r < lr && i < m && c < PASTIS_NSYM)
-                                                  ? (int)gmat[qcodes[qo + i] * PASTIS_NSYM + c] + o : o - 64);
-            }
-        }
-        // the segment's pairs by target length, longest first, so that the two pairs of
-        // a warp match and the last pairs taken are the shortest
-        if (threadIdx.x < SEG_MAX) {
+        // the segment's pairs by target length, longest first, so that the pairs of a warp
+        // match and the last pairs taken are the shortest
+        int np2 = 2;
+        while (np2 < cnt) np2 <<= 1;
+        for (int x = threadIdx.x; x < np2; x += SW_THREADS) {
             uint32_t key = 0xFFFFFFFFu;
-            if ((int)threadIdx.x < cnt) {
-                const int j = pairs[p0 + threadIdx.x].j;
-                key = ((uint32_t)(65535 - (toffsets[j + 1] - toffsets[j])) << 7) | threadIdx.x;
+            if (x < cnt) {
+                const int j = pairs[p0 + x].j;
+                key = ((uint32_t)(65535 - (toffsets[j + 1] - toffsets[j])) << 9) | (uint32_t)x;
             }
-            s_key[threadIdx.x] = key;
+            s_key[x] = key;
         }
         __syncthreads();
-        for (int k = 2; k <= SEG_MAX; k <<= 1) {
+        for (int k = 2; k <= np2; k <<= 1) {
             for (int jj = k >> 1; jj > 0; jj >>= 1) {
-                const int x = threadIdx.x, y = x ^ jj;
-                if (x < SEG_MAX && y > x) {
+                for (int t = threadIdx.x; t < np2 / 2; t += SW_THREADS) {
+                    const int x = 2 * t - (t & (jj - 1)), y = x + jj;
                     const uint32_t u = s_key[x], v = s_key[y];
                     if ((u > v) == ((x & k) == 0)) { s_key[x] = v; s_key[y] = u; }
                 }
                 __syncthreads();
             }
         }
+        const int nt = 65535 - (int)(s_key[0] >> 9);
+        for (int x = threadIdx.x; x < cnt; x += SW_THREADS) s_ord[x] = (uint16_t)(s_key[x] & (SEG_MAX - 1));
+        const sw_tile tl = pick_tile(m, int32_bin ? 0 : extra[bin], cnt, nt, prow_cap);
+        __syncthreads();
+        // query profile: row i = (st * G + l) * lr + r of the query at byte
+        // st * sbytes + (r / 16) * 16 G + 16 l + r % 16 of residue c = M[q_i][c] + o; o - 64
+        // for the pad residue, unused slots and rows past the query
+        if (tl.prow <= prow_cap) {
+            const int gl = __ffs(tl.G) - 1, planes = tl.lr > SLOT ? 2 : 1;
+            for (int x = threadIdx.x; x < tl.prow; x += SW_THREADS) {
+                const int lq = (x >> 4) & (tl.G - 1), pl = x >> (4 + gl);
+                const int st = planes == 2 ? pl >> 1 : pl, r = (planes == 2 ? (pl & 1) * SLOT : 0) + (x & 15);
+                const int i = (st * tl.G + lq) * tl.lr + r;
+                const bool in = r < tl.lr && i < m;
+                const int8_t *row = gmat + (in ? (int)qcodes[qo + i] * PASTIS_NSYM : 0);
+#pragma unroll
+                for (int c = 0; c < NRES; ++c)
+                    s_prof[c * tl.prow + x] = (uint8_t)(int8_t)(in && c < PASTIS_NSYM ? (int)row[c < PASTIS_NSYM ? c : 0] + o : o - 64);
+            }
+        }
+        __syncthreads();
+        const int grp = lane / tl.G, lg = lane & (tl.G - 1);
         for (;;) {
             int pk = 0;
-            if (lane == 0) pk = atomicAdd(&s_next, 2);
+            if (lane == 0) pk = atomicAdd(&s_next, 64 / tl.G);
             pk = __shfl_sync(0xffffffffu, pk, 0);
             if (pk >= cnt) break;
+            pk += 2 * grp;
             int64_t pp[2];
             int nn[2], st[2];                                     // st: 0 zero, 1 big, 2 run
             const uint8_t *tp[2];
             for (int u = 0; u < 2; ++u) {
-                pp[u] = pk + u < cnt ? p0 + (int64_t)(s_key[pk + u] & (SEG_MAX - 1)) : -1;
+                pp[u] = pk + u < cnt ? p0 + (int64_t)s_ord[pk + u] : -1;
                 nn[u] = 0; st[u] = 0; tp[u] = tcodes;
                 if (pp[u] < 0) continue;
                 const pastis_cand c = pairs[pp[u]];
@@ -674,51 +796,46 @@ __global__ void __launch_bounds__(SW_THREADS, 2) k_sw_score(const uint8_t *qcode
                 nn[u] = (int)(toffsets[c.j + 1] - to);
                 tp[u] = tcodes + to;
                 if (m == 0 || nn[u] == 0) st[u] = 0;
-                else if (int32_bin || !packable || prow8 > prow_cap ||
+                else if (int32_bin || !packable || tl.prow > prow_cap ||
                          (int64_t)max_s * (int64_t)min(m, nn[u]) >= SCORE_MAX) st[u] = 1;
                 else st[u] = 2;
             }
-            end_cell res[2];
-            res[0].h = res[1].h = 0;
-            if (st[0] == 2 || st[1] == 2) {
-                // both halves busy; a lone pair fills both
-                const int ua = st[0] == 2 ? 0 : 1, ub = st[1] == 2 ? 1 : 0;
-                int16_t *bma = bm_all + bm_off[pp[ua]], *bmb = bm_all + bm_off[pp[ub]];
-                end_cell ea, eb;
-#define PASTIS_SW_CASE(L)                                                                                       \
-    case L:                                                                                                     \
-        score_pair<L>(s_prof, prow8, tp[ua], nn[ua], tp[ub], nn[ub], m, o, e, one, my, sstride, bma, bmb, &ea, &eb); \
-        break;
-                switch (lr) {
-                    PASTIS_SW_CASE(2) PASTIS_SW_CASE(3) PASTIS_SW_CASE(4) PASTIS_SW_CASE(5)
-                    PASTIS_SW_CASE(6) PASTIS_SW_CASE(7) PASTIS_SW_CASE(8) PASTIS_SW_CASE(9)
-                    PASTIS_SW_CASE(10) PASTIS_SW_CASE(11) PASTIS_SW_CASE(12) PASTIS_SW_CASE(13)
-                    PASTIS_SW_CASE(14) PASTIS_SW_CASE(15)
-                    default:
-                        score_pair<16>(s_prof, prow8, tp[ua], nn[ua], tp[ub], nn[ub], m, o, e, one, my, sstride, bma,
-                                       bmb, &ea, &eb);
-                        break;
-                }
-#undef PASTIS_SW_CASE
+            end_cell ea, eb;
+            ea.h = eb.h = 0;
+            ea.i = ea.j = eb.i = eb.j = 0;
+            if (__any_sync(0xffffffffu, st[0] == 2 || st[1] == 2)) {
+                pair_io io;
+                io.tA = tp[0]; io.tB = tp[1];
+                io.nA = st[0] == 2 ? nn[0] : 0;                   // a half without a pair runs on pad columns
+                io.nB = st[1] == 2 ? nn[1] : 0;
+                io.bmA = st[0] == 2 ? bm_all + bm_off[pp[0]] : nullptr;
+                io.bmB = st[1] == 2 ? bm_all + bm_off[pp[1]] : nullptr;
+                // one loop body per lane count and rows per lane, and for several stripes: with
+                // the lane count and the hand-on as run-time values pass 1 took 6% longer
+                if (tl.ns > 1) score_rows<32, true>(tl, s_prof, io, m, o, e, one, my, sstride, &ea, &eb);
+                else if (tl.G == 32) score_rows<32, false>(tl, s_prof, io, m, o, e, one, my, sstride, &ea, &eb);
+                else if (tl.G == 16) score_rows<16, false>(tl, s_prof, io, m, o, e, one, my, sstride, &ea, &eb);
+                else score_rows<8, false>(tl, s_prof, io, m, o, e, one, my, sstride, &ea, &eb);
                 __syncwarp();
-                if (st[ua] == 2) res[ua] = ea;
-                if (st[ub] == 2 && ub != ua) res[ub] = eb;
             }
-            for (int u = 0; u < 2; ++u) {
-                if (pp[u] < 0) continue;
-                sw_score_out r;
-                r.score = 0; r.end_i = 0; r.end_j = 0; r.rect_i = 0; r.rect_j = 0; r.big = st[u] == 1;
-                if (st[u] == 2) {
-                    if (res[u].h > 0) { r.score = res[u].h; r.end_i = res[u].i; r.end_j = res[u].j; }
-                    my_cells += (unsigned long long)m * (unsigned long long)nn[u];
+            if (lg == 0) {
+                for (int u = 0; u < 2; ++u) {
+                    if (pp[u] < 0) continue;
+                    const end_cell &en = u ? eb : ea;
+                    sw_score_out r;
+                    r.score = 0; r.end_i = 0; r.end_j = 0; r.rect_i = 0; r.rect_j = 0; r.big = st[u] == 1;
+                    if (st[u] == 2) {
+                        if (en.h > 0) { r.score = en.h; r.end_i = en.i; r.end_j = en.j; }
+                        my_cells += (unsigned long long)m * (unsigned long long)nn[u];
+                    }
+                    out[pp[u]] = r;
                 }
-                if (lane == 0) out[pp[u]] = r;
             }
         }
         __syncthreads();
         if (tune && threadIdx.x == 0) atomicAdd(&tune[bin], (unsigned long long)(clock64() - t_seg));
     }
-    if (lane == 0 && cells && my_cells) atomicAdd(cells, my_cells);
+    if (cells && my_cells) atomicAdd(cells, my_cells);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1083,20 +1200,30 @@ pastis_status sw_align(pastis_ctx *ctx, const uint8_t *d_qcodes, const int64_t *
     for (int x = 0; x < PASTIS_NSYM * PASTIS_NSYM; ++x) max_s = std::max(max_s, (int)p->matrix[x]);
     // segments of pairs sharing a query
     uint32_t *sflags;
-    PASTIS_WS(sflags, ctx, WS_ALN_ORDER, sizeof(uint32_t) * (2 * (size_t)n_pairs + 2) + sizeof(int64_t) * (n_pairs + 2) + 16);
-    uint32_t *soff = sflags + n_pairs + 1;
-    int64_t *seg_start = (int64_t *)(((uintptr_t)(soff + n_pairs + 1) + 7) & ~(uintptr_t)7);
+    PASTIS_WS(sflags, ctx, WS_ALN_ORDER, sizeof(uint32_t) * (2 * (size_t)n_pairs + 2 + 2 * SEG_BINS) +
+                                             sizeof(int64_t) * (n_pairs + 2) + 16);
+    uint32_t *soff = sflags + n_pairs + 1, *hist = soff + n_pairs + 1;
+    int64_t *seg_start = (int64_t *)(((uintptr_t)(hist + 2 * SEG_BINS) + 7) & ~(uintptr_t)7);
+    PASTIS_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * 2 * SEG_BINS, st));
     k_seg_flags<<<(unsigned)ceil_div64(n_pairs, 256), 256, 0, st>>>(d_pairs, n_pairs, sflags, dn);
     PASTIS_LAUNCHED(ctx);
     pastis_status s = exclusive_scan_u32(ctx, sflags, soff, n_pairs);
     if (s != PASTIS_OK) return s;
-    k_seg_starts<<<(unsigned)ceil_div64(n_pairs, 256), 256, 0, st>>>(sflags, soff, n_pairs, seg_start, dn);
+    k_seg_starts<<<(unsigned)ceil_div64(n_pairs, 256), 256, 0, st>>>(d_pairs, d_qoffsets, sflags, soff, n_pairs,
+                                                                     seg_start, hist, dn, chk);
     PASTIS_LAUNCHED(ctx);
     uint32_t h_nseg = 0;
     if (!dn) {
         PASTIS_CUDA_TRY(cudaMemcpyAsync(&h_nseg, soff + n_pairs, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
         PASTIS_CUDA_TRY(cudaStreamSynchronize(st));
     }
+
+    // the flags have served: the segments' order takes their place
+    const int64_t seg_cap = dn ? n_pairs : (int64_t)h_nseg;
+    k_seg_order<<<(unsigned)ceil_div64(seg_cap, 256), 256, 0, st>>>(d_pairs, d_qoffsets, seg_start, seg_cap,
+                                                                    dn ? soff + n_pairs : nullptr, hist,
+                                                                    hist + SEG_BINS, sflags, chk);
+    PASTIS_LAUNCHED(ctx);
 
     // row-pair bounds of pass 1 for pass 2: (query length + 1) / 2 int16 per pair
     int64_t *bm_cnt;
@@ -1119,10 +1246,11 @@ pastis_status sw_align(pastis_ctx *ctx, const uint8_t *d_qcodes, const int64_t *
     // pass 1+2: profile rows up to the longest query (in whole stripes), within shared memory
     int max_extra = 0;
     for (int b = 0; b < PASTIS_SW_BINS; ++b) max_extra = std::max(max_extra, (int)ctx->sw_lay.extra[b]);
-    int prow_cap = ((lmax + STRIPE1 - 1) / STRIPE1 + max_extra) * STRIPE1;
-    if (prow_cap < STRIPE1) prow_cap = STRIPE1;
+    // profile bytes per residue: 512 up to 512 query rows, else 1,024 per 1,024 rows
+    int prow_cap = lmax <= STRIPE1 && max_extra == 0 ? STRIPE1
+                                                     : ((lmax + 2 * STRIPE1 - 1) / (2 * STRIPE1) + max_extra) * 2 * STRIPE1;
     auto shm_for = [](int pc) { return (size_t)NRES * pc; };
-    while (prow_cap > STRIPE1 && shm_for(prow_cap) + 1024 > ctx->smem_optin) prow_cap -= STRIPE1;
+    while (prow_cap > STRIPE1 && shm_for(prow_cap) + 1088 > ctx->smem_optin) prow_cap -= STRIPE1;
     const size_t shm1 = shm_for(prow_cap);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sw_score, SW_THREADS, shm1);
@@ -1137,7 +1265,7 @@ pastis_status sw_align(pastis_ctx *ctx, const uint8_t *d_qcodes, const int64_t *
     PASTIS_WS(scratch, ctx, WS_ALN_SCRATCH, std::max(scr1, scr3));
     prof_begin(ctx, "sw_pass1");
     k_sw_score<<<blocks1, SW_THREADS, shm1, st>>>(d_qcodes, d_qoffsets, d_tcodes, d_toffsets, d_pairs, seg_start,
-                                                  (int64_t)h_nseg, dmat,
+                                                  sflags, (int64_t)h_nseg, dmat,
                                                   p->gap_open, p->gap_extend, max_s, prow_cap, 1u, (char *)scratch,
                                                   warp_bytes, sstride, flags + 1, bm_all, bm_off, res,
                                                   (unsigned long long *)d_cells, (const uint8_t *)dmat + 640,

@@ -46,7 +46,7 @@ extern "C" pastis_status pastis_ctx_create(pastis_ctx **ctx, int device, void *s
     // Kernels with a per-call dynamic shared-memory size get the device's limit once
     // here; a per-call setting could lower it under a launch of another thread.
     if (sw_set_smem_limit(c->smem_optin) != cudaSuccess || spgemm_set_smem_limit(c->smem_optin) != cudaSuccess ||
-        radix_set_smem_limit() != cudaSuccess) {
+        radix_set_smem_limit() != cudaSuccess || mlp_set_smem_limit() != cudaSuccess) {
         cudaGetLastError();
         free(c);
         return PASTIS_ERR_CUDA;

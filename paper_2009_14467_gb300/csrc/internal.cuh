@@ -144,6 +144,7 @@ pastis_status exclusive_scan_i64(pastis_ctx *c, const int64_t *in, int64_t *out,
 cudaError_t sw_set_smem_limit(size_t bytes);
 cudaError_t spgemm_set_smem_limit(size_t bytes);
 cudaError_t radix_set_smem_limit();
+cudaError_t mlp_set_smem_limit();
 
 // Validates the parameters shared by the calls; returns PASTIS_OK or INVALID_ARG.
 pastis_status check_params(const pastis_params *p);

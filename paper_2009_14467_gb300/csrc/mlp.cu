@@ -12,10 +12,12 @@
 //
 // Arithmetic: bf16 weights and activations, float32 accumulation on the tensor cores
 // (mma.sync m16n8k16, bf16 inputs, f32 accumulators), float32 master weights and Adam
-// moments.  Every product of forward and backward goes through one tiled GEMM kernel;
-// bias, ReLU, loss and optimizer steps are small elementwise kernels.
+// moments.  One kernel runs the network forward (in training also back to layer 1), one
+// forms the gradients of W1 and W2, one sums the others and takes the Adam step.
 #include <cuda_bf16.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "internal.cuh"
 
@@ -67,170 +69,469 @@ __global__ void k_pair_features(const uint8_t *qcodes, const int64_t *qoffsets, 
 }
 
 // ---------------------------------------------------------------------------------
-// GEMM: C[M x N] = op(A)[M x K] * op(B)[K x N] (+ epilogue), bf16 in, f32 accumulate.
-// A is row-major M x K (TA = false) or K x M (TA = true); B is row-major K x N (TB =
-// false) or N x K (TB = true).  Block tile 64 x 64, 4 warps, each warp 16 rows x 64
-// columns = 8 mma tiles of 16 x 8, K in steps of 16 staged through shared memory.
-// Epilogue: EP_F32 stores f32 (optionally accumulating), EP_BIAS_RELU stores
-// bf16(relu(acc + bias[n])), EP_BIAS stores f32 acc + bias[n].
+// The network: one persistent kernel takes 64 rows at a time through all three layers
+// (and, in training, back to the gradient at layer 1), with the activations in shared
+// memory.  A CTA's two groups of eight warps each work on a tile of their own, so one's
+// epilogues run under the other's products.  W2 stays there for the kernel's life, in rows of 256 + 8 values so that the
+// eight rows of an ldmatrix lie in different banks.  A warp owns 32 rows x 64 columns of
+// every product; the k steps of 16 run in order from a zero accumulator, so a logit does
+// not depend on the batch it is computed in.
+// What bounds it is the rate of mma.sync with every operand fragment read from shared
+// memory.  mma.sync, not tcgen05: its sums are the ones the selection thresholds in use
+// were calibrated on, and a step of the path spends about 1% here.
 // ---------------------------------------------------------------------------------
-enum { EP_F32 = 0, EP_F32_ACC = 1, EP_BIAS_RELU = 2, EP_BIAS = 3 };
+constexpr int TM = 64;                               // rows of a tile
+constexpr int MLP_GROUPS = 2;                        // groups of eight warps, a tile each
+constexpr int LDH = HID + 8, LDX = FEAT + 8;         // row pitches in shared memory
+constexpr int GROUP = 256, MLP_THREADS = MLP_GROUPS * GROUP;
+constexpr int PART = 3 * HID + 2;                    // a CTA's partial sums: g_b1, g_b2, g_w3, g_b3, loss
+constexpr size_t MLP_SMEM = sizeof(__nv_bfloat16) * ((size_t)HID * LDH + FEAT * LDH + MLP_GROUPS * (TM * LDH + TM * LDX)) +
+                            sizeof(float) * 3 * HID;
 
-template <bool TA, bool TB, int EP>
-__global__ void __launch_bounds__(128) k_gemm_bf16(const __nv_bfloat16 *__restrict__ A, const __nv_bfloat16 *__restrict__ B,
-                                                   int M, int N, int K, const float *__restrict__ bias, float *Cf,
-                                                   __nv_bfloat16 *Cb) {
-    __shared__ __nv_bfloat16 sA[64][16 + 8];      // [m][k], padded
-    __shared__ __nv_bfloat16 sB[64][16 + 8];      // [n][k], padded (B stored transposed)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gid = lane >> 2, tig = lane & 3;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    float acc[8][4];
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Two columns of a fragment as they are stored: relu(acc + bias) in bf16.
+__device__ __forceinline__ uint32_t bias_relu2(float v0, float v1, const float *bias) {
+    __nv_bfloat162 h;
+    h.x = __float2bfloat16(fmaxf(v0 + bias[0], 0.f));
+    h.y = __float2bfloat16(fmaxf(v1 + bias[1], 0.f));
+    return *reinterpret_cast<uint32_t *>(&h);
+}
+// Eight bf16 from memory that may not be 16-byte aligned (the caller's buffers).
+__device__ __forceinline__ uint4 load8(const __nv_bfloat16 *p, bool aligned) {
+    if (aligned) return *reinterpret_cast<const uint4 *>(p);
+    const uint16_t *q = reinterpret_cast<const uint16_t *>(p);
+    uint32_t w[4];
 #pragma unroll
-    for (int t = 0; t < 8; ++t)
+    for (int i = 0; i < 4; ++i) w[i] = (uint32_t)q[2 * i] | ((uint32_t)q[2 * i + 1] << 16);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// acc[2][8][4] = the warp's 32 rows (mw) x 64 columns (nw) of s_h (bf16, 64 x 256) times
+// W2 (TW: its transpose).
+template <bool TW>
+__device__ __forceinline__ void tile_product(float (&acc)[2][8][4], uint32_t h, uint32_t w2, int mw, int nw, int lane) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[t][q] = 0.f;
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int x = threadIdx.x; x < 64 * 16; x += 128) {
-            const int r = x / 16, kk = x % 16;
-            const int m = m0 + r, kg = k0 + kk;
-            __nv_bfloat16 va = __float2bfloat16(0.f);
-            if (m < M && kg < K) va = TA ? A[(int64_t)kg * M + m] : A[(int64_t)m * K + kg];
-            sA[r][kk] = va;
-            const int nn = n0 + r;
-            __nv_bfloat16 vb = __float2bfloat16(0.f);
-            if (nn < N && kg < K) vb = TB ? B[(int64_t)nn * K + kg] : B[(int64_t)kg * N + nn];
-            sB[r][kk] = vb;
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[i][t][q] = 0.f;
+    const uint32_t ha = h + (uint32_t)(((mw * 32 + (lane & 15)) * LDH + (lane >> 4) * 8) * 2);
+    const uint32_t wb = TW ? w2 + (uint32_t)(((nw * 64 + (lane & 7) + ((lane >> 4) << 3)) * LDH + ((lane >> 3) & 1) * 8) * 2)
+                           : w2 + (uint32_t)(((lane & 15) * LDH + nw * 64 + (lane >> 4) * 8) * 2);
+#pragma unroll 2
+    for (int k = 0; k < HID; k += 16) {
+        uint32_t a[2][4];
+        ldsm4(a[0], ha + k * 2);
+        ldsm4(a[1], ha + (16 * LDH + k) * 2);
+#pragma unroll
+        for (int t = 0; t < 8; t += 2) {
+            uint32_t b[4];
+            if (TW) ldsm4(b, wb + (t * 8 * LDH + k) * 2);
+            else ldsm4t(b, wb + (k * LDH + t * 8) * 2);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                mma16816(acc[i][t], a[i], b[0], b[1]);
+                mma16816(acc[i][t + 1], a[i], b[2], b[3]);
+            }
         }
+    }
+}
+
+struct mlp_w {
+    const __nv_bfloat16 *w1, *w2, *w3;
+    const float *b1, *b2, *b3;
+};
+struct mlp_train_io {           // training only
+    const float *y;
+    float pos_weight;
+    __nv_bfloat16 *h1, *dh1, *dh2;   // n x 256 each, for the gradients of W1 and W2
+    float *part;                // PART floats per CTA
+};
+
+// z[r] = the logit of row r.  TRAIN: also the weighted logistic loss, dz = w * (sigmoid(z)
+// - y) / n, the gradients dh2 = dz * w3 where layer 2 is active and dh1 = dh2 W2^T where
+// layer 1 is, and the gradients of the biases and W3 as partial sums per CTA (fixed order,
+// so a training step is deterministic).  Measured on 10^6 rows: 3.99 ms with
+// one 64 x 64 tile and 2-byte loads a CTA and h1, h2 through memory, 0.355 ms so (137 GF:
+// 0.6 of the rate mma.sync reaches alone); a training step of 65,536 rows 28.1 ms with the
+// column sums in one CTA each, 0.39 ms so.
+template <bool TRAIN>
+__global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bfloat16 *__restrict__ x, int64_t n,
+                                                        float *__restrict__ z, mlp_train_io tr) {
+    const int lane = threadIdx.x & 31, group = threadIdx.x / GROUP;
+    const int tid = threadIdx.x % GROUP, warp = tid >> 5;                // within the group
+    const int gid = lane >> 2, tig = lane & 3;
+    const int mw = warp >> 2, nw = warp & 3;             // the warp's 32 rows x 64 columns
+    auto sync = [group]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(GROUP) : "memory"); };
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    __nv_bfloat16 *s_w2 = reinterpret_cast<__nv_bfloat16 *>(mlp_smem);   // [256][LDH], input-major
+    __nv_bfloat16 *s_w1 = s_w2 + HID * LDH;                              // [16][LDH]
+    __nv_bfloat16 *s_h = s_w1 + FEAT * LDH + group * TM * LDH;           // [64][LDH]: h1, then h2, dh2, dh1
+    __nv_bfloat16 *s_x = s_w1 + FEAT * LDH + MLP_GROUPS * TM * LDH + group * TM * LDX;   // [64][LDX]
+    float *s_b1 = reinterpret_cast<float *>(s_w1 + FEAT * LDH + MLP_GROUPS * TM * (LDH + LDX));
+    float *s_b2 = s_b1 + HID, *s_w3 = s_b2 + HID;
+    const bool wal = ((((uintptr_t)net.w1) | ((uintptr_t)net.w2)) & 15) == 0, xal = (((uintptr_t)x) & 15) == 0;
+    for (int i = threadIdx.x; i < (HID + FEAT) * HID / 8; i += MLP_THREADS) {
+        const int r = i >> 5, c = (i & 31) * 8;
+        const uint4 v = r < HID ? load8(net.w2 + r * HID + c, wal) : load8(net.w1 + (r - HID) * HID + c, wal);
+        *reinterpret_cast<uint4 *>(s_w2 + r * LDH + c) = v;              // W1's rows follow W2's
+    }
+    if (group == 0) {
+        s_b1[tid] = net.b1[tid];
+        s_b2[tid] = net.b2[tid];
+        s_w3[tid] = bf(net.w3[tid]);
+    }
+    __syncthreads();
+    const float b3 = net.b3[0];
+    const uint32_t u_h = smem_u32(s_h), u_w1 = smem_u32(s_w1), u_w2 = smem_u32(s_w2), u_x = smem_u32(s_x);
+    // TRAIN: sums kept over the CTA's tiles
+    float gw3[8], gb2[8], gb1[16], gb3 = 0.f, loss = 0.f;
+    if constexpr (TRAIN) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) { gw3[t] = 0.f; gb2[t] = 0.f; }
+#pragma unroll
+        for (int t = 0; t < 16; ++t) gb1[t] = 0.f;
+    }
+    const int64_t tiles = (n + TM - 1) / TM;
+    const int xr = tid >> 1, xc = (tid & 1) * 8;         // 128 threads load 8 features of a tile each
+    auto load_x = [&](int64_t tile) {
+        const int64_t r = tile * TM + xr;
+        return xr < TM && tile < tiles && r < n ? load8(x + r * FEAT + xc, xal) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    const int64_t step = (int64_t)gridDim.x * MLP_GROUPS, tile0 = (int64_t)group * gridDim.x + blockIdx.x;
+    uint4 xv = load_x(tile0);
+    for (int64_t tile = tile0; tile < tiles; tile += step) {
+        const int64_t r0 = tile * TM;
+        if (xr < TM) *reinterpret_cast<uint4 *>(s_x + xr * LDX + xc) = xv;
+        sync();                                          // x here; the group is done with its last tile
+        xv = load_x(tile + step);
+        // layer 1: one k step
+        uint32_t act[2] = {0u, 0u};                      // TRAIN: which of the warp's fragment values are active
+        {
+            uint32_t a[2][4];
+            ldsm4(a[0], u_x + (uint32_t)(((mw * 32 + (lane & 15)) * LDX + (lane >> 4) * 8) * 2));
+            ldsm4(a[1], u_x + (uint32_t)(((mw * 32 + 16 + (lane & 15)) * LDX + (lane >> 4) * 8) * 2));
+#pragma unroll
+            for (int t = 0; t < 8; t += 2) {
+                uint32_t b[4];
+                ldsm4t(b, u_w1 + (uint32_t)(((lane & 15) * LDH + nw * 64 + t * 8 + (lane >> 4) * 8) * 2));
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        float c[4] = {0.f, 0.f, 0.f, 0.f};
+                        mma16816(c, a[i], b[2 * u], b[2 * u + 1]);
+                        const int col = nw * 64 + (t + u) * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
+                        const uint32_t lo = bias_relu2(c[0], c[1], s_b1 + col), hi = bias_relu2(c[2], c[3], s_b1 + col);
+                        *reinterpret_cast<uint32_t *>(s_h + row * LDH + col) = lo;
+                        *reinterpret_cast<uint32_t *>(s_h + (row + 8) * LDH + col) = hi;
+                        if constexpr (TRAIN) {           // stored halves are never negative: non-zero is active
+                            const uint32_t m = ((lo & 0x7FFFu) ? 1u : 0u) | ((lo & 0x7FFF0000u) ? 2u : 0u) |
+                                               ((hi & 0x7FFFu) ? 4u : 0u) | ((hi & 0x7FFF0000u) ? 8u : 0u);
+                            act[i] |= m << (4 * (t + u));
+                        }
+                    }
+            }
+        }
+        sync();
+        if constexpr (TRAIN)
+            for (int i = tid; i < TM * (HID / 8); i += GROUP) {
+                const int64_t r = r0 + (i >> 5);
+                if (r < n)
+                    *reinterpret_cast<uint4 *>(tr.h1 + r * HID + (i & 31) * 8) =
+                        *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
+            }
+        float acc[2][8][4];
+        tile_product<false>(acc, u_h, u_w2, mw, nw, lane);
+        sync();                                 // h1 is read: h2 takes its place
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const int col = nw * 64 + t * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
+                *reinterpret_cast<uint32_t *>(s_h + row * LDH + col) = bias_relu2(acc[i][t][0], acc[i][t][1], s_b2 + col);
+                *reinterpret_cast<uint32_t *>(s_h + (row + 8) * LDH + col) =
+                    bias_relu2(acc[i][t][2], acc[i][t][3], s_b2 + col);
+            }
+        sync();
+        // the head: a warp takes 16 rows, a lane every 32nd column
+#pragma unroll 2
+        for (int q = 0; q < TM / 8; ++q) {
+            const int row = warp * (TM / 8) + q;
+            float h[8], s = 0.f;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                h[t] = bf(s_h[row * LDH + lane + 32 * t]);
+                s += h[t] * s_w3[lane + 32 * t];
+            }
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+            const float zz = s + b3;
+            if (r0 + row < n && lane == 0) z[r0 + row] = zz;
+            if constexpr (TRAIN) {
+                float d = 0.f;
+                if (r0 + row < n) {
+                    const float yy = tr.y[r0 + row];
+                    const float w = yy > 0.5f ? tr.pos_weight : 1.f;
+                    const float sg = 1.f / (1.f + __expf(-zz));
+                    d = w * (sg - yy) / (float)n;
+                    const float sp = zz > 0.f ? zz + log1pf(__expf(-zz)) : log1pf(__expf(zz));
+                    gb3 += d;
+                    loss += w * (sp - yy * zz) / (float)n;
+                }
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    const bool on = r0 + row < n && h[t] > 0.f;
+                    const __nv_bfloat16 dv = __float2bfloat16(on ? d * s_w3[lane + 32 * t] : 0.f);
+                    s_h[row * LDH + lane + 32 * t] = dv;
+                    gw3[t] += h[t] * d;              // d = 0 past the batch
+                    gb2[t] += bf(dv);
+                }
+            }
+        }
+        if constexpr (TRAIN) {
+            sync();
+            for (int i = tid; i < TM * (HID / 8); i += GROUP) {
+                const int64_t r = r0 + (i >> 5);
+                if (r < n)
+                    *reinterpret_cast<uint4 *>(tr.dh2 + r * HID + (i & 31) * 8) =
+                        *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
+            }
+            tile_product<true>(acc, u_h, u_w2, mw, nw, lane);
+            sync();                             // dh2 is read: dh1 takes its place
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int col = nw * 64 + t * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
+                    const uint32_t m = act[i] >> (4 * t);
+                    float v[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[q] = (m >> q) & 1u ? acc[i][t][q] : 0.f;
+                    gb1[2 * t] += v[0] + v[2];
+                    gb1[2 * t + 1] += v[1] + v[3];
+                    __nv_bfloat162 p0, p1;
+                    p0.x = __float2bfloat16(v[0]); p0.y = __float2bfloat16(v[1]);
+                    p1.x = __float2bfloat16(v[2]); p1.y = __float2bfloat16(v[3]);
+                    *reinterpret_cast<__nv_bfloat162 *>(s_h + row * LDH + col) = p0;
+                    *reinterpret_cast<__nv_bfloat162 *>(s_h + (row + 8) * LDH + col) = p1;
+                }
+            }
+            sync();
+            for (int i = tid; i < TM * (HID / 8); i += GROUP) {
+                const int64_t r = r0 + (i >> 5);
+                if (r < n)
+                    *reinterpret_cast<uint4 *>(tr.dh1 + r * HID + (i & 31) * 8) =
+                        *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
+            }
+        }
+        sync();                                 // s_x and s_h are free
+    }
+    if constexpr (TRAIN) {
+        // the CTA's partial sums, through shared memory: [16 warps][256] g_b2, the same g_w3,
+        // [2 groups x 2][256] g_b1
         __syncthreads();
-        // A fragment: rows warp*16 + gid (+8), cols tig*2 (+1) and +8
-        const int ar = warp * 16 + gid;
-        uint32_t a0 = *reinterpret_cast<const uint32_t *>(&sA[ar][tig * 2]);
-        uint32_t a1 = *reinterpret_cast<const uint32_t *>(&sA[ar + 8][tig * 2]);
-        uint32_t a2 = *reinterpret_cast<const uint32_t *>(&sA[ar][tig * 2 + 8]);
-        uint32_t a3 = *reinterpret_cast<const uint32_t *>(&sA[ar + 8][tig * 2 + 8]);
+        constexpr int W = MLP_THREADS / 32;
+        const int aw = threadIdx.x >> 5;
+        float *part = tr.part + (int64_t)blockIdx.x * PART;
+        float *s_red = reinterpret_cast<float *>(s_w1 + FEAT * LDH);
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            // B fragment: k rows tig*2 (+1) and +8, column t*8 + gid
-            const int bc = t * 8 + gid;
-            uint32_t b0 = *reinterpret_cast<const uint32_t *>(&sB[bc][tig * 2]);
-            uint32_t b1 = *reinterpret_cast<const uint32_t *>(&sB[bc][tig * 2 + 8]);
-            asm volatile(
-                "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                "{%0,%1,%2,%3};\n"
-                : "+f"(acc[t][0]), "+f"(acc[t][1]), "+f"(acc[t][2]), "+f"(acc[t][3])
-                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+            s_red[aw * HID + lane + 32 * t] = gb2[t];
+            s_red[(W + aw) * HID + lane + 32 * t] = gw3[t];
+        }
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {                   // over the eight rows' lanes of a column
+            float v = gb1[t];
+            v += __shfl_xor_sync(0xffffffffu, v, 4);
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            if (gid == 0) s_red[(2 * W + group * 2 + mw) * HID + nw * 64 + (t >> 1) * 8 + tig * 2 + (t & 1)] = v;
+        }
+        float *s_one = s_red + (2 * W + 2 * MLP_GROUPS) * HID;
+        if (lane == 0) {
+            s_one[aw] = gb3;
+            s_one[W + aw] = loss;
         }
         __syncthreads();
-    }
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int m = m0 + warp * 16 + gid + (q >= 2 ? 8 : 0);
-            const int nn = n0 + t * 8 + tig * 2 + (q & 1);
-            if (m >= M || nn >= N) continue;
-            const float v = acc[t][q];
-            const int64_t o = (int64_t)m * N + nn;
-            if (EP == EP_F32) Cf[o] = v;
-            else if (EP == EP_F32_ACC) Cf[o] += v;
-            else if (EP == EP_BIAS_RELU) Cb[o] = __float2bfloat16(fmaxf(v + bias[nn], 0.f));
-            else Cf[o] = v + bias[nn];
+        if (group == 0) {
+            float a = 0.f, b = 0.f, c = 0.f;
+            for (int w = 0; w < W; ++w) { a += s_red[w * HID + tid]; b += s_red[(W + w) * HID + tid]; }
+            for (int w = 0; w < 2 * MLP_GROUPS; ++w) c += s_red[(2 * W + w) * HID + tid];
+            part[tid] = c;
+            part[HID + tid] = a;
+            part[2 * HID + tid] = b;
+            if (tid < 2) {
+                float v = 0.f;
+                for (int w = 0; w < W; ++w) v += s_one[tid * W + w];
+                part[3 * HID + tid] = v;
+            }
         }
-}
-
-// logits z[r] = h2[r, :] . w3 + b3 (one warp per row)
-__global__ void k_head(const __nv_bfloat16 *h2, const __nv_bfloat16 *w3, const float *b3, int64_t n, float *z) {
-    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (r >= n) return;
-    float s = 0.f;
-    for (int c = lane; c < HID; c += 32) s += bf(h2[r * HID + c]) * bf(w3[c]);
-    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-    if (lane == 0) z[r] = s + b3[0];
-}
-
-// Per row: the weighted logistic loss term, dz = w * (sigmoid(z) - y) / n and the
-// gradient at layer 2's pre-activation, dh2 = dz * w3 where the activation is positive.
-// Reductions over rows happen in the fixed-order kernels below (no float atomics), so a
-// training step is deterministic.
-__global__ void k_loss_rows(const float *z, const float *y, int64_t n, float pos_weight, const __nv_bfloat16 *h2,
-                            const __nv_bfloat16 *w3, float *dz, float *lrow, __nv_bfloat16 *dh2) {
-    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (r >= n) return;
-    const float zz = z[r], yy = y[r];
-    const float w = yy > 0.5f ? pos_weight : 1.f;
-    const float sg = 1.f / (1.f + __expf(-zz));
-    const float d = w * (sg - yy) / (float)n;
-    if (lane == 0) {
-        dz[r] = d;
-        const float sp = zz > 0.f ? zz + log1pf(__expf(-zz)) : log1pf(__expf(zz));
-        lrow[r] = w * (sp - yy * zz) / (float)n;
-    }
-    for (int c = lane; c < HID; c += 32) {
-        const float hv = bf(h2[r * HID + c]);
-        dh2[r * HID + c] = __float2bfloat16(hv > 0.f ? d * bf(w3[c]) : 0.f);
     }
 }
 
-// g_w3[c] = sum_r h2[r, c] * dz[r], one thread per column, rows in order
-__global__ void k_head_wgrad(const __nv_bfloat16 *h2, const float *dz, int64_t n, float *g_w3) {
-    const int c = threadIdx.x;
-    float s = 0.f;
-    for (int64_t r = 0; r < n; ++r) s += bf(h2[r * HID + c]) * dz[r];
-    g_w3[c] = s;
-}
+// The gradients of W2 (h1^T dh2) and W1 (x^T dh1): every entry is one chain of mma.sync over
+// the rows, 16 at a time in order, so what bounds it is the latency of 65,536 / 16
+// dependent products; the chains run side by side, 32 inputs x 32 outputs a CTA (two
+// chains a warp), 64 CTAs for W2 and 8 for W1, each reading only its columns through a
+// ring of cp.async stages.  Tiles of 64 x 64 with 2-byte loads took 16.8 ms of a 65,536-row
+// step, 0.23 ms so; chains split over the rows and added up would be faster still, but the
+// sums would differ from these by more than a re-ordering (3e-4: the tensor core truncates
+// what it aligns to a long chain's accumulator).
+constexpr int WG_ROWS = 64, WG_STAGES = 6, WG_COLS = 32, LDG = WG_COLS + 8;
+constexpr int WG_PROD = 128, WG_THREADS = WG_PROD + 256;   // four warps of products, then eight that fetch
+constexpr int WG_STAGE = 2 * WG_ROWS * LDG;              // bf16 values of a stage
+constexpr size_t WG_SMEM = sizeof(__nv_bfloat16) * WG_STAGES * WG_STAGE;
 
-// two fixed-order sums over n floats (one block of 256 threads): out0 = sum a, out1 = sum b
-__global__ void k_pair_sums(const float *a, const float *b, int64_t n, float *out0, float *out1) {
-    __shared__ float sa[256], sb[256];
-    float x = 0.f, w = 0.f;
-    for (int64_t r = threadIdx.x; r < n; r += 256) { x += a[r]; w += b[r]; }
-    sa[threadIdx.x] = x;
-    sb[threadIdx.x] = w;
-    __syncthreads();
-    for (int d = 128; d > 0; d >>= 1) {
-        if (threadIdx.x < d) { sa[threadIdx.x] += sa[threadIdx.x + d]; sb[threadIdx.x] += sb[threadIdx.x + d]; }
+__global__ void __launch_bounds__(WG_THREADS) k_mlp_wgrad(const __nv_bfloat16 *__restrict__ x,
+                                                          const __nv_bfloat16 *__restrict__ h1,
+                                                          const __nv_bfloat16 *__restrict__ dh1,
+                                                          const __nv_bfloat16 *__restrict__ dh2, int64_t n,
+                                                          float *__restrict__ g_w1, float *__restrict__ g_w2) {
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    __nv_bfloat16 *s = reinterpret_cast<__nv_bfloat16 *>(mlp_smem);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int mw = (warp >> 1) & 1, nw = warp & 1;       // a product warp's 16 x 16 entries
+    const bool first = blockIdx.x >= 64;                 // W1
+    const int i0 = first ? 0 : (blockIdx.x >> 3) * WG_COLS, o0 = (blockIdx.x & 7) * WG_COLS;
+    const int stages = (int)((n + WG_ROWS - 1) / WG_ROWS);
+    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    if (warp >= WG_PROD / 32) {
+        // warps 4 .. 11 fetch: a thread always takes the same 16-byte piece of a row, of A or of
+        // B, from every 32nd row; W1's A has two pieces, W2's four
+        const __nv_bfloat16 *A = first ? x : h1 + i0, *B = (first ? dh1 : dh2) + o0;
+        const int t = threadIdx.x - WG_PROD, c = t & 7, row0 = t >> 3;
+        const bool from_b = c >= 4, mine = from_b || c < (first ? FEAT / 8 : WG_COLS / 8);
+        const int ld = !from_b && first ? FEAT : HID;
+        const __nv_bfloat16 *src = (from_b ? B + (c - 4) * 8 : A + (mine ? c * 8 : 0)) + (int64_t)row0 * ld;
+        const bool aligned = (((uintptr_t)src) & 15) == 0;               // x is the caller's
+        __nv_bfloat16 *const dst = s + (from_b ? WG_ROWS * LDG + (c - 4) * 8 : c * 8) + row0 * LDG;
+        int left = (int)n - row0;                        // rows from this thread's next one on
+        int put = 0;                                     // ring slot of the next fetch
+        auto fetch = [&]() {
+            if (left > 0 && mine) {
+                __nv_bfloat16 *d = dst + put * WG_STAGE;
+                const uint32_t d32 = smem_u32(d);
+                if (aligned && left > 32) {
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d32), "l"(src));
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d32 + 32 * LDG * 2), "l"(src + 32 * ld));
+                } else {
+                    *reinterpret_cast<uint4 *>(d) = load8(src, aligned);
+                    *reinterpret_cast<uint4 *>(d + 32 * LDG) =
+                        left > 32 ? load8(src + 32 * ld, aligned) : make_uint4(0u, 0u, 0u, 0u);
+                }
+            } else if (mine) {                           // rows past the batch are zero
+                __nv_bfloat16 *d = dst + put * WG_STAGE;
+                *reinterpret_cast<uint4 *>(d) = make_uint4(0u, 0u, 0u, 0u);
+                *reinterpret_cast<uint4 *>(d + 32 * LDG) = make_uint4(0u, 0u, 0u, 0u);
+            }
+            src += (int64_t)WG_ROWS * ld;
+            left -= WG_ROWS;
+            put = put + 1 == WG_STAGES ? 0 : put + 1;
+            asm volatile("cp.async.commit_group;");
+        };
+#pragma unroll
+        for (int st = 0; st < WG_STAGES - 1; ++st) fetch();
+        for (int st = 0; st < stages; ++st) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(WG_STAGES - 2));
+            __syncthreads();                             // stage st is here, and stage st - 1 is read
+            fetch();
+        }
+        asm volatile("cp.async.wait_group 0;");
+        return;
+    }
+    const int q = lane >> 3;
+    const uint32_t a_at = smem_u32(s) + (uint32_t)((((lane & 7) + (q >> 1) * 8) * LDG + mw * 16 + (q & 1) * 8) * 2);
+    const uint32_t b_at = smem_u32(s) + (uint32_t)((WG_ROWS * LDG + (lane & 15) * LDG + nw * 16 + (lane >> 4) * 8) * 2);
+    uint32_t at = 0;                                     // byte offset of the stage in the ring
+    int rows = (int)n;                                   // rows from this stage on
+    for (int st = 0; st < stages; ++st) {
         __syncthreads();
+        if (!(first && mw == 1)) {                       // W1 has 16 inputs
+            uint32_t a[WG_ROWS / 16][4], b[WG_ROWS / 16][4];
+#pragma unroll
+            for (int k = 0; k < WG_ROWS / 16; ++k) {
+                ldsm4t(a[k], a_at + at + k * 16 * LDG * 2);
+                ldsm4t(b[k], b_at + at + k * 16 * LDG * 2);
+            }
+#pragma unroll
+            for (int k = 0; k < WG_ROWS / 16; ++k) {
+                if (k * 16 < rows) {
+                    mma16816(acc[0], a[k], b[k][0], b[k][1]);
+                    mma16816(acc[1], a[k], b[k][2], b[k][3]);
+                }
+            }
+        }
+        rows -= WG_ROWS;
+        at = at + WG_STAGE * 2 == WG_STAGES * WG_STAGE * 2 ? 0u : at + WG_STAGE * 2;
     }
-    if (threadIdx.x == 0) { *out0 = sa[0]; if (out1) *out1 = sb[0]; }
+    if (first && mw == 1) return;
+    float *out = first ? g_w1 : g_w2;
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            out[(i0 + mw * 16 + (lane >> 2) + (q >> 1) * 8) * HID + o0 + nw * 16 + t * 8 + (lane & 3) * 2 + (q & 1)] =
+                acc[t][q];
 }
 
-// dact = bf16(dpre where the activation is positive, else 0)
-__global__ void k_relu_back(const float *dpre, const __nv_bfloat16 *act, int64_t total, __nv_bfloat16 *dact) {
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x < total) dact[x] = __float2bfloat16(bf(act[x]) > 0.f ? dpre[x] : 0.f);
-}
+// Every parameter's Adam step on its float32 master, with the gradients of the biases and
+// W3 summed here from the CTAs' partial sums (in order); refreshes the bf16 copies.  The
+// last thread sums the loss.
+struct adam_args {
+    float *w1, *b1, *w2, *b2, *w3, *b3;
+    __nv_bfloat16 *w1b, *w2b, *w3b;
+    float *grad, *m, *v, *loss;
+    float lr, beta1, beta2, eps, c1, c2;
+};
 
-// g_b[c] = sum_r (masked) values of column c, rows in order (f32 input or bf16 input)
-__global__ void k_colsum_masked_f32(const float *dpre, const __nv_bfloat16 *act, int64_t n, float *g_b) {
-    const int c = threadIdx.x;
-    float s = 0.f;
-    for (int64_t r = 0; r < n; ++r) s += bf(act[r * HID + c]) > 0.f ? dpre[r * HID + c] : 0.f;
-    g_b[c] = s;
-}
-
-__global__ void k_colsum_bf16(const __nv_bfloat16 *d, int64_t n, float *g_b) {
-    const int c = threadIdx.x;
-    float s = 0.f;
-    for (int64_t r = 0; r < n; ++r) s += bf(d[r * HID + c]);
-    g_b[c] = s;
-}
-
-// Adam on float32 masters; refreshes the bf16 copies
-__global__ void k_adam(float *w, float *m1, float *m2, const float *g, __nv_bfloat16 *wb, int64_t n, float lr,
-                       float b1, float b2, float eps, float c1, float c2) {
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= n) return;
-    const float gg = g[x];
-    const float a = b1 * m1[x] + (1.f - b1) * gg;
-    const float b = b2 * m2[x] + (1.f - b2) * gg * gg;
-    m1[x] = a;
-    m2[x] = b;
-    const float v = w[x] - lr * (a / c1) / (sqrtf(b / c2) + eps);
-    w[x] = v;
-    if (wb) wb[x] = __float2bfloat16(v);
+__global__ void __launch_bounds__(256) k_mlp_adam(adam_args a, const float *__restrict__ part, int n_part) {
+    constexpr int NW1 = FEAT * HID, NW2 = HID * HID, O1 = NW1, O2 = O1 + HID, O3 = O2 + NW2, O4 = O3 + HID,
+                  O5 = O4 + HID, N = O5 + 1;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x > N || (x == N && !a.loss)) return;
+    float g;
+    if (x < O1 || (x >= O2 && x < O3)) {
+        g = a.grad[x];
+    } else {
+        const float *p = part + (x < O2 ? x - O1 : x - O3 + HID);     // b1, then b2, w3, b3, loss
+        g = 0.f;
+#pragma unroll 8
+        for (int q = 0; q < n_part; ++q) g += p[q * PART];
+        if (x == N) { *a.loss = g; return; }
+        a.grad[x] = g;
+    }
+    float *w;
+    __nv_bfloat16 *wb = nullptr;
+    if (x < O1) { w = a.w1 + x; wb = a.w1b + x; }
+    else if (x < O2) w = a.b1 + (x - O1);
+    else if (x < O3) { w = a.w2 + (x - O2); wb = a.w2b + (x - O2); }
+    else if (x < O4) w = a.b2 + (x - O3);
+    else if (x < O5) { w = a.w3 + (x - O4); wb = a.w3b + (x - O4); }
+    else w = a.b3;
+    const float m = a.beta1 * a.m[x] + (1.f - a.beta1) * g;
+    const float v = a.beta2 * a.v[x] + (1.f - a.beta2) * g * g;
+    a.m[x] = m;
+    a.v[x] = v;
+    const float nw = *w - a.lr * (m / a.c1) / (sqrtf(v / a.c2) + a.eps);
+    *w = nw;
+    if (wb) *wb = __float2bfloat16(nw);
 }
 
 __global__ void k_select(const pastis_cand *pairs, const float *z, int64_t n, float thr, uint32_t *flags) {
@@ -242,17 +543,6 @@ __global__ void k_select_scatter(const pastis_cand *pairs, const uint32_t *flags
                                  pastis_cand *out) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p < n && flags[p]) out[off[p]] = pairs[p];
-}
-
-template <bool TA, bool TB, int EP>
-pastis_status gemm(pastis_ctx *ctx, const __nv_bfloat16 *A, const __nv_bfloat16 *B, int M, int N, int K,
-                   const float *bias, float *Cf, __nv_bfloat16 *Cb) {
-    dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
-    prof_begin(ctx, "mlp_gemm");
-    k_gemm_bf16<TA, TB, EP><<<grid, 128, 0, ctx->stream>>>(A, B, M, N, K, bias, Cf, Cb);
-    PASTIS_LAUNCHED(ctx);
-    prof_end(ctx);
-    return PASTIS_OK;
 }
 
 }  // namespace
@@ -289,38 +579,18 @@ extern "C" pastis_status pastis_pair_features_qt(pastis_ctx *ctx, const uint8_t 
     return features_qt(ctx, d_qcodes, d_qoffsets, d_tcodes, d_toffsets, d_pairs, n_pairs, params, d_x);
 }
 
-// Scratch activations for n rows: h1, h2 (bf16 n x 256), z (f32 n), and for training
-// dpre (f32 n x 256), dh (bf16 n x 256), dz (f32 n).
-static pastis_status mlp_scratch(pastis_ctx *ctx, int64_t n, bool train, __nv_bfloat16 **h1, __nv_bfloat16 **h2,
-                                 float **z, float **dpre, __nv_bfloat16 **dh, float **dz) {
-    size_t bytes = (size_t)n * HID * 2 * 2 + (size_t)n * 4 + 256;
-    if (train) bytes += (size_t)n * HID * 4 + (size_t)n * HID * 2 + (size_t)n * 4 + 256;
-    char *b;
-    PASTIS_WS(b, ctx, WS_MLP, bytes);
-    *h1 = (__nv_bfloat16 *)b; b += (size_t)n * HID * 2;
-    *h2 = (__nv_bfloat16 *)b; b += (size_t)n * HID * 2;
-    *z = (float *)b; b += ((size_t)n * 4 + 255) & ~(size_t)255;
-    if (train) {
-        *dpre = (float *)b; b += (size_t)n * HID * 4;
-        *dh = (__nv_bfloat16 *)b; b += (size_t)n * HID * 2;
-        *dz = (float *)b;
-    }
-    return PASTIS_OK;
+static mlp_w mlp_weights(const pastis_mlp *net) {
+    return mlp_w{(const __nv_bfloat16 *)net->w1b, (const __nv_bfloat16 *)net->w2b, (const __nv_bfloat16 *)net->w3b,
+                 net->b1, net->b2, net->b3};
 }
 
-static pastis_status mlp_fwd(pastis_ctx *ctx, const pastis_mlp *net, const __nv_bfloat16 *x, int64_t n,
-                             __nv_bfloat16 *h1, __nv_bfloat16 *h2, float *z) {
-    pastis_status s = gemm<false, false, EP_BIAS_RELU>(ctx, x, (const __nv_bfloat16 *)net->w1b, (int)n, HID, FEAT,
-                                                       net->b1, nullptr, h1);
-    if (s != PASTIS_OK) return s;
-    s = gemm<false, false, EP_BIAS_RELU>(ctx, h1, (const __nv_bfloat16 *)net->w2b, (int)n, HID, HID, net->b2, nullptr, h2);
-    if (s != PASTIS_OK) return s;
-    prof_begin(ctx, "mlp_head");
-    k_head<<<(unsigned)ceil_div64(n * 32, 256), 256, 0, ctx->stream>>>(h2, (const __nv_bfloat16 *)net->w3b, net->b3,
-                                                                       n, z);
-    PASTIS_LAUNCHED(ctx);
-    prof_end(ctx);
-    return PASTIS_OK;
+cudaError_t mlp_set_smem_limit() {
+    cudaError_t e = cudaFuncSetAttribute(k_mlp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MLP_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MLP_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM);
+    return e;
 }
 
 extern "C" pastis_status pastis_mlp_forward(pastis_ctx *ctx, const pastis_mlp *net, const void *d_x, int64_t n,
@@ -328,16 +598,12 @@ extern "C" pastis_status pastis_mlp_forward(pastis_ctx *ctx, const pastis_mlp *n
     if (!ctx || !net || n < 0 || n > (1 << 30)) return PASTIS_ERR_INVALID_ARG;
     if (n == 0) return PASTIS_OK;
     if (!d_x || !d_logits) return PASTIS_ERR_INVALID_ARG;
-    const int64_t chunk = 1 << 20;
-    for (int64_t r0 = 0; r0 < n; r0 += chunk) {
-        const int64_t nr = n - r0 < chunk ? n - r0 : chunk;
-        __nv_bfloat16 *h1, *h2, *dh;
-        float *z, *dpre, *dz;
-        pastis_status s = mlp_scratch(ctx, nr, false, &h1, &h2, &z, &dpre, &dh, &dz);
-        if (s != PASTIS_OK) return s;
-        s = mlp_fwd(ctx, net, (const __nv_bfloat16 *)d_x + r0 * FEAT, nr, h1, h2, d_logits + r0);
-        if (s != PASTIS_OK) return s;
-    }
+    const unsigned grid = (unsigned)std::min<int64_t>(ceil_div64(n, TM), ctx->sm_count);
+    prof_begin(ctx, "mlp_forward");
+    k_mlp<false><<<grid, MLP_THREADS, MLP_SMEM, ctx->stream>>>(mlp_weights(net), (const __nv_bfloat16 *)d_x, n, d_logits,
+                                                               mlp_train_io{});
+    PASTIS_LAUNCHED(ctx);
+    prof_end(ctx);
     return PASTIS_OK;
 }
 
@@ -345,64 +611,42 @@ extern "C" pastis_status pastis_mlp_train_step(pastis_ctx *ctx, pastis_mlp *net,
                                                int64_t n, float lr, float pos_weight, float *d_loss) {
     if (!ctx || !net || n <= 0 || n > (1 << 22) || !d_x || !d_y) return PASTIS_ERR_INVALID_ARG;
     cudaStream_t st = ctx->stream;
-    __nv_bfloat16 *h1, *h2, *dh;
-    float *z, *dpre, *dz;
-    pastis_status s = mlp_scratch(ctx, n, true, &h1, &h2, &z, &dpre, &dh, &dz);
-    if (s != PASTIS_OK) return s;
-    const __nv_bfloat16 *x = (const __nv_bfloat16 *)d_x;
-    s = mlp_fwd(ctx, net, x, n, h1, h2, z);
-    if (s != PASTIS_OK) return s;
-    // gradients (zeroed) live after the parameters in the grad buffer
-    const int64_t nw1 = FEAT * HID, nw2 = HID * HID;
-    float *g = net->grad;
-    float *g_w1 = g, *g_b1 = g_w1 + nw1, *g_w2 = g_b1 + HID, *g_b2 = g_w2 + nw2, *g_w3 = g_b2 + HID, *g_b3 = g_w3 + HID;
-    const int64_t ntot = nw1 + HID + nw2 + HID + HID + 1;
-    PASTIS_CUDA_TRY(cudaMemsetAsync(g, 0, sizeof(float) * ntot, st));
-    float *loss = d_loss;   // may be null
-    // per-row loss terms and dz share one float buffer of 2n after z
-    float *lrow;
-    PASTIS_WS(lrow, ctx, WS_FILT_SCAN, sizeof(float) * (size_t)n + 64);
-    prof_begin(ctx, "mlp_loss");
-    k_loss_rows<<<(unsigned)ceil_div64(n * 32, 256), 256, 0, st>>>(z, d_y, n, pos_weight, h2,
-                                                                   (const __nv_bfloat16 *)net->w3b, dz, lrow, dh);
+    // scratch: h1, dh1 and dh2 (bf16 n x 256), the logits, and the partial sums of the gradients
+    const int grid = (int)std::min<int64_t>(ceil_div64(n, TM), ctx->sm_count);
+    const size_t act = (size_t)n * HID * 2, zb = ((size_t)n * 4 + 255) & ~(size_t)255;
+    const size_t pb = ((size_t)grid * PART * 4 + 255) & ~(size_t)255;
+    char *b;
+    PASTIS_WS(b, ctx, WS_MLP, 3 * act + zb + pb);
+    mlp_train_io tr;
+    tr.y = d_y;
+    tr.pos_weight = pos_weight;
+    tr.h1 = (__nv_bfloat16 *)b;
+    tr.dh1 = (__nv_bfloat16 *)(b + act);
+    tr.dh2 = (__nv_bfloat16 *)(b + 2 * act);
+    float *z = (float *)(b + 3 * act);
+    tr.part = (float *)(b + 3 * act + zb);
+    prof_begin(ctx, "mlp_train");
+    k_mlp<true><<<grid, MLP_THREADS, MLP_SMEM, st>>>(mlp_weights(net), (const __nv_bfloat16 *)d_x, n, z, tr);
     PASTIS_LAUNCHED(ctx);
     prof_end(ctx);
-    k_head_wgrad<<<1, HID, 0, st>>>(h2, dz, n, g_w3);
+    prof_begin(ctx, "mlp_wgrad");
+    k_mlp_wgrad<<<64 + 8, WG_THREADS, WG_SMEM, st>>>((const __nv_bfloat16 *)d_x, tr.h1, tr.dh1, tr.dh2, n, net->grad,
+                                                    net->grad + FEAT * HID + HID);
     PASTIS_LAUNCHED(ctx);
-    k_pair_sums<<<1, 256, 0, st>>>(dz, lrow, n, g_b3, loss);
-    PASTIS_LAUNCHED(ctx);
-    // layer 2: g_w2 = h1^T dh2, g_b2 = colsum(dh2), dpre1 = dh2 w2^T
-    s = gemm<true, false, EP_F32>(ctx, h1, dh, HID, HID, (int)n, nullptr, g_w2, nullptr);
-    if (s != PASTIS_OK) return s;
-    k_colsum_bf16<<<1, HID, 0, st>>>(dh, n, g_b2);
-    PASTIS_LAUNCHED(ctx);
-    s = gemm<false, true, EP_F32>(ctx, dh, (const __nv_bfloat16 *)net->w2b, (int)n, HID, HID, nullptr, dpre, nullptr);
-    if (s != PASTIS_OK) return s;
-    // back through the ReLU of layer 1 (dh now holds the layer-1 gradient), g_b1
-    k_colsum_masked_f32<<<1, HID, 0, st>>>(dpre, h1, n, g_b1);
-    PASTIS_LAUNCHED(ctx);
-    k_relu_back<<<(unsigned)ceil_div64(n * HID, 256), 256, 0, st>>>(dpre, h1, n * HID, dh);
-    PASTIS_LAUNCHED(ctx);
-    // layer 1: g_w1 = x^T dh1
-    s = gemm<true, false, EP_F32>(ctx, x, dh, FEAT, HID, (int)n, nullptr, g_w1, nullptr);
-    if (s != PASTIS_OK) return s;
-    // Adam
+    prof_end(ctx);
     net->step += 1;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.f - powf(b1, (float)net->step);
-    const float c2 = 1.f - powf(b2, (float)net->step);
-    struct seg { float *w; __nv_bfloat16 *wb; int64_t off, n; } segs[6] = {
-        {net->w1, (__nv_bfloat16 *)net->w1b, 0, nw1}, {net->b1, nullptr, nw1, HID},
-        {net->w2, (__nv_bfloat16 *)net->w2b, nw1 + HID, nw2}, {net->b2, nullptr, nw1 + HID + nw2, HID},
-        {net->w3, (__nv_bfloat16 *)net->w3b, nw1 + 2 * HID + nw2, HID}, {net->b3, nullptr, nw1 + 3 * HID + nw2, 1}};
-    for (int q = 0; q < 6; ++q) {
-        prof_begin(ctx, "mlp_adam");
-        k_adam<<<(unsigned)ceil_div64(segs[q].n, 256), 256, 0, st>>>(segs[q].w, net->adam_m + segs[q].off,
-                                                                     net->adam_v + segs[q].off, g + segs[q].off,
-                                                                     segs[q].wb, segs[q].n, lr, b1, b2, 1e-8f, c1, c2);
-        PASTIS_LAUNCHED(ctx);
-        prof_end(ctx);
-    }
+    adam_args a;
+    a.w1 = net->w1; a.b1 = net->b1; a.w2 = net->w2; a.b2 = net->b2; a.w3 = net->w3; a.b3 = net->b3;
+    a.w1b = (__nv_bfloat16 *)net->w1b; a.w2b = (__nv_bfloat16 *)net->w2b; a.w3b = (__nv_bfloat16 *)net->w3b;
+    a.grad = net->grad; a.m = net->adam_m; a.v = net->adam_v; a.loss = d_loss;
+    a.lr = lr; a.beta1 = 0.9f; a.beta2 = 0.999f; a.eps = 1e-8f;
+    a.c1 = 1.f - powf(a.beta1, (float)net->step);
+    a.c2 = 1.f - powf(a.beta2, (float)net->step);
+    const int np = FEAT * HID + HID * HID + 3 * HID + 2;
+    prof_begin(ctx, "mlp_adam");
+    k_mlp_adam<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(a, tr.part, grid);
+    PASTIS_LAUNCHED(ctx);
+    prof_end(ctx);
     return PASTIS_OK;
 }
 

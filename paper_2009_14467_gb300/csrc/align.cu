@@ -988,14 +988,15 @@ static pastis_status align_qt(pastis_ctx *ctx, const uint8_t *d_qcodes, const in
     PASTIS_WS(dmat, ctx, WS_FLAGS, 1024);
     int *flags = (int *)(dmat + 768);   // [0] error, [1] [3] [8] pair counters, [2] max length, [4] bad pair,
                                         // [5] bad code, [6..7] [12..13] [14..15] [16..17] task counters,
-                                        // [9] [18] the 16-bit x-drop's deferred tasks (without, with carries)
+                                        // [9] [18] the 16-bit x-drop's deferred tasks (without, with carries),
+                                        // [20..23] Smith-Waterman's banded pairs (four lists), [24..27] their counters
     // the matrix, then the pass-1 layout at dmat + 640
     uint8_t hconst[640 + PASTIS_SW_BINS];
     memcpy(hconst, params->matrix, 576);
     memset(hconst + 576, 0, 64);
     memcpy(hconst + 640, ctx->sw_lay.extra, PASTIS_SW_BINS);
     if (!g) PASTIS_CUDA_TRY(cudaMemcpyAsync(dmat, hconst, sizeof(hconst), cudaMemcpyHostToDevice, st));
-    PASTIS_CUDA_TRY(cudaMemsetAsync(flags, 0, 80, st));
+    PASTIS_CUDA_TRY(cudaMemsetAsync(flags, 0, 112, st));
     const int xd = params->mode == PASTIS_XD || params->mode == PASTIS_XD_FILTERED;
     const int xd_filtered = params->mode == PASTIS_XD_FILTERED;
     const int64_t *dn = g ? g->dc : nullptr;

@@ -19,7 +19,7 @@ enum ws_slot {
     WS_AS_TMP_KEY, WS_AS_KEEP,
     WS_SPG_ROWWORK, WS_SPG_ROWOFF, WS_SPG_TMP, WS_SPG_CURSORS, WS_SPG_BIN,
     WS_SPG_RESULT,
-    WS_ALN_SCRATCH, WS_ALN_PASS1, WS_ALN_ORDER, WS_ALN_BOUND, WS_ALN_BOFF,
+    WS_ALN_SCRATCH, WS_ALN_PASS1, WS_ALN_ORDER, WS_ALN_BOUND, WS_ALN_BOFF, WS_ALN_BAND,
     WS_FILT_FLAGS, WS_FILT_SCAN, WS_CC,
     WS_MLP,
     WS_TUNE,

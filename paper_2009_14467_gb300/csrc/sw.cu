@@ -21,16 +21,17 @@
 //   Queries longer than one stripe of 32 * 32 rows go in stripes whose last row is
 //   handed on through a per-warp buffer.
 // Pass 2 (its own kernel, one warp per pair; a band around the path): an anchored DP
-//   over the reversed prefixes from the end (ei, ej), row by row with up to 64 columns
-//   per row (two per lane; antidiagonal by antidiagonal when a row needs more or the
+//   over the reversed prefixes from the end (ei, ej), row by row with up to 128 columns
+//   per row (four per lane; antidiagonal by antidiagonal when a row needs more or the
 //   gap costs have o < e).  A suffix of the traced path starting on row i scores S minus
 //   the forward value before it, which is at most the largest H pass 1 met on row
 //   i-1's pair of rows; cells below that threshold die, the path's suffixes all
 //   survive, and the cells reaching S bound the begin.  Their extent gives a rectangle
 //   that contains the whole traced path.
-// Pass 3 (that rectangle): the DP again with zero boundaries; each state carries its
-//   begin cell and (identities << 16 | matched columns) along the predecessor a
-//   traceback would take.  Inside a rectangle holding the path, the path's cells keep
+// Pass 3 (k_sw_band: inside the columns that pass 2 left each row, where it kept them;
+//   k_sw_carry: the whole rectangle): the DP again with zero boundaries; each state
+//   carries its begin cell and (identities << 16 | matched columns) along the predecessor a
+//   traceback would take.  Inside a region holding the path, the path's cells keep
 //   their values and every choice along it is the same, so the carry at the end cell
 //   is the traceback's.  cols = span_q + span_t - matched.
 // Pairs whose scores could reach SCORE_MAX (max score * shorter length), gap opens
@@ -56,7 +57,8 @@ struct sw_score_out {                      // pass 1 result per pair
     int32_t score;
     int32_t end_i, end_j;
     int32_t rect_i, rect_j;                // pass 2: start of the bounding rectangle
-    int32_t big;                           // scores may not fit the pass-1 key
+    int32_t big;                           // 1: not scored by pass 1 (k_sw_carry takes the whole
+                                           // matrix); 2: pass 2 listed the pair for k_sw_band
 };
 
 // The filter-only mode (PASTIS_SW_FILTERED): the traced path lies in the rectangle
@@ -439,6 +441,9 @@ __device__ __forceinline__ void score_rows(const sw_tile &tl, const uint8_t *pro
 // the two antidiagonals before come by shuffles.  A live band wider than BAND cells
 // returns false and the caller keeps the whole up-left rectangle.
 constexpr int BAND = 64;
+// Paths of at most this many rows take k_sw_carry (four rectangles a warp), longer ones with
+// a row-by-row band k_sw_band.
+constexpr int BAND_MIN_ROWS = 24;
 
 // The value the previous antidiagonal holds at band index idx (NEG outside the band).
 // `wide` is the same on every lane.
@@ -519,110 +524,174 @@ __device__ __noinline__ bool band_walk(const uint8_t *__restrict__ q, const uint
     return true;
 }
 
-// The value the previous row holds at window index idx (two columns per lane; NEG
-// outside the window).  `wide` (the previous row used its second chunk) is the same
-// on every lane.
-__device__ __forceinline__ int row_get(const int (&X)[2], int idx, bool wide) {
-    const int v0 = __shfl_sync(0xffffffffu, X[0], idx & 31);
-    int v = v0;
-    if (wide) {
-        const int v1 = __shfl_sync(0xffffffffu, X[1], idx & 31);
-        v = idx >= 32 ? v1 : v0;
-    }
-    return (unsigned)idx < (wide ? 64u : 32u) ? v : NEG;
-}
+// The same reverse DP row by row, for o >= e.  The row's columns c0 .. lie in chunks of 32,
+// lane L holding column c0 + 32 c + L of each: H, F and the target residue, which stay in
+// their lanes from row to row, so that only the diagonal comes by shuffle; when moving the
+// window to the first live column saves a chunk, the values are shifted there.  E along the
+// row is an exclusive prefix maximum over the columns to the left, taken over max(D, F):
+// with o >= e a gap that E itself opened never beats extending E, and as the threshold is
+// the same along a row, a gap run through a cell below it stays below it; it is formed
+// only when some cell is high enough for a gap opened there to stay alive.  So the live
+// cells and their values are those of the antidiagonal form.  Returns false when a row
+// needs more than ROW_COLS columns: near the begin of a path another alignment often holds
+// the largest H of a row, the threshold is low, and some 60 to 100 columns stay alive.
+// band[k] (null: not wanted) receives, for the forward rows ei - 8 k - 7 .. ei - 8 k, the
+// first and the last (<< 16) column that the traced path can visit there: a diagonal step
+// at forward cell (i, j) starts a suffix at reverse cell (a, b) = (ei - i + 1, ej - j + 1); a
+// step of a vertical gap at (i, j) one at (a, b - 1), so the row's range reaches one column
+// further left; a step of a horizontal gap one at (a - 1, b), so it takes in the range of
+// the row below.
+// Measured: 10^5 pairs of 1,000 residues 7.3 ms with the window moved every row, 64 columns
+// and E formed always, 5.7 ms so; 10^6 pairs of 20,000 proteins 8.7 -> 7.5 ms.
+constexpr int ROW_CHUNKS = 4;
+constexpr int ROW_COLS = 32 * ROW_CHUNKS;
 
-// The same reverse DP row by row, for o >= e: lane L holds columns c0 + L and
-// c0 + 32 + L of reverse row a, where c0 is the first live column of row a - 1 (no
-// cell left of it has a live predecessor).  E along the row is an exclusive prefix
-// maximum over the columns to the left, taken over max(D, F): with o >= e a gap that
-// E itself opened never beats extending E, and as the threshold is the same along a
-// row, a gap run through a cell below it stays below it.  So the live cells and their
-// values are those of the antidiagonal form.  Returns false when a row needs more
-// than 64 columns.
 __device__ bool band_rows(const uint8_t *__restrict__ q, const uint8_t *__restrict__ t, const int *s_mat, int o,
                           int e, int S, int ei, int ej, const int16_t *__restrict__ bm, int *amax_out,
-                          int *bmax_out) {
+                          int *bmax_out, uint32_t *__restrict__ band) {
     const int lane = threadIdx.x & 31;
     const int A = ei + 1, B = ej + 1;
     const int slack = max(o - e, 0);
-    int Hp[2] = {NEG, NEG}, Fp[2] = {NEG, NEG};        // row a - 1 at columns c0p + 32 c + lane
-    int c0p = 0, plo = 0, phi = -1;                     // its window start and live columns
-    bool pwide = false;
-    int amax = 0, bmax = 0;
-    for (int a = 0; a <= A; ++a) {
-        if (a > 0 && phi < plo) break;                  // row a - 1 had no live cell
-        const int c0 = a == 0 ? 0 : plo;
-        if (a > 0 && phi + 1 > c0 + 63) return false;   // its diagonal successors leave the window
-        const int i = ei - a + 1;                       // forward row of this reverse row
-        const int thr = S - (i >= 1 ? (int)bm[(i - 1) >> 1] : 0) - slack;
-        const int qa = a >= 1 ? (int)q[i] * PASTIS_NSYM : 0;
-        const int dsh = c0 - c0p;
-        int H[2] = {NEG, NEG}, F[2] = {NEG, NEG};
-        unsigned live[2] = {0u, 0u};
-        int carry = NEG;                                // max of max(D, F) + k e left of the chunk
-        int tb = -1;                                    // this lane's largest column reaching S
-        bool wide = false;
+    int H[ROW_CHUNKS], F[ROW_CHUNKS], tc[ROW_CHUNKS];   // row a - 1, then row a; residue of column b
+    int c0 = 0, plo = 0, phi = 0;                       // window start; live columns of row a - 1
+    auto residue = [&](int b) { return b >= 1 && b <= B ? (int)t[ej - b + 1] : 0; };
+    // row 0: the end (column 0), and the gaps opened from it
+    const int thr0 = S - (int)bm[ei >> 1] - slack;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            if (c == 1) {
-                // the second chunk when row a - 1 reaches past the first, or an E run
-                // leaves it still at or above the threshold
-                const int e_next = carry - o - 31 * e;
-                if (!(phi + 1 > c0 + 31 || e_next >= thr)) break;
-                wide = true;
-            }
-            const int k = 32 * c + lane, b = c0 + k;
-            const int src = k + dsh;
-            const int hb = row_get(Hp, src, pwide), fb = row_get(Fp, src, pwide);
-            const int hd = row_get(Hp, src - 1, pwide);
-            int hh = NEG, fv = NEG;
-            if (b <= B) {
-                if (a >= 1) {
-                    fv = max(max(hb - o, fb - e), NEG);
-                    const int dv = (b >= 1 && hd != NEG) ? hd + s_mat[qa + (int)t[ej - b + 1]] : NEG;
-                    hh = max(dv, fv);
-                } else if (b == 0) {
-                    hh = 0;                             // the end cell
+    for (int c = 0; c < ROW_CHUNKS; ++c) {
+        const int b = 32 * c + lane;
+        const int h = b == 0 ? 0 : (b <= B ? -o - (b - 1) * e : NEG);
+        H[c] = h >= thr0 ? h : NEG;
+        F[c] = NEG;
+        tc[c] = residue(b);
+        const unsigned live = __ballot_sync(0xffffffffu, H[c] != NEG);
+        if (live) phi = 32 * c + 31 - __clz(live);
+    }
+    if (0 < thr0) plo = 1, phi = 0;                     // the end itself below its threshold
+    else if (phi == ROW_COLS - 1 && -o - (ROW_COLS - 1) * e >= thr0 && ROW_COLS <= B) return false;
+    int amax = 0, bmax = 0;
+    int alive = 0;                                      // the last row with a live cell
+    int blo = plo, bhi = phi;                           // live columns of the block's rows and the row below it
+    auto put_band = [&](int k) {
+        if (lane == 0) band[k] = (uint32_t)max(ej - bhi, 0) | (uint32_t)min(ej - blo + 1, ej) << 16;
+    };
+    for (int a = 1; a <= A && plo <= phi; ++a) {
+        if (phi + 1 - plo >= ROW_COLS) return false;    // the diagonal successors leave the window
+        if (((phi + 1 - plo) >> 5) < ((phi + 1 - c0) >> 5)) {
+            const int sh = plo - c0, lane_to = (lane + sh) & 31;
+            for (int x = sh >> 5; x > 0; --x) {         // whole chunks
+#pragma unroll
+                for (int c = 0; c < ROW_CHUNKS; ++c) {
+                    H[c] = c + 1 < ROW_CHUNKS ? H[(c + 1) % ROW_CHUNKS] : NEG;
+                    F[c] = c + 1 < ROW_CHUNKS ? F[(c + 1) % ROW_CHUNKS] : NEG;
                 }
             }
-            int incl = hh > NEG ? hh + k * e : NEG;
+            const bool own = lane + (sh & 31) < 32;
 #pragma unroll
-            for (int x = 1; x < 32; x <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, x);
-                if (lane >= x) incl = max(incl, y);
+            for (int c = 0; c < ROW_CHUNKS; ++c) {
+                const int h0 = __shfl_sync(0xffffffffu, H[c], lane_to), f0 = __shfl_sync(0xffffffffu, F[c], lane_to);
+                int h1 = NEG, f1 = NEG;
+                if (c + 1 < ROW_CHUNKS) {
+                    h1 = __shfl_sync(0xffffffffu, H[(c + 1) % ROW_CHUNKS], lane_to);
+                    f1 = __shfl_sync(0xffffffffu, F[(c + 1) % ROW_CHUNKS], lane_to);
+                }
+                H[c] = own ? h0 : h1;
+                F[c] = own ? f0 : f1;
             }
-            int excl = __shfl_up_sync(0xffffffffu, incl, 1);
-            if (lane == 0) excl = NEG;
-            excl = max(excl, carry);
-            carry = max(carry, __shfl_sync(0xffffffffu, incl, 31));
-            const int ev = (b >= 1 && excl > NEG) ? excl - o - (k - 1) * e : NEG;
-            int h = max(hh, ev);
-            if (b > B || h < thr) { h = NEG; fv = NEG; }
-            H[c] = h; F[c] = fv;
-            live[c] = __ballot_sync(0xffffffffu, h != NEG);
-            if (h == S) tb = b;
+            c0 = plo;
+#pragma unroll
+            for (int c = 0; c < ROW_CHUNKS; ++c) tc[c] = residue(c0 + 32 * c + lane);
         }
-        if (wide) {
-            // a live run still going past the second chunk needs more than 64 columns
-            if (carry - o - 63 * e >= thr) return false;
+        const int i = ei - a + 1;                       // forward row of this reverse row
+        const int thr = S - (i >= 1 ? (int)bm[(i - 1) >> 1] : 0) - slack;
+        const int *row = s_mat + (int)q[i] * PASTIS_NSYM;
+        int carry = NEG;                                // max of max(D, F) + k e left of the chunk
+        int left = NEG;                                 // H of row a - 1 in the column before the chunk
+        int tb = -1;                                    // this lane's largest column reaching S
+        int nlo = 0x7FFFFFFF, nhi = -1;                 // live columns of this row
+        bool more = false;
+#pragma unroll
+        for (int c = 0; c < ROW_CHUNKS; ++c) {
+            // as far as row a - 1 reaches, or a gap run that stays at or above the threshold
+            more = carry - o - (32 * c - 1) * e >= thr;
+            if (phi + 1 < c0 + 32 * c && !more) break;
+            const int k = 32 * c + lane, b = c0 + k;
+            int hd = __shfl_up_sync(0xffffffffu, H[c], 1);
+            if (lane == 0) hd = left;
+            left = __shfl_sync(0xffffffffu, H[c], 31);
+            int fv = max(max(H[c] - o, F[c] - e), NEG);
+            int h = max(hd != NEG ? hd + row[tc[c]] : NEG, fv);
+            if (b > B) h = NEG;
+            if (more || __any_sync(0xffffffffu, h - o >= thr)) {
+                int incl = h > NEG ? h + k * e : NEG;
+#pragma unroll
+                for (int x = 1; x < 32; x <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, incl, x);
+                    if (lane >= x) incl = max(incl, y);
+                }
+                int excl = __shfl_up_sync(0xffffffffu, incl, 1);
+                if (lane == 0) excl = NEG;
+                excl = max(excl, carry);
+                carry = max(carry, __shfl_sync(0xffffffffu, incl, 31));
+                if (excl > NEG && b <= B) h = max(h, excl - o - (k - 1) * e);
+            }
+            const bool dead = h < thr || b > B;
+            H[c] = dead ? NEG : h;
+            F[c] = dead ? NEG : fv;
+            const unsigned live = __ballot_sync(0xffffffffu, !dead);
+            if (live) {
+                nlo = min(nlo, c0 + 32 * c + __ffs(live) - 1);
+                nhi = c0 + 32 * c + 31 - __clz(live);
+            }
+            if (!dead && h == S) tb = b;
+            if (c + 1 == ROW_CHUNKS) more = carry - o - (ROW_COLS - 1) * e >= thr;
+            else more = false;
         }
+        if (more) return false;                         // a run still going past the last chunk
         if (__any_sync(0xffffffffu, tb >= 0)) {
             amax = a;
             bmax = max(bmax, __reduce_max_sync(0xffffffffu, tb < 0 ? 0 : tb));
         }
-        Hp[0] = H[0]; Hp[1] = H[1]; Fp[0] = F[0]; Fp[1] = F[1];
-        c0p = c0; pwide = wide;
-        if (live[0] | live[1]) {
-            plo = c0 + (live[0] ? __ffs(live[0]) - 1 : 32 + __ffs(live[1]) - 1);
-            phi = c0 + (live[1] ? 63 - __clz(live[1]) : 31 - __clz(live[0]));
+        if (nhi >= 0) {
+            plo = nlo; phi = nhi;
+            blo = min(blo, plo);
+            bhi = max(bhi, phi);
+            alive = a;
+            if ((a & 7) == 0) {
+                if (band) put_band((a - 1) >> 3);
+                blo = plo;
+                bhi = phi;
+            }
         } else {
             plo = 1; phi = 0;
         }
     }
+    if (band && (alive & 7) != 0) put_band((alive - 1) >> 3);     // the last block, partly filled
     *amax_out = amax;
     *bmax_out = bmax;
     return true;
+}
+
+// Where the block ranges of pair p start (entries of bm_off are row pairs, four to a block;
+// one more per pair covers the rounding).
+__device__ __forceinline__ int64_t band_at(int64_t bm_off, int64_t p) { return (bm_off >> 2) + p; }
+
+// Four lists of pairs in two arrays of one entry per pair: rings of 4 and 16 lanes from the
+// two ends of the first, of 8 and 32 of the second.
+constexpr int BAND_RINGS = 4;
+__host__ __device__ __forceinline__ int64_t band_slot(int ring, int x, int64_t cap) {
+    return (ring & 1) * cap + (ring < 2 ? x : cap - 1 - x);
+}
+
+// Whether a ring of G lanes can take the K blocks of a band in turn (k_sw_band): a lane
+// that takes block b (in forward order) at steps column + b has to be done with it one step
+// before the step at which block b + G, which it takes next, starts.
+__device__ __forceinline__ bool band_fits(const uint32_t *band, int K, int G) {
+    const int lane = threadIdx.x & 31;
+    bool ok = true;
+    for (int k = G + lane; k < K; k += 32)              // block k comes G blocks before block k - G
+        ok &= (int)(band[k] >> 16) - (int)(band[k - G] & 0xFFFFu) < G - 1;
+    return __all_sync(0xffffffffu, ok);
 }
 
 // Pass 2 over every pair pass 1 scored: one warp per pair, a few pairs per grab.
@@ -631,26 +700,29 @@ __global__ void __launch_bounds__(SW_THREADS, 5) k_sw_bound(const uint8_t *qcode
                                                          const pastis_cand *pairs, int64_t n_pairs,
                                                          const int8_t *gmat, int o, int e, const int16_t *bm_all,
                                                          const int64_t *bm_off, unsigned long long *next_pair,
-                                                         sw_score_out *res, int cov_cut, const int64_t *dn,
-                                                         const int *chk) {
+                                                         sw_score_out *res, int cov_cut, uint32_t *band_all,
+                                                         uint32_t *list, int64_t list_cap, int *n_band,
+                                                         const int64_t *dn, const int *chk) {
     if (dn) n_pairs = *dn;
     if (chk && (chk[0] | chk[1])) return;
     __shared__ int s_mat[PASTIS_NSYM * PASTIS_NSYM];
     for (int x = threadIdx.x; x < PASTIS_NSYM * PASTIS_NSYM; x += blockDim.x) s_mat[x] = gmat[x];
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    constexpr int GRAB = 8;
+    // eight pairs a grab, fewer when there are not enough for four grabs a warp
+    const int64_t warps = (int64_t)gridDim.x * SW_WARPS;
+    const int grab = (int)min((int64_t)8, max((int64_t)1, n_pairs / (4 * warps)));
     for (;;) {
         unsigned long long g = 0;
-        if (lane == 0) g = atomicAdd(next_pair, (unsigned long long)GRAB);
+        if (lane == 0) g = atomicAdd(next_pair, (unsigned long long)grab);
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g >= (unsigned long long)n_pairs) break;
-        // lane u < GRAB fetches pair g + u's pass-1 result, sequences and bounds, so the
+        // lane u < grab fetches pair g + u's pass-1 result, sequences and bounds, so the
         // grab's load chains run side by side instead of one after the other
-        int ok_l = 0, sc_l = 0, ei_l = 0, ej_l = 0;
+        int ok_l = 0, sc_l = 0, ei_l = 0, ej_l = 0, lq_l = 0, lt_l = 0;
         int64_t qo_l = 0, to_l = 0, bo_l = 0;
         const int64_t pl = (int64_t)g + lane;
-        if (lane < GRAB && pl < n_pairs) {
+        if (lane < grab && pl < n_pairs) {
             const sw_score_out r = res[pl];
             if (!r.big && r.score > 0) {
                 const pastis_cand c = pairs[pl];
@@ -658,28 +730,46 @@ __global__ void __launch_bounds__(SW_THREADS, 5) k_sw_bound(const uint8_t *qcode
                 to_l = toffsets[c.j];
                 bo_l = bm_off[pl];
                 sc_l = r.score; ei_l = r.end_i; ej_l = r.end_j;
-                ok_l = 1;
+                lq_l = (int)(qoffsets[c.i + 1] - qo_l);
+                lt_l = (int)(toffsets[c.j + 1] - to_l);
                 // the filter-only mode: a pair whose end already rules out coverage
-                if (cov_cut >= 0 &&
-                    cannot_cover(r, (int)(qoffsets[c.i + 1] - qo_l), (int)(toffsets[c.j + 1] - to_l), cov_cut))
-                    ok_l = 0;
+                ok_l = !(cov_cut >= 0 && cannot_cover(r, lq_l, lt_l, cov_cut));
             }
         }
-        for (int u = 0; u < GRAB; ++u) {
+        for (int u = 0; u < grab; ++u) {
             if (!__shfl_sync(0xffffffffu, ok_l, u)) continue;
             const int64_t p = (int64_t)g + u;
             const int score = __shfl_sync(0xffffffffu, sc_l, u);
             const int ei = __shfl_sync(0xffffffffu, ei_l, u), ej = __shfl_sync(0xffffffffu, ej_l, u);
             const uint8_t *qp = qcodes + __shfl_sync(0xffffffffu, qo_l, u);
             const uint8_t *tp = tcodes + __shfl_sync(0xffffffffu, to_l, u);
-            const int16_t *bm = bm_all + __shfl_sync(0xffffffffu, bo_l, u);
+            const int64_t bo = __shfl_sync(0xffffffffu, bo_l, u);
+            const int lq = __shfl_sync(0xffffffffu, lq_l, u), lt = __shfl_sync(0xffffffffu, lt_l, u);
+            const int16_t *bm = bm_all + bo;
+            uint32_t *band = band_all ? band_all + band_at(bo, p) : nullptr;
             int amax = 0, bmax = 0;
-            bool ok = o >= e && band_rows(qp, tp, s_mat, o, e, score, ei, ej, bm, &amax, &bmax);
+            bool ok = o >= e && band_rows(qp, tp, s_mat, o, e, score, ei, ej, bm, &amax, &bmax, band);
+            const bool banded = ok && band;
             if (!ok) ok = band_walk(qp, tp, s_mat, o, e, score, ei, ej, bm, &amax, &bmax);
-            if (ok && amax > 0 && bmax > 0 && lane == 0) {
-                res[p].rect_i = ei + 1 - amax;
-                res[p].rect_j = ej + 1 - bmax;
-            }                                      // else: the whole up-left rectangle (0, 0)
+            if (ok && amax > 0 && bmax > 0) {      // else: the whole up-left rectangle (0, 0)
+                sw_score_out r;
+                r.end_i = ei; r.end_j = ej; r.rect_i = ei + 1 - amax; r.rect_j = ej + 1 - bmax;
+                int ring = BAND_RINGS;             // the pair on a ring of 4 << ring lanes, if any
+                if (banded && amax > BAND_MIN_ROWS && !(cov_cut >= 0 && cannot_cover(r, lq, lt, cov_cut))) {
+                    __syncwarp();                  // lane 0 wrote the ranges
+                    const int K = (amax + 7) >> 3;
+                    ring = 0;
+                    while (ring < BAND_RINGS && !band_fits(band, K, 4 << ring)) ++ring;
+                }
+                if (lane == 0) {
+                    res[p].rect_i = r.rect_i;
+                    res[p].rect_j = r.rect_j;
+                    if (ring < BAND_RINGS) {
+                        res[p].big = 2;
+                        list[band_slot(ring, atomicAdd(&n_band[ring], 1), list_cap)] = (uint32_t)p;
+                    }
+                }
+            }
         }
     }
 }
@@ -1057,6 +1147,167 @@ __device__ void finish_record(pastis_aln &rec, int S, int ei, int ej, int qb, in
     if (filtered && !rec.passes) { rec.qb = rec.tb = 0; rec.ident = rec.cols = 0; }
 }
 
+// Pass 3 inside a band: the pairs whose path pass 2 bounded row by row, a pair on a ring of
+// G lanes.  The rows from the end upwards lie in blocks of 8; a lane takes blocks l, l + G,
+// ... of the K blocks in forward order, block b at column c in step c + b, only over the
+// columns pass 2 left it.  The row above a block comes by shuffle from the lane before it in
+// the ring, which did that column one step earlier.  Cells outside the band count as
+// zero cells a path may start after (no forward value is below zero, so no value inside
+// exceeds the true one), and the band holds the traced path, so along it the values and
+// choices are the traceback's.  What bounds it is instruction issue, 30 a cell; a band of
+// some 25 columns a row instead of the whole rectangle leaves a tenth of the cells of two
+// homologous proteins.  Pass 3 of the benchmark recipe at 5,000 proteins (1.18 M pairs, 97,000
+// traced) 35.6 ms over the rectangles, 4.2 ms so; of 10^5 pairs of 1,000 residues 33.3 ->
+// 3.5 ms; of 1,000 proteins (15,000 pairs, where the slowest warp counts) 9.1 -> 0.93 ms.
+
+struct band_args {
+    const uint8_t *qcodes;
+    const int64_t *qoffsets;
+    const uint8_t *tcodes;
+    const int64_t *toffsets;
+    const pastis_cand *pairs;
+    int o, e, ani, cov, filtered;
+    const uint32_t *band_all;
+    const int64_t *bm_off;
+    const uint32_t *list;
+    int64_t list_cap;
+    const int *n_list;
+    int *next;
+    const sw_score_out *res;
+    pastis_aln *out;
+    int *err;
+};
+
+template <int G>
+__device__ __noinline__ void band_ring(const band_args &g, const int *s_mat) {
+    const int o = g.o, e = g.e;
+    const int lane = threadIdx.x & 31, lg = lane & (G - 1), from = (lane & ~(G - 1)) | ((lane + G - 1) & (G - 1));
+    constexpr int RING = G == 4 ? 0 : (G == 8 ? 1 : (G == 16 ? 2 : 3));
+    const int cnt = g.n_list[RING];
+    int *const next = g.next + RING;
+    // the group's pair
+    bool busy = false, done = false;
+    int64_t p = 0;
+    const uint8_t *q = g.qcodes, *t = g.tcodes;
+    const uint32_t *band = g.band_all;
+    int K = 0, top = 0, ei = 0, ej = 0, rj = 0, step = 0;
+    // the lane's block: rows row0 .. row0 + 7, columns lo .. hi; plo .. phi those of the block above
+    int b = 0, row0 = 0, lo = 1, hi = 0, plo = 1, phi = 0;
+    int qoff[8], Hc[8], Ec[8];
+    uint32_t HB[8], EB[8], HM[8], EM[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) { qoff[r] = 0; Hc[r] = 0; Ec[r] = NEG; HB[r] = EB[r] = HM[r] = EM[r] = 0u; }
+    int dh = 0, out_h = 0, out_f = NEG;
+    uint32_t db = 0u, dm = 0u, out_hb = 0u, out_fb = 0u, out_hm = 0u, out_fm = 0u;
+    auto open_block = [&]() {
+        if (b >= K) { lo = 1; hi = 0; return; }
+        const uint32_t own = band[K - 1 - b], above = b > 0 ? band[K - b] : 1u;
+        lo = max((int)(own & 0xFFFFu), rj); hi = (int)(own >> 16);
+        plo = max((int)(above & 0xFFFFu), b > 0 ? rj : 1); phi = (int)(above >> 16);
+        row0 = top + 8 * b;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            qoff[r] = (row0 + r >= 0 ? (int)q[row0 + r] : PASTIS_NSYM) * 32;
+            Hc[r] = 0; Ec[r] = NEG;
+            HB[r] = pack_rc(row0 + r + 1, lo); EB[r] = 0u; HM[r] = 0u; EM[r] = 0u;
+        }
+    };
+    for (;;) {
+        if (__any_sync(0xffffffffu, !busy && !done)) {
+            int slot = 0;
+            if (!busy && !done && lg == 0) slot = atomicAdd(next, 1);
+            slot = __shfl_sync(0xffffffffu, slot, lane & ~(G - 1));
+            int t0 = 0x7FFFFFFF;
+            const bool take = !busy && !done && slot < cnt;
+            if (!busy && !done && slot >= cnt) done = true;
+            if (take) {
+                p = g.list[band_slot(RING, slot, g.list_cap)];
+                const pastis_cand c = g.pairs[p];
+                const sw_score_out r = g.res[p];
+                q = g.qcodes + g.qoffsets[c.i];
+                t = g.tcodes + g.toffsets[c.j];
+                band = g.band_all + band_at(g.bm_off[p], p);
+                ei = r.end_i; ej = r.end_j; rj = r.rect_j;
+                K = (ei + 1 - r.rect_i + 7) >> 3;
+                top = ei + 1 - 8 * K;
+                b = lg;
+                open_block();
+                busy = true;
+                if (b < K) t0 = lo + b - 1;
+            }
+#pragma unroll
+            for (int d = G >> 1; d > 0; d >>= 1) t0 = min(t0, __shfl_xor_sync(0xffffffffu, t0, d));
+            if (take) step = t0;
+            if (__all_sync(0xffffffffu, done)) break;
+        }
+        // the row above at this lane's column, from the lane before it in the ring
+        int up_h = __shfl_sync(0xffffffffu, out_h, from), up_f = __shfl_sync(0xffffffffu, out_f, from);
+        uint32_t up_hb = __shfl_sync(0xffffffffu, out_hb, from), up_fb = __shfl_sync(0xffffffffu, out_fb, from);
+        uint32_t up_hm = __shfl_sync(0xffffffffu, out_hm, from), up_fm = __shfl_sync(0xffffffffu, out_fm, from);
+        const int c = step - b;
+        if (c < plo || c > phi) { up_h = 0; up_f = NEG; up_hb = pack_rc(row0, c + 1); up_fb = 0u; up_hm = 0u; up_fm = 0u; }
+        if (busy && c >= lo && c <= hi) {
+            const int tj = t[c];
+            int ph = dh, ah = up_h, f = up_f;
+            uint32_t pb = db, pm = dm, ab = up_hb, am = up_hm, fb = up_fb, fm = up_fm;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const int eo = Hc[r] - o, ex = Ec[r] - e;
+                const bool eop = eo >= ex;
+                const int ev = eop ? eo : ex;
+                const uint32_t evb = eop ? HB[r] : EB[r], evm = eop ? HM[r] : EM[r];
+                const int fo = ah - o, fx = f - e;
+                const bool fop = fo >= fx;
+                f = fop ? fo : fx;
+                fb = fop ? ab : fb;
+                fm = fop ? am : fm;
+                int h = ph + s_mat[qoff[r] + tj];
+                uint32_t hb = pb, hm = pm + ((qoff[r] == tj * 32) ? 0x10001u : 1u);
+                if (f > h) { h = f; hb = fb; hm = fm; }
+                if (ev > h) { h = ev; hb = evb; hm = evm; }
+                if (h <= 0) { h = 0; hb = pack_rc(row0 + r + 1, c + 1); hm = 0u; }
+                ph = Hc[r]; pb = HB[r]; pm = HM[r];
+                Hc[r] = h; HB[r] = hb; HM[r] = hm;
+                Ec[r] = ev; EB[r] = evb; EM[r] = evm;
+                ah = h; ab = hb; am = hm;
+            }
+            out_h = ah; out_f = f; out_hb = ab; out_fb = fb; out_hm = am; out_fm = fm;
+            if (b == K - 1 && c == ej) {           // the end: the last row of the last block
+                const sw_score_out r1 = g.res[p];
+                const pastis_cand cd = g.pairs[p];
+                const int lq = (int)(g.qoffsets[cd.i + 1] - g.qoffsets[cd.i]);
+                const int lt = (int)(g.toffsets[cd.j + 1] - g.toffsets[cd.j]);
+                if (Hc[7] != r1.score) atomicExch(g.err, 1);
+                pastis_aln rec;
+                rec.seed_used = 0; rec.passes = 0; rec.reserved = 0;
+                finish_record(rec, r1.score, ei, ej, (int)(HB[7] >> 16), (int)(HB[7] & 0xFFFFu), (int)(HM[7] >> 16),
+                              (int)(HM[7] & 0xFFFFu), lq, lt, g.ani, g.cov, g.filtered);
+                g.out[p] = rec;
+            }
+            if (c == hi) { b += G; open_block(); }
+        }
+        dh = up_h; db = up_hb; dm = up_hm;
+        if (busy && step == ej + K - 1) busy = false;   // the same step for the whole group
+        ++step;
+    }
+}
+
+// The widest bands, of which there are few, first; a warp that finds a list empty goes on
+// to the next, so the lists' last pairs run beside the next list's.
+__global__ void __launch_bounds__(SW_THREADS, 2) k_sw_band(band_args g, const int8_t *gmat, const int *chk) {
+    if (chk && (chk[0] | chk[1])) return;
+    __shared__ int s_mat[(PASTIS_NSYM + 1) * 32];
+    for (int x = threadIdx.x; x < (PASTIS_NSYM + 1) * 32; x += blockDim.x) {
+        const int a = x / 32, b = x % 32;
+        s_mat[x] = (a < PASTIS_NSYM && b < PASTIS_NSYM) ? (int)gmat[a * PASTIS_NSYM + b] : PAD_SCORE;
+    }
+    __syncthreads();
+    band_ring<32>(g, s_mat);
+    band_ring<16>(g, s_mat);
+    band_ring<8>(g, s_mat);
+    band_ring<4>(g, s_mat);
+}
+
 __global__ void __launch_bounds__(SW_THREADS) k_sw_carry(const uint8_t *qcodes, const int64_t *qoffsets,
                                                          const uint8_t *tcodes, const int64_t *toffsets,
                                                          const pastis_cand *pairs, int64_t n_pairs,
@@ -1122,6 +1373,7 @@ __global__ void __launch_bounds__(SW_THREADS) k_sw_carry(const uint8_t *qcodes, 
             const int64_t p = p0 + k;
             if (p >= n_pairs) break;
             const sw_score_out r1 = res[p];
+            if (r1.big == 2) continue;             // k_sw_band's
             const pastis_cand c = pairs[p];
             const int64_t qo = qoffsets[c.i], to = toffsets[c.j];
             const int lq = (int)(qoffsets[c.i + 1] - qo), lt = (int)(toffsets[c.j + 1] - to);
@@ -1240,6 +1492,17 @@ pastis_status sw_align(pastis_ctx *ctx, const uint8_t *d_qcodes, const int64_t *
     }
     int16_t *bm_all;
     PASTIS_WS(bm_all, ctx, WS_ALN_BOUND, sizeof(int16_t) * (size_t)h_bm + 16);
+    // pass 2's column ranges per 8 rows; without room for them pass 3 takes the rectangles
+    uint32_t *band = nullptr;
+    if (p->mode != PASTIS_SW_SCORE) {
+        const size_t bytes = sizeof(uint32_t) * ((size_t)(h_bm >> 2) + (size_t)n_pairs + 2);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (dn) PASTIS_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+        // a capture allocates nothing: what its sizing run could not have, it goes without
+        if (cap == cudaStreamCaptureStatusNone || ctx->ws_bytes[WS_ALN_BAND] >= bytes)
+            band = (uint32_t *)ws_get(ctx, WS_ALN_BAND, bytes);
+    }
+    uint32_t *list = (uint32_t *)bm_cnt;       // the counts have served: two lists of pairs
 
     sw_score_out *res;
     PASTIS_WS(res, ctx, WS_ALN_PASS1, sizeof(sw_score_out) * (size_t)n_pairs);
@@ -1282,11 +1545,19 @@ pastis_status sw_align(pastis_ctx *ctx, const uint8_t *d_qcodes, const int64_t *
         k_sw_bound<<<ctx->sm_count * per_sm2, SW_THREADS, 0, st>>>(d_qcodes, d_qoffsets, d_tcodes, d_toffsets,
                                                                    d_pairs, n_pairs, dmat, p->gap_open, p->gap_extend,
                                                                    bm_all, bm_off, (unsigned long long *)(flags + 10),
-                                                                   res, filtered ? p->cov_min_pct : -1, dn, chk);
+                                                                   res, filtered ? p->cov_min_pct : -1, band, list,
+                                                                   n_pairs, flags + 20, dn, chk);
         PASTIS_LAUNCHED(ctx);
         prof_end(ctx);
     }
     prof_begin(ctx, "sw_pass3");
+    if (band) {
+        const band_args g{d_qcodes, d_qoffsets, d_tcodes, d_toffsets, d_pairs, p->gap_open, p->gap_extend,
+                          p->ani_min_pct, p->cov_min_pct, filtered, band, bm_off, list, n_pairs, flags + 20,
+                          flags + 24, res, d_out, flags};
+        k_sw_band<<<ctx->sm_count * 2, SW_THREADS, 0, st>>>(g, dmat, chk);
+        PASTIS_LAUNCHED(ctx);
+    }
     k_sw_carry<<<blocks3, SW_THREADS, 0, st>>>(d_qcodes, d_qoffsets, d_tcodes, d_toffsets, d_pairs, n_pairs, dmat,
                                                p->gap_open,
                                                p->gap_extend, p->ani_min_pct, p->cov_min_pct,

@@ -68,3 +68,33 @@ def test_tied_scores(o, e, extra):
     ps = synth.from_strings(_seqs(lengths, "AG", 10 * o + extra))
     i, j = np.triu_indices(len(lengths), 1)
     _check(ps, _cands(i, j), 0, layout=np.full(64, extra, np.uint8), gap_open=o, gap_extend=e)
+
+
+@pytest.mark.parametrize("gap", [0, 1, 3, 6, 7, 8, 20, 31, 33, 45, 62, 66, 90, 130, 200])
+@pytest.mark.parametrize("o,e", [(11, 1), (5, 2), (12, 0)])
+def test_bands_of_gapped_homologs(gap, o, e):
+    """Relatives with one long gap on either side (narrow to very wide bands of the reverse
+    pass, every ring of the banded third pass and its fall-backs), at 5% to 60%
+    substitutions, paths of a few to 700 rows that start and end anywhere."""
+    rng = np.random.default_rng(1000 * gap + 10 * o + e)
+    letters = np.array(list("ACDEFGHIKLMNPQRSTVWY"))
+    strings = []
+    for n in (23, 24, 25, 33, 64, 150, 400, 700):
+        base = rng.choice(letters, size=n)
+        strings.append("".join(base))
+        for p_sub in (0.05, 0.3, 0.6):
+            x = base.copy()
+            hit = rng.random(n) < p_sub
+            x[hit] = rng.choice(letters, size=int(hit.sum()))
+            cut = int(rng.integers(0, n + 1))
+            x = np.concatenate([x[:cut], rng.choice(letters, size=gap), x[cut:]])
+            flank = rng.choice(letters, size=int(rng.integers(0, 60)))
+            strings.append("".join(np.concatenate([flank, x])))
+    ps = synth.from_strings(strings)
+    i = np.repeat(np.arange(0, 32, 4), 3)
+    j = i + np.tile([1, 2, 3], 8)
+    far = [(a, b) for a in range(0, 32, 4) for b in range(a + 4, 32, 9)]
+    ii = np.concatenate([i, j, [a for a, _ in far]])
+    jj = np.concatenate([j, i, [b for _, b in far]])
+    _check(ps, _cands(ii, jj), 0, gap_open=o, gap_extend=e)
+    _check(ps, _cands(ii, jj), 3, gap_open=o, gap_extend=e)

@@ -314,17 +314,21 @@ __device__ bool xd_diag_warp(const uint8_t *q, int A, int qs, const uint8_t *t, 
 // which every lane of the warp has its own copy in its own shared-memory bank.  Per
 // register and antidiagonal the recurrence is the packed one of the Smith-Waterman
 // pass 1 without the floor at 0: E and F as __viaddmax_s16x2, the diagonal as
-// __vadd2, H as __vimax3_s16x2.  The x-drop test (H >= best - X) and the computed range
-// [clo, chi] become a per-half mask by clamps alone: min(max(H, lim - 1), lim) - lim
-// is -1 exactly where H < lim, min(row - clo, chi - row) is negative exactly outside
-// the range, and the mask selects the dead value.
+// __vadd2, H as __vimax3_s16x2 and kept less the gap open, which is what E and F take.
+// The x-drop test (H >= best - X) and the computed range [clo, chi] become one per-half
+// mask: row - clo, chi - row and max(H, lim - 1) - lim are negative exactly outside the
+// range and where H < lim, and the sign of the smallest, replicated over its half,
+// selects the dead value.
 //
-// Dead cells hold XD16_NEG in H, E and F.  Live values lie in [best - X - o - e, best
-// + the largest substitution score], values derived from dead ones in [XD16_NEG - o -
-// e, XD16_NEG + 63], and every one of them is pruned (XD16_NEG + 63 < -X), so no sum
-// wraps when X, the best score and o + e stay within the bounds checked below; an
-// extension outside them, or whose computed range outgrows the window, is listed for
-// the 32-bit kernel, which computes it from the start.
+// Dead cells hold XD16_NEG in H.  Their E and F stay as they are: both lie below lim, which
+// never falls, and a gap that goes on from them only loses, so they can neither win nor
+// tie a live cell; past a sequence's end, where they may be higher, no cell of the range
+// takes them.  Live values lie in [best - X - o - e, best + the largest substitution
+// score], values derived from dead ones in [XD16_NEG - o - e, XD16_NEG + 63 + o], and every
+// one of them is pruned (XD16_NEG + 63 + o < -X), so no sum wraps when X, the best score
+// and o + e stay within the bounds checked below; an extension outside them, or whose
+// computed range outgrows the window, is listed for the 32-bit kernel, which computes it
+// from the start.
 //
 // Every lane runs every step, an odd antidiagonal and an even one per turn of one
 // loop, so the segments' parities agree and the packed sources need no per-segment
@@ -333,20 +337,27 @@ __device__ bool xd_diag_warp(const uint8_t *q, int A, int qs, const uint8_t *t, 
 // found once per extension: the step that raises the best score keeps a copy of its
 // H registers, and the first row holding the best is read from that copy at the end.
 //
-// The carried statistics (identities and aligned columns along the path a traceback
-// from the cell would take, Sec. IV-E) are one 32-bit word per cell beside H, E and F,
-// for both parities.  A cell's words follow its winning predecessor: E and F take H's
-// (gap open) unless the extension wins outright, H takes the diagonal's plus one
-// column (and one identity when the residues match) unless F, then E, is strictly
-// larger.  Which candidate won is read off the packed results: a half of max(x, y)
-// equals x's exactly when x won or tied.  The score table then holds each score's byte
-// and the match bit (q == t) above it; the scores are sign-extended from the bytes.
+// The carried statistics (aligned columns and identities along the path a traceback from
+// the cell would take, Sec. IV-E) are 16-bit halves like the scores, a register of each
+// beside every register of H, E and F, for both parities.  They follow a cell's winning
+// predecessor: E and F take H's (gap open) unless the extension wins outright, H takes the
+// diagonal's plus one column (and one identity when the residues match) unless F, then
+// E, is strictly larger.  Which candidate won is read off the packed results: a half of
+// max(x, y) less x is zero exactly when x won or tied, and the mask of the zero halves
+// selects both cells' carries at once.  The score table then holds each score's byte and
+// the match bit (q == t) above it; the scores are sign-extended from the bytes.
+//
+// What bounds both forms is the integer pipe (ncu: 85% busy, 3.0 instructions a cycle).
+// Measured on 2 M exact candidates of 200,000 proteins: first phase 63.8 ms with separate
+// range and limit masks, dead E and F cleared, and the best score reduced in every step,
+// 53.1 ms so; second phase 14.5 ms with one 32-bit word of statistics per cell, 11.9 ms so;
+// 300,000 family-rich pairs with carries throughout 25.8 -> 20.6 ms.
 // ---------------------------------------------------------------------------------
 constexpr int XD16_NEG = -32512;                 // 0x8100
 constexpr uint32_t XD16_NEG2 = (uint32_t)(XD16_NEG & 0xffff) * 0x10001u;   // 0x81008100
 constexpr int XD16_LIM = 30000;                  // bound on X and on an extension's best score
 // Score table, int16: byte offset q * 1536 + (t >> 1) * 128 + (t & 1) * 2 + 4 * lane holds
-// s(q, t) (with carries: the byte of s(q, t), then [q == t]) for every lane, so lane L
+// s(q, t) + o (with carries: the byte of s(q, t), then [q == t]) for every lane, so lane L
 // always reads bank L.
 constexpr int XD16_TAB = PASTIS_NSYM * PASTIS_NSYM * 32;   // entries
 constexpr uint32_t XD16_QOFF = PASTIS_NSYM / 2 * 128;      // bytes per query residue
@@ -364,6 +375,18 @@ __device__ __forceinline__ uint32_t xd16_sext_lo_bytes(uint32_t a, uint32_t b) {
     return r;
 }
 
+// Each half's sign bit over the half (prmt with the sign-replicate bit of its selector).
+__device__ __forceinline__ uint32_t xd16_signs(uint32_t a) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %1, 0xBB99;" : "=r"(r) : "r"(a));
+    return r;
+}
+
+// Halves that are zero: 0xffff where v's half is, else 0.
+__device__ __forceinline__ uint32_t xd16_zeros(uint32_t v) {
+    return __vsub2(__vminu2(v, 0x00010001u), 0x00010001u);
+}
+
 // Live bits of four cells in row order from the dead masks of two registers (halves of
 // 0xffff or 0): the high byte of each half, gathered in row order, then its top bit
 // moved to bit j by one multiply (the partial products below bit 28 never carry into it).
@@ -377,13 +400,13 @@ struct xd16_ext {
     uint32_t H[2][R], E[2][R], F[2][R];          // [parity of the diagonals][register]
     uint32_t QW[R], TW[R];                       // cells 2r (low half), 2r + 1: table offsets of q and t
     uint32_t HS[R];                              // H of the antidiagonal sd that last raised best
-    // C: the carried statistics (identities << 16 | columns) of H, E and F, one word per
-    // cell [parity][register][half], and those of HS
-    uint32_t HC[2][C ? R : 1][2], EC[2][C ? R : 1][2], FC[2][C ? R : 1][2], HSC[C ? R : 1][2];
+    // C: the carried columns ([0]) and identities ([1]) of H, E and F, in halves like them,
+    // and those of HS
+    uint32_t HC[2][2][C ? R : 1], EC[2][2][C ? R : 1], FC[2][2][C ? R : 1], HSC[2][C ? R : 1];
     const uint8_t *q, *t;
     int st, A, B;                                // A = B = 0 while the segment has no extension
     int d, best, sd, sa0, llo, lhi, kbase;
-    long long cells;
+    int cells;                                   // at most 64 per antidiagonal
     int64_t task;
     bool active;
 };
@@ -420,13 +443,16 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
     constexpr int G = 32 / R, WD = 4 * R, NC = 2 * R;
     constexpr int P = PAR, Q = 1 - PAR;
     const int d = x.d + 1;
-    const int clo = max(max(x.llo, d - x.B), 0);
-    const int chi = min(min(x.lhi + 1, x.A), d);
-    const bool empty = clo > chi;                        // the extension ended (d > A + B included)
-    bool defer = !empty && chi - clo + 1 > G * NC;
-    // the computed range's diagonals, with their E and F predecessors, inside the window
-    const int kmin = 2 * clo - d - 1, kmax = 2 * chi - d + 1;
-    const bool move = !empty && !defer && (kmin < x.kbase || kmax > x.kbase + 127);
+    // the computed range (rows 0 and d bound it by themselves); empty when the extension has
+    // ended, and then every cell below is dead
+    const int clo = max(x.llo, d - x.B);
+    const int chi = min(x.lhi + 1, x.A);
+    bool defer = false;
+    // its diagonals, with their E and F predecessors, inside the window; looked at on odd
+    // antidiagonals with one more diagonal a side, which is as far as the next one's range
+    // can reach
+    const int kmin = 2 * clo - d - 2, kmax = 2 * chi - d + 2;
+    const bool move = P == 1 && clo <= chi && (kmin < x.kbase || kmax > x.kbase + 127);
     int a0 = (d + x.kbase + WD * ls + P) >> 1;          // this lane's first row on d
     if (P == 1) {        // rows moved on by one: a new last query residue
 #pragma unroll
@@ -437,7 +463,7 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
         for (int r = R - 1; r >= 0; --r)
             x.TW[r] = __byte_perm(r == 0 ? xd16_toff(x, d - a0 - 1, lane4) << 16 : x.TW[r - 1], x.TW[r], 0x5432);
     }
-    if (__any_sync(0xffffffffu, move)) {
+    if (P == 1 && __any_sync(0xffffffffu, move)) {
         if (move) {
             const int sh = ((kmin + kmax) / 2 - (x.kbase + 64)) / WD;      // whole lanes, centring the range
             x.kbase += WD * sh;
@@ -458,13 +484,13 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
                         x.F[p][r] = in ? ff : XD16_NEG2;
                         if constexpr (C) {
 #pragma unroll
-                            for (int hf = 0; hf < 2; ++hf) {
-                                const uint32_t hc = __shfl_sync(smask, x.HC[p][r][hf], src & (G - 1), G);
-                                const uint32_t ec = __shfl_sync(smask, x.EC[p][r][hf], src & (G - 1), G);
-                                const uint32_t fc = __shfl_sync(smask, x.FC[p][r][hf], src & (G - 1), G);
-                                x.HC[p][r][hf] = in ? hc : 0u;
-                                x.EC[p][r][hf] = in ? ec : 0u;
-                                x.FC[p][r][hf] = in ? fc : 0u;
+                            for (int w = 0; w < 2; ++w) {
+                                const uint32_t hc = __shfl_sync(smask, x.HC[w][p][r], src & (G - 1), G);
+                                const uint32_t ec = __shfl_sync(smask, x.EC[w][p][r], src & (G - 1), G);
+                                const uint32_t fc = __shfl_sync(smask, x.FC[w][p][r], src & (G - 1), G);
+                                x.HC[w][p][r] = in ? hc : 0u;
+                                x.EC[w][p][r] = in ? ec : 0u;
+                                x.FC[w][p][r] = in ? fc : 0u;
                             }
                         }
                     }
@@ -475,23 +501,24 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
     }
     const int lim = x.best - X;
     const uint32_t lim2 = xd16_pk(lim), limm2 = __vsub2(lim2, 0x00010001u);
-    const uint32_t span2 = xd16_pk(chi - clo), rb2 = xd16_pk(a0 - clo);
+    const uint32_t rb2 = xd16_pk(a0 - clo), span2 = xd16_pk(chi - clo);
     // the sources on d - 1 that cross a lane boundary
     uint32_t bh, bx, bhc = 0u, bxc = 0u;
     if (P == 0) {        // F of the first cell: the previous lane's last odd diagonal
         bh = __shfl_up_sync(0xffffffffu, x.H[Q][R - 1], 1, G);
         bx = __shfl_up_sync(0xffffffffu, x.F[Q][R - 1], 1, G);
         if constexpr (C) {
-            bhc = __shfl_up_sync(0xffffffffu, x.HC[Q][R - 1][1], 1, G);
-            bxc = __shfl_up_sync(0xffffffffu, x.FC[Q][R - 1][1], 1, G);
+            // columns and identities of the cell in one word
+            bhc = __shfl_up_sync(0xffffffffu, __byte_perm(x.HC[0][Q][R - 1], x.HC[1][Q][R - 1], 0x7632), 1, G);
+            bxc = __shfl_up_sync(0xffffffffu, __byte_perm(x.FC[0][Q][R - 1], x.FC[1][Q][R - 1], 0x7632), 1, G);
         }
         if (ls == 0) { bh = XD16_NEG2; bx = XD16_NEG2; }
     } else {             // E of the last cell: the next lane's first even diagonal
         bh = __shfl_down_sync(0xffffffffu, x.H[Q][0], 1, G);
         bx = __shfl_down_sync(0xffffffffu, x.E[Q][0], 1, G);
         if constexpr (C) {
-            bhc = __shfl_down_sync(0xffffffffu, x.HC[Q][0][0], 1, G);
-            bxc = __shfl_down_sync(0xffffffffu, x.EC[Q][0][0], 1, G);
+            bhc = __shfl_down_sync(0xffffffffu, __byte_perm(x.HC[0][Q][0], x.HC[1][Q][0], 0x5410), 1, G);
+            bxc = __shfl_down_sync(0xffffffffu, __byte_perm(x.EC[0][Q][0], x.EC[1][Q][0], 0x5410), 1, G);
         }
         if (ls == G - 1) { bh = XD16_NEG2; bx = XD16_NEG2; }
     }
@@ -509,52 +536,61 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
             eh = __byte_perm(x.H[Q][r], r == R - 1 ? bh : x.H[Q][r + 1], 0x5432);
             ex = __byte_perm(x.E[Q][r], r == R - 1 ? bx : x.E[Q][r + 1], 0x5432);
         }
-        const uint32_t eo = __vsub2(eh, o2), fo = __vsub2(fh, o2);
+        const uint32_t eo = eh, fo = fh;                  // H is kept less the gap open
         const uint32_t en = __viaddmax_s16x2(ex, ne2, eo);
         const uint32_t fn = __viaddmax_s16x2(fx, ne2, fo);
         // substitution scores of rows a0 + 2r and a0 + 2r + 1 from this lane's table column
         const uint32_t ix = x.QW[r] + x.TW[r];
         const uint32_t s0 = *(const uint16_t *)(tab + (ix & 0xffffu));
         const uint32_t s1 = *(const uint16_t *)(tab + (ix >> 16));
-        // with carries an entry is the score's byte, then [q == t]: the scores sign-extended
-        const uint32_t dg = __vadd2(x.H[P][r], C ? xd16_sext_lo_bytes(s0, s1) : __byte_perm(s0, s1, 0x5410));
+        // with carries an entry is the score's byte, then [q == t]: the scores sign-extended;
+        // without, it is the score plus the gap open
+        const uint32_t dg = C ? __vadd2(__vadd2(x.H[P][r], o2), xd16_sext_lo_bytes(s0, s1))
+                              : __vadd2(x.H[P][r], __byte_perm(s0, s1, 0x5410));
         const uint32_t hn = __vimax3_s16x2(dg, en, fn);
         if constexpr (C) {
             // each cell's carries along the predecessor a traceback takes: E and F from H
             // (the gap opens) on ties, H from the diagonal, then from F, then from E; a
             // packed result equals the candidate it came from
-            const uint32_t xe = en ^ eo, xf = fn ^ fo, xdg = dg ^ hn, xfh = fn ^ hn;
+            const uint32_t me = xd16_zeros(__vsub2(en, eo)), mf = xd16_zeros(__vsub2(fn, fo));
+            const uint32_t md = xd16_zeros(__vsub2(hn, dg)), mh = xd16_zeros(__vsub2(hn, fn));
+            auto pick = [](uint32_t m, uint32_t u, uint32_t v) { return (u & m) | (v & ~m); };
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                auto zero = [hf](uint32_t v) { return hf ? (v >> 16) == 0u : (v & 0xffffu) == 0u; };
+            for (int w = 0; w < 2; ++w) {
                 uint32_t ehc, exc, fhc, fxc;
-                if (P == 0) {
-                    ehc = x.HC[Q][r][hf]; exc = x.EC[Q][r][hf];
-                    fhc = hf ? x.HC[Q][r][0] : (r == 0 ? bhc : x.HC[Q][r > 0 ? r - 1 : 0][1]);
-                    fxc = hf ? x.FC[Q][r][0] : (r == 0 ? bxc : x.FC[Q][r > 0 ? r - 1 : 0][1]);
+                if (P == 0) {        // the previous lane's word holds columns, then identities
+                    ehc = x.HC[w][Q][r]; exc = x.EC[w][Q][r];
+                    fhc = r == 0 ? __byte_perm(bhc, x.HC[w][Q][0], w ? 0x5432 : 0x5410)
+                                 : __byte_perm(x.HC[w][Q][r > 0 ? r - 1 : 0], x.HC[w][Q][r], 0x5432);
+                    fxc = r == 0 ? __byte_perm(bxc, x.FC[w][Q][0], w ? 0x5432 : 0x5410)
+                                 : __byte_perm(x.FC[w][Q][r > 0 ? r - 1 : 0], x.FC[w][Q][r], 0x5432);
                 } else {
-                    fhc = x.HC[Q][r][hf]; fxc = x.FC[Q][r][hf];
-                    ehc = hf ? (r == R - 1 ? bhc : x.HC[Q][r < R - 1 ? r + 1 : 0][0]) : x.HC[Q][r][1];
-                    exc = hf ? (r == R - 1 ? bxc : x.EC[Q][r < R - 1 ? r + 1 : 0][0]) : x.EC[Q][r][1];
+                    fhc = x.HC[w][Q][r]; fxc = x.FC[w][Q][r];
+                    ehc = r == R - 1 ? __byte_perm(x.HC[w][Q][R - 1], bhc, w ? 0x7632 : 0x5432)
+                                     : __byte_perm(x.HC[w][Q][r], x.HC[w][Q][r < R - 1 ? r + 1 : 0], 0x5432);
+                    exc = r == R - 1 ? __byte_perm(x.EC[w][Q][R - 1], bxc, w ? 0x7632 : 0x5432)
+                                     : __byte_perm(x.EC[w][Q][r], x.EC[w][Q][r < R - 1 ? r + 1 : 0], 0x5432);
                 }
-                const uint32_t evc = zero(xe) ? ehc : exc;
-                const uint32_t fvc = zero(xf) ? fhc : fxc;
-                const uint32_t dvc = x.HC[P][r][hf] + 1u + (((hf ? s1 : s0) >> 8) << 16);
-                x.HC[P][r][hf] = zero(xdg) ? dvc : (zero(xfh) ? fvc : evc);
-                x.EC[P][r][hf] = evc;
-                x.FC[P][r][hf] = fvc;
+                const uint32_t evc = pick(me, ehc, exc), fvc = pick(mf, fhc, fxc);
+                const uint32_t dvc = __vadd2(x.HC[w][P][r], w ? __byte_perm(s0, s1, 0x6521) : 0x00010001u);
+                x.HC[w][P][r] = pick(md, dvc, pick(mh, fvc, evc));
+                x.EC[w][P][r] = evc;
+                x.FC[w][P][r] = fvc;
             }
         }
-        // dead halves: H < lim, or the row outside [clo, chi]
+        // dead halves: H < lim, or the row outside [clo, chi]; the sign of the smallest of
+        // row - clo, chi - row and max(H, lim - 1) - lim, replicated
         const uint32_t rr = __vadd2(rb2, (uint32_t)((2 * r) | ((2 * r + 1) << 16)));
-        const uint32_t w = __vmins2(rr, __vsub2(span2, rr));
-        const uint32_t d1 = __vsub2(__vmins2(__vmaxs2(hn, limm2), lim2), lim2);
-        const uint32_t dm = __vmins2(d1, __vmaxs2(w, 0xffffffffu));
-        x.H[P][r] = (hn & ~dm) | (XD16_NEG2 & dm);
-        x.E[P][r] = (en & ~dm) | (XD16_NEG2 & dm);
-        x.F[P][r] = (fn & ~dm) | (XD16_NEG2 & dm);
+        // (chi - row from row - clo by a subtraction of registers: from chi - a0 less a constant,
+        // this compiler left rows past chi alive with two extensions a warp)
+        const uint32_t rs = __vsub2(span2, rr);
+        const uint32_t dm = xd16_signs(__vimin3_s16x2(rr, rs, __vsub2(__vmaxs2(hn, limm2), lim2)));
+        x.H[P][r] = (__vsub2(hn, o2) & ~dm) | (XD16_NEG2 & dm);
+        x.E[P][r] = en;
+        x.F[P][r] = fn;
         dmk[r] = dm;
-        hmax = __vmaxs2(hmax, x.H[P][r]);
+        if (r & 1) hmax = __vimax3_s16x2(hmax, x.H[P][r - 1], x.H[P][r]);
+        else if (r + 1 == R) hmax = __vmaxs2(hmax, x.H[P][r]);
     }
     // live cells of this lane, bit j = row a0 + j
     uint32_t lb;
@@ -562,35 +598,39 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
         const uint32_t y = ~dmk[0] & 0x80008000u;
         lb = ((y >> 15) & 1u) | (y >> 30);
     } else {
-        lb = xd16_live4(dmk[0], dmk[R > 1 ? 1 : 0]);
-        if (R == 4) lb |= xd16_live4(dmk[R > 2 ? 2 : 0], dmk[R > 3 ? 3 : 0]) << 4;
+        lb = 0u;
+#pragma unroll
+        for (int r = 0; r + 1 < R; r += 2) lb |= xd16_live4(dmk[r], dmk[r + 1]) << (2 * r);
     }
-    x.cells += empty ? 0 : chi - clo + 1;
+    x.cells += max(chi - clo + 1, 0);
     x.d = d;
     const unsigned bal = (__ballot_sync(0xffffffffu, lb != 0u) >> sbase) & (G == 32 ? 0xffffffffu : ((1u << G) - 1u));
-    const int myh = max((int)(short)(hmax & 0xffffu), (int)hmax >> 16);
-    // the segment's maximum by a butterfly of full-warp shuffles (a reduction with a
-    // per-segment member mask runs once per distinct mask)
-    int toph = myh;
+    // a new best score: the segment's maximum by a butterfly of full-warp shuffles (a
+    // reduction with a per-segment member mask runs once per distinct mask), in the steps in
+    // which some lane of the warp exceeds its segment's best (5% faster)
+    const uint32_t best2 = xd16_pk(x.best - (int)(o2 & 0xffffu));
+    if (__any_sync(0xffffffffu, __vmaxs2(hmax, best2) != best2)) {
+        int toph = max((int)(short)(hmax & 0xffffu), (int)hmax >> 16) + (int)(o2 & 0xffffu);
 #pragma unroll
-    for (int m = G / 2; m > 0; m >>= 1) toph = max(toph, __shfl_xor_sync(0xffffffffu, toph, m, G));
-    const bool raise = !empty && !defer && toph > x.best;
+        for (int m = G / 2; m > 0; m >>= 1) toph = max(toph, __shfl_xor_sync(0xffffffffu, toph, m, G));
+        const bool raise = !defer && toph > x.best;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        x.HS[r] = raise ? x.H[P][r] : x.HS[r];
-        if constexpr (C) {
-            x.HSC[r][0] = raise ? x.HC[P][r][0] : x.HSC[r][0];
-            x.HSC[r][1] = raise ? x.HC[P][r][1] : x.HSC[r][1];
+        for (int r = 0; r < R; ++r) {
+            x.HS[r] = raise ? x.H[P][r] : x.HS[r];
+            if constexpr (C) {
+                x.HSC[0][r] = raise ? x.HC[0][P][r] : x.HSC[0][r];
+                x.HSC[1][r] = raise ? x.HC[1][P][r] : x.HSC[1][r];
+            }
         }
+        x.sa0 = raise ? a0 : x.sa0;
+        x.sd = raise ? d : x.sd;
+        x.best = raise ? toph : x.best;
     }
-    x.sa0 = raise ? a0 : x.sa0;
-    x.sd = raise ? d : x.sd;
-    x.best = raise ? toph : x.best;
     const int first = __ffs(bal) - 1, last = 31 - __clz(bal);
     x.llo = __shfl_sync(0xffffffffu, a0 + __ffs(lb) - 1, first & (G - 1), G);
     x.lhi = __shfl_sync(0xffffffffu, a0 + 31 - __clz(lb), last & (G - 1), G);
     // the end of the extension, or its hand-over to the 32-bit kernel
-    const bool stop = x.active && (defer || empty || bal == 0u);
+    const bool stop = x.active && (defer || bal == 0u);
     if (__any_sync(0xffffffffu, stop)) {
         if (stop) {
             if (defer) {
@@ -602,9 +642,10 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
 #pragma unroll
                 for (int j = NC - 1; j >= 0; --j) {
                     const uint32_t v = x.HS[j >> 1];
-                    if (((j & 1) ? (int)v >> 16 : (int)(short)(v & 0xffffu)) == x.best) {
+                    if (((j & 1) ? (int)v >> 16 : (int)(short)(v & 0xffffu)) + (int)(o2 & 0xffffu) == x.best) {
                         mya = (unsigned)(x.sa0 + j);
-                        if constexpr (C) myc = x.HSC[j >> 1][j & 1];
+                        if constexpr (C)
+                            myc = __byte_perm(x.HSC[0][j >> 1], x.HSC[1][j >> 1], (j & 1) ? 0x7632 : 0x5410);
                     }
                 }
                 const int ta = (int)__reduce_min_sync(smask, mya);
@@ -649,7 +690,7 @@ __device__ __forceinline__ void xd16_run(const uint8_t *qcodes, const int64_t *q
         // i = q * 768 + (t >> 1) * 64 + lane * 2 + (t & 1)
         const int q = i / 768, t = ((i % 768) >> 6) * 2 + (i & 1);
         const int v = gmat[q * PASTIS_NSYM + t];
-        s_tab[i] = C ? (uint16_t)((v & 0xff) | (q == t ? 0x100 : 0)) : (uint16_t)v;
+        s_tab[i] = C ? (uint16_t)((v & 0xff) | (q == t ? 0x100 : 0)) : (uint16_t)(v + o);
     }
     __syncthreads();
     const char *tab = (const char *)s_tab;
@@ -669,9 +710,9 @@ __device__ __forceinline__ void xd16_run(const uint8_t *qcodes, const int64_t *q
         x.QW[r] = 0u; x.TW[r] = lane4 | (lane4 << 16); x.HS[r] = XD16_NEG2;
         if constexpr (C)
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                x.HC[0][r][hf] = x.HC[1][r][hf] = x.EC[0][r][hf] = x.EC[1][r][hf] = 0u;
-                x.FC[0][r][hf] = x.FC[1][r][hf] = x.HSC[r][hf] = 0u;
+            for (int w = 0; w < 2; ++w) {
+                x.HC[w][0][r] = x.HC[w][1][r] = x.EC[w][0][r] = x.EC[w][1][r] = 0u;
+                x.FC[w][0][r] = x.FC[w][1][r] = x.HSC[w][r] = 0u;
             }
     }
     bool exhausted = false;
@@ -715,11 +756,11 @@ __device__ __forceinline__ void xd16_run(const uint8_t *qcodes, const int64_t *q
                         x.H[pp][r] = XD16_NEG2; x.E[pp][r] = XD16_NEG2; x.F[pp][r] = XD16_NEG2;
                         if constexpr (C)
 #pragma unroll
-                            for (int hf = 0; hf < 2; ++hf) {
-                                x.HC[pp][r][hf] = 0u; x.EC[pp][r][hf] = 0u; x.FC[pp][r][hf] = 0u;
+                            for (int w = 0; w < 2; ++w) {
+                                x.HC[w][pp][r] = 0u; x.EC[w][pp][r] = 0u; x.FC[w][pp][r] = 0u;
                             }
                     }
-                if (ls == 64 / WD) x.H[0][0] = XD16_NEG2 & 0xffff0000u;
+                if (ls == 64 / WD) x.H[0][0] = (XD16_NEG2 & 0xffff0000u) | ((uint32_t)(-o) & 0xffffu);
                 x.d = 0; x.best = 0; x.sd = 0; x.sa0 = 0; x.llo = 0; x.lhi = 0; x.cells = 1;
                 xd16_load_windows(x, 0, (x.kbase + WD * ls) >> 1, lane4);
                 x.active = true;
@@ -750,9 +791,7 @@ __global__ void __launch_bounds__(ALN_THREADS) k_xd_ext16(XD16_PARAMS) {
 }
 
 // With carries: the filter-only mode's second phase (over its task list) and PASTIS_XD.
-// Held to two CTAs per SM: with four extensions per warp the words take 150 registers
-// unbounded (one CTA), 128 with a few spilled, and the second occupancy pays more than
-// the spills cost.
+// Held to two CTAs per SM (128 registers with four extensions per warp).
 template <int R>
 __global__ void __launch_bounds__(ALN_THREADS, 2) k_xd_ext16_carry(XD16_PARAMS) {
     __shared__ uint16_t s_tab[XD16_TAB];

@@ -139,6 +139,11 @@ pastis_status exclusive_scan_u32(pastis_ctx *c, const uint32_t *in, uint32_t *ou
 // Exclusive scan of n int64 values into int64 offsets (n+1 entries).
 pastis_status exclusive_scan_i64(pastis_ctx *c, const int64_t *in, int64_t *out, int64_t n);
 
+// Column pointers of sorted codes: col_ptr[c] = keep_off[first x with keys[x] >= c], c = 0 ..
+// ncodes (ncodes + 1 entries); keep_off has n + 1 entries, the last the total.
+pastis_status fill_col_ptr(pastis_ctx *c, const uint32_t *keys, const uint32_t *keep_off, int64_t n, int64_t ncodes,
+                           uint32_t *col_ptr);
+
 // Raise the dynamic shared-memory limit of the kernels that size it per call to the
 // device's opt-in maximum (the current device; done at context creation).
 cudaError_t sw_set_smem_limit(size_t bytes);

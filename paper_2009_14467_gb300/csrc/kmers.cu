@@ -62,39 +62,77 @@ __global__ void k_encode(const uint8_t *__restrict__ in, int64_t n, uint8_t *__r
 
 // One thread per residue position x: the window starting at x, if it fits in its
 // sequence, becomes (key = code, value = seq << 16 | pos); otherwise key = invalid,
-// which sorts after every code.  Counts the valid windows.
-__global__ void k_windows(const uint8_t *__restrict__ codes, const int64_t *__restrict__ offsets,
-                          int32_t n, int64_t R, int k, uint32_t invalid, uint32_t *keys,
-                          uint64_t *vals, unsigned long long *n_valid, int *bad_code) {
-    int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool valid = false;
-    if (x < R) {
-        // sequence of x: the last s with offsets[s] <= x
-        int32_t lo = 0, hi = n - 1;
+// which sorts after every code.  Counts the valid windows.  A CTA takes WIN_TILE positions:
+// its residues go through shared memory, and two searches over all offsets bound the
+// sequences it meets (a search of 17 dependent loads per position took five times as long).
+constexpr int WIN_THREADS = 256, WIN_TILE = 4096, WIN_SEQS = 1024;
+
+__global__ void __launch_bounds__(WIN_THREADS) k_windows(const uint8_t *__restrict__ codes,
+                                                         const int64_t *__restrict__ offsets, int32_t n, int64_t R,
+                                                         int k, uint32_t invalid, uint32_t *keys, uint64_t *vals,
+                                                         unsigned long long *n_valid, int *bad_code) {
+    __shared__ uint8_t s_code[WIN_TILE + 8];
+    __shared__ int64_t s_off[WIN_SEQS];
+    __shared__ int32_t s_seq[2];
+    __shared__ int s_cnt[WIN_THREADS / 32];
+    const int64_t x0 = (int64_t)blockIdx.x * WIN_TILE;
+    const int m = (int)min((int64_t)WIN_TILE, R - x0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        // sequence of the first (last) position: the last s with offsets[s] <= x, 32 probes a round
+        const int64_t x = warp == 0 ? x0 : x0 + m - 1;
+        int64_t lo = 0, hi = n - 1;              // offsets[lo] <= x
         while (lo < hi) {
-            int32_t mid = (lo + hi + 1) >> 1;
-            if (offsets[mid] <= x) lo = mid; else hi = mid - 1;
+            const int64_t step = (hi - lo + 31) / 32, s = lo + step * (lane + 1);
+            const unsigned le = __ballot_sync(0xffffffffu, s <= hi && offsets[s] <= x);
+            const int c = __popc(le);            // a prefix of the probes
+            const int64_t nlo = lo + step * c;
+            hi = min(hi, nlo + step - 1);
+            lo = nlo;
         }
-        int64_t p = x - offsets[lo];
-        int64_t L = offsets[lo + 1] - offsets[lo];
+        if (lane == 0) s_seq[warp] = (int32_t)lo;
+    }
+    for (int i = threadIdx.x; i < m + k - 1; i += WIN_THREADS) s_code[i] = x0 + i < R ? codes[x0 + i] : 0;
+    __syncthreads();
+    const int32_t q0 = s_seq[0], q1 = s_seq[1];
+    const bool near = q1 - q0 + 2 <= WIN_SEQS;   // offsets q0 .. q1 + 1 fit
+    if (near)
+        for (int i = threadIdx.x; i < q1 - q0 + 2; i += WIN_THREADS) s_off[i] = offsets[q0 + i];
+    __syncthreads();
+    int valid = 0;
+    for (int i = threadIdx.x; i < m; i += WIN_THREADS) {
+        const int64_t x = x0 + i;
+        int32_t lo = q0, hi = q1;
+        while (lo < hi) {
+            const int32_t mid = (lo + hi + 1) >> 1;
+            if ((near ? s_off[mid - q0] : offsets[mid]) <= x) lo = mid; else hi = mid - 1;
+        }
+        const int64_t o0 = near ? s_off[lo - q0] : offsets[lo], o1 = near ? s_off[lo + 1 - q0] : offsets[lo + 1];
+        const int64_t p = x - o0;
         uint32_t key = invalid;
         uint64_t val = 0;
-        if (p + k <= L) {
+        if (p + k <= o1 - o0) {
             uint32_t c = 0;
             for (int t = 0; t < k; ++t) {
-                uint32_t r = codes[x + t];
+                uint32_t r = s_code[i + t];
                 if (r >= PASTIS_NSYM) { *bad_code = 1; r = 0; }
                 c = c * PASTIS_NSYM + r;
             }
             key = c;
             val = ((uint64_t)(uint32_t)lo << 16) | (uint64_t)p;
-            valid = true;
+            ++valid;
         }
         keys[x] = key;
         vals[x] = val;
     }
-    unsigned b = __ballot_sync(0xffffffffu, valid);
-    if ((threadIdx.x & 31) == 0 && b) atomicAdd(n_valid, (unsigned long long)__popc(b));
+    const int w = __reduce_add_sync(0xffffffffu, valid);
+    if (lane == 0) s_cnt[warp] = w;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int tot = 0;
+        for (int u = 0; u < WIN_THREADS / 32; ++u) tot += s_cnt[u];
+        if (tot) atomicAdd(n_valid, (unsigned long long)tot);
+    }
 }
 
 // keep[x] = 1 for the first tuple of each (code, seq) run among the valid ones
@@ -107,10 +145,10 @@ __global__ void k_first_of_run(const uint32_t *keys, const uint64_t *vals, int64
 }
 
 // Compacts the kept tuples into the CSC arrays and prepares the CSR sort input
-// (key = seq, value = code << 16 | pos); counts entries per code for col_ptr.
+// (key = seq, value = code << 16 | pos).
 __global__ void k_compact_csc(const uint32_t *keys, const uint64_t *vals, const uint32_t *keep,
                               const uint32_t *keep_off, int64_t nv, int32_t *col_seq, uint16_t *col_pos,
-                              uint32_t *code_count, uint32_t *rkeys, uint64_t *rvals) {
+                              uint32_t *rkeys, uint64_t *rvals) {
     int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= nv || !keep[x]) return;
     uint32_t o = keep_off[x];
@@ -118,7 +156,6 @@ __global__ void k_compact_csc(const uint32_t *keys, const uint64_t *vals, const 
     uint32_t pos = (uint32_t)(vals[x] & 0xFFFF);
     col_seq[o] = (int32_t)seq;
     col_pos[o] = (uint16_t)pos;
-    atomicAdd(&code_count[keys[x]], 1u);
     rkeys[o] = seq;
     rvals[o] = ((uint64_t)keys[x] << 16) | pos;
 }
@@ -221,10 +258,9 @@ extern "C" pastis_status pastis_build_kmers(pastis_ctx *ctx, const uint8_t *d_co
     if (R > 0 && !d_codes) return PASTIS_ERR_INVALID_ARG;
     if (R > 0xFFFFFFFFll) return PASTIS_ERR_UNSUPPORTED;
 
-    // col_ptr counts start at zero
-    PASTIS_CUDA_TRY(cudaMemsetAsync(A->col_ptr, 0, sizeof(uint32_t) * (ncodes + 1), st));
-    PASTIS_CUDA_TRY(cudaMemsetAsync(A->row_ptr, 0, sizeof(int64_t) * (n + 1), st));
     if (R == 0 || n == 0) {
+        PASTIS_CUDA_TRY(cudaMemsetAsync(A->col_ptr, 0, sizeof(uint32_t) * (ncodes + 1), st));
+        PASTIS_CUDA_TRY(cudaMemsetAsync(A->row_ptr, 0, sizeof(int64_t) * (n + 1), st));
         A->nnz = 0;
         if (nnz_out) *nnz_out = 0;
         PASTIS_CUDA_TRY(cudaStreamSynchronize(st));
@@ -238,7 +274,7 @@ extern "C" pastis_status pastis_build_kmers(pastis_ctx *ctx, const uint8_t *d_co
     PASTIS_WS(va, ctx, WS_SORT_VALS_A, sizeof(uint64_t) * R);
     PASTIS_WS(vb, ctx, WS_SORT_VALS_B, sizeof(uint64_t) * R);
     prof_begin(ctx, "kmer_windows");
-    k_windows<<<(unsigned)ceil_div64(R, 256), 256, 0, st>>>(d_codes, d_offsets, n, R, k,
+    k_windows<<<(unsigned)ceil_div64(R, WIN_TILE), WIN_THREADS, 0, st>>>(d_codes, d_offsets, n, R, k,
                                                           (uint32_t)ncodes, ka, va, n_valid, flags + 1);
     PASTIS_LAUNCHED(ctx);
     prof_end(ctx);
@@ -278,12 +314,11 @@ extern "C" pastis_status pastis_build_kmers(pastis_ctx *ctx, const uint8_t *d_co
     if (nv > 0) {
         prof_begin(ctx, "kmer_compact");
         k_compact_csc<<<(unsigned)ceil_div64(nv, 256), 256, 0, st>>>(sk, sv, keep, keep_off, nv, A->col_seq,
-                                                                   A->col_pos, A->col_ptr, rk, rv);
+                                                                   A->col_pos, rk, rv);
         PASTIS_LAUNCHED(ctx);
         prof_end(ctx);
     }
-    // col_ptr: exclusive scan of per-code counts, in place through the scan's tile order
-    s = exclusive_scan_u32(ctx, A->col_ptr, A->col_ptr, ncodes);
+    s = fill_col_ptr(ctx, sk, keep_off, nv, ncodes, A->col_ptr);
     if (s != PASTIS_OK) return s;
     // CSR: stable sort by sequence keeps codes ascending within a row
     uint32_t *rk2 = sk, *rko;

@@ -15,9 +15,12 @@
 //      their sorted slot, slot = (number of k-mers closer than it) + (its rank among
 //      equal distances in code order).
 // Sec. IV-C: AS(i, s) keeps the start of the k-mer of sequence i nearest to s (the
-// smaller start on ties).  AS is expanded from the rows of A and S, radix-sorted by s
-// (stable, so sequences stay ascending), reduced to one entry per (s, i), and sorted
-// again by sequence for its CSR view.
+// smaller start on ties).  Both products meet AS only at codes that A holds (AS rows against
+// A's posting lists, A's rows against AS's), so only the substitutes present in A are
+// kept: about a seventh of them at 20,000 proteins (182 M entries; building AS and the product
+// 31 ms with all of them, 12 ms so), two fifths at 100,000.  AS is expanded from the
+// rows of A and these rows of S, radix-sorted by s (stable, so sequences stay ascending),
+// reduced to one entry per (s, i), and sorted again by sequence for its CSR view.
 #include <string.h>
 
 #include "internal.cuh"
@@ -103,10 +106,15 @@ __device__ __noinline__ int subk_cut_far(const uint8_t *s_hist, uint32_t digs, i
 // shared memory, and a CTA's rows, contiguous in the output, leave in one linear copy.
 // Measured with m = 25 and k = 6 on the distinct 6-mers of 20,000 proteins: 69.8 ms with the
 // counts in local memory and every replacement tried at every level, 6.0 ms so.
+// PRESENT: only the entries whose code's bit is set in `bits` leave, in their order at the
+// front of the root's row, and their number in out_n.
+template <bool PRESENT>
 __global__ void __launch_bounds__(SUBK_THREADS) k_subkmers(const uint32_t *__restrict__ roots, int64_t n_roots,
                                                            int k, int m, const int8_t *__restrict__ gmat,
+                                                           const uint32_t *__restrict__ bits,
                                                            uint32_t *__restrict__ out_code,
-                                                           int32_t *__restrict__ out_dist, int *err) {
+                                                           int32_t *__restrict__ out_dist,
+                                                           uint32_t *__restrict__ out_n, int *err) {
     extern __shared__ __align__(16) unsigned char subk_smem[];
     __shared__ __align__(16) uint8_t s_hist[PASTIS_NSYM * SUBK_DLIM];   // replacements of a residue at each expense
     __shared__ uint32_t s_mask[PASTIS_NSYM * SUBK_DLIM];                // replacements of a residue within a budget
@@ -202,7 +210,28 @@ __global__ void __launch_bounds__(SUBK_THREADS) k_subkmers(const uint32_t *__res
                 dist_row[1 + slot] = (int16_t)((int)ps + shift_total);
             }
         }
+        if (PRESENT) {
+            uint32_t cnt = 0;
+            const int64_t o = r * (m + 1);
+            for (int w0 = 0; w0 <= m && (cut >= 0 || m == 0); w0 += 8) {
+                uint32_t word[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) word[u] = w0 + u <= m ? bits[code_row[w0 + u] >> 5] : 0u;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (w0 + u > m) break;
+                    const uint32_t code = code_row[w0 + u];
+                    if ((word[u] >> (code & 31u)) & 1u) {
+                        out_code[o + cnt] = code;
+                        out_dist[o + cnt] = dist_row[w0 + u];
+                        ++cnt;
+                    }
+                }
+            }
+            out_n[r] = cnt;
+        }
     }
+    if (PRESENT) return;
     __syncthreads();
     const int64_t left = n_roots - r0;
     const int words = (int)(left < T ? left : T) * (m + 1);
@@ -223,39 +252,119 @@ int subk_threads(int m) {
     return T;
 }
 
-__global__ void k_present_flags(const uint32_t *col_ptr, int64_t ncodes, uint32_t *flags) {
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < ncodes) flags[c] = col_ptr[c + 1] > col_ptr[c] ? 1u : 0u;
+// The codes A holds, as a bit map over all codes (one read of col_ptr), with the number set
+// in each tile of ROOT_TILE codes.
+constexpr int ROOT_THREADS = 256, ROOT_TILE = ROOT_THREADS * 32;
+
+__global__ void __launch_bounds__(ROOT_THREADS) k_present_bits(const uint32_t *__restrict__ col_ptr, int64_t ncodes,
+                                                               uint32_t *__restrict__ bits,
+                                                               uint32_t *__restrict__ tile_n) {
+    __shared__ uint32_t s_n[ROOT_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t c0 = (int64_t)blockIdx.x * ROOT_TILE;
+    uint32_t n = 0;
+#pragma unroll 4
+    for (int w = warp; w < ROOT_TILE / 32; w += ROOT_THREADS / 32) {
+        const int64_t c = c0 + w * 32 + lane;
+        const uint32_t here = c <= ncodes ? col_ptr[c] : 0u;
+        uint32_t next = __shfl_down_sync(0xffffffffu, here, 1);
+        if (lane == 31) next = c < ncodes ? col_ptr[c + 1] : 0u;
+        const uint32_t b = __ballot_sync(0xffffffffu, c < ncodes && next > here);
+        if (lane == 0 && c0 + w * 32 < ncodes) bits[(c0 >> 5) + w] = b;
+        n += __popc(b);
+    }
+    if (lane == 0) s_n[warp] = n;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t t = 0;
+        for (int w = 0; w < ROOT_THREADS / 32; ++w) t += s_n[w];
+        tile_n[blockIdx.x] = t;
+    }
 }
 
-__global__ void k_gather_roots(const uint32_t *flags, const uint32_t *idx, int64_t ncodes, uint32_t *roots) {
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < ncodes && flags[c]) roots[idx[c]] = (uint32_t)c;
+// The present codes in order, and before each word of the bit map the number set before it,
+// so that a code's place among the roots is two cached reads.
+__global__ void __launch_bounds__(ROOT_THREADS) k_roots(const uint32_t *__restrict__ bits, int64_t nwords,
+                                                        const uint32_t *__restrict__ tile_off,
+                                                        uint32_t *__restrict__ before, uint32_t *__restrict__ roots) {
+    __shared__ uint32_t s_n[ROOT_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w = (int64_t)blockIdx.x * ROOT_THREADS + threadIdx.x;
+    uint32_t b = w < nwords ? bits[w] : 0u;
+    uint32_t incl = __popc(b);
+    const uint32_t own = incl;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += y;
+    }
+    if (lane == 31) s_n[warp] = incl;
+    __syncthreads();
+    uint32_t at = tile_off[blockIdx.x] + incl - own;
+    for (int u = 0; u < warp; ++u) at += s_n[u];
+    if (w < nwords) before[w] = at;
+    while (b) {
+        const int x = __ffs(b) - 1;
+        b &= b - 1u;
+        roots[at++] = (uint32_t)(w * 32 + x);
+    }
 }
 
-// Expansion of AS: entry (x, t) of A row i and substitute t of its code becomes
-// key = substitute code, value = i << 32 | dist << 16 | pos.  Rows are walked in order,
-// so equal substitutes keep ascending i after a stable sort by key.
-__global__ void k_expand_as(const int64_t *row_ptr, const uint32_t *row_code, const uint16_t *row_pos,
-                            int32_t n, const uint32_t *root_index, const uint32_t *sub_code,
-                            const int32_t *sub_dist, int m, uint32_t *keys, uint64_t *vals) {
-    int64_t nnz = row_ptr[n];
-    int64_t tot = nnz * (m + 1);
-    for (int64_t y = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; y < tot;
-         y += (int64_t)gridDim.x * blockDim.x) {
-        int64_t x = y / (m + 1);
-        int t = (int)(y - x * (m + 1));
-        // row of x
-        int32_t lo = 0, hi = n - 1;
+__device__ __forceinline__ uint32_t root_of(const uint32_t *bits, const uint32_t *before, uint32_t code) {
+    const uint32_t w = code >> 5;
+    return before[w] + __popc(bits[w] & ((1u << (code & 31u)) - 1u));
+}
+
+// Substitutes kept for each entry of A.
+__global__ void k_as_count(const uint32_t *__restrict__ row_code, int64_t nnz, const uint32_t *__restrict__ bits,
+                           const uint32_t *__restrict__ before, const uint32_t *__restrict__ sub_n,
+                           uint32_t *__restrict__ cnt) {
+    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (x < nnz) cnt[x] = sub_n[root_of(bits, before, row_code[x])];
+}
+
+// Expansion of AS: entry x of A row i and substitute t of its code becomes key =
+// substitute code, value = i << 32 | dist << 16 | pos, from off[x] on.  Rows are walked in
+// order, so equal substitutes keep ascending i after a stable sort by key.
+__global__ void __launch_bounds__(256) k_expand_as(const int64_t *__restrict__ row_ptr,
+                                                   const uint32_t *__restrict__ row_code,
+                                                   const uint16_t *__restrict__ row_pos, int32_t n, int64_t nnz,
+                                                   const uint32_t *__restrict__ bits,
+                                                   const uint32_t *__restrict__ before,
+                                                   const uint32_t *__restrict__ sub_code,
+                                                   const int32_t *__restrict__ sub_dist, int m,
+                                                   const uint32_t *__restrict__ off, uint32_t *__restrict__ keys,
+                                                   uint64_t *__restrict__ vals) {
+    // the rows of the CTA's first and last entry bound the search of each
+    __shared__ int32_t s_row[2];
+    const int64_t x0 = (int64_t)blockIdx.x * blockDim.x, x = x0 + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        const int64_t y = warp == 0 ? x0 : min(x0 + blockDim.x, nnz) - 1;
+        int64_t lo = 0, hi = n - 1;              // the last row with row_ptr[row] <= y
         while (lo < hi) {
-            int32_t mid = (lo + hi + 1) >> 1;
-            if (row_ptr[mid] <= x) lo = mid; else hi = mid - 1;
+            const int64_t step = (hi - lo + 31) / 32, r = lo + step * (lane + 1);
+            const int c = __popc(__ballot_sync(0xffffffffu, r <= hi && row_ptr[r] <= y));
+            const int64_t nlo = lo + step * c;
+            hi = min(hi, nlo + step - 1);
+            lo = nlo;
         }
-        uint32_t ri = root_index[row_code[x]];
-        int64_t sidx = (int64_t)ri * (m + 1) + t;
-        keys[y] = sub_code[sidx];
+        if (lane == 0) s_row[warp] = (int32_t)lo;
+    }
+    __syncthreads();
+    if (x >= nnz) return;
+    int32_t lo = s_row[0], hi = s_row[1];
+    while (lo < hi) {
+        const int32_t mid = (lo + hi + 1) >> 1;
+        if (row_ptr[mid] <= x) lo = mid; else hi = mid - 1;
+    }
+    const int64_t sidx = (int64_t)root_of(bits, before, row_code[x]) * (m + 1);
+    const uint64_t base = ((uint64_t)(uint32_t)lo << 32) | row_pos[x];
+    const uint32_t o = off[x], c = off[x + 1] - o;
+    for (uint32_t t = 0; t < c; ++t) {
+        keys[o + t] = sub_code[sidx + t];
         // distances are biased by 1024 so that (dist, pos) orders as one unsigned word
-        vals[y] = ((uint64_t)(uint32_t)lo << 32) | ((uint64_t)(uint32_t)(sub_dist[sidx] + 1024) << 16) | row_pos[x];
+        vals[o + t] = base | ((uint64_t)(uint32_t)(sub_dist[sidx + t] + 1024) << 16);
     }
 }
 
@@ -279,7 +388,7 @@ __global__ void k_reduce_as_runs(const uint32_t *keys, uint64_t *vals, int64_t n
 
 __global__ void k_compact_as(const uint32_t *keys, const uint64_t *vals, const uint32_t *keep,
                              const uint32_t *off, int64_t n, int32_t *col_seq, uint16_t *col_pos,
-                             uint32_t *code_count, uint32_t *rkeys, uint64_t *rvals) {
+                             uint32_t *rkeys, uint64_t *rvals) {
     int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= n || !keep[x]) return;
     uint32_t o = off[x];
@@ -287,7 +396,6 @@ __global__ void k_compact_as(const uint32_t *keys, const uint64_t *vals, const u
     uint16_t pos = (uint16_t)(vals[x] & 0xFFFF);
     col_seq[o] = (int32_t)seq;
     col_pos[o] = pos;
-    atomicAdd(&code_count[keys[x]], 1u);
     rkeys[o] = seq;
     rvals[o] = ((uint64_t)keys[x] << 16) | pos;
 }
@@ -318,7 +426,8 @@ int bits_for_u64(uint64_t v) {
 }
 
 pastis_status launch_subkmers(pastis_ctx *ctx, const uint32_t *d_roots, int64_t n_roots, int k, int m,
-                              const pastis_params *params, uint32_t *d_code, int32_t *d_dist) {
+                              const pastis_params *params, uint32_t *d_code, int32_t *d_dist,
+                              const uint32_t *d_bits = nullptr, uint32_t *d_n = nullptr) {
     int8_t *dmat;
     PASTIS_WS(dmat, ctx, WS_FLAGS, 1024);
     int *err = (int *)(dmat + 768);
@@ -327,8 +436,9 @@ pastis_status launch_subkmers(pastis_ctx *ctx, const uint32_t *d_roots, int64_t 
     if (n_roots > 0) {
         prof_begin(ctx, "subkmers");
         const int T = subk_threads(m);
-        k_subkmers<<<(unsigned)ceil_div64(n_roots, T), T, subk_smem_bytes(T, m), ctx->stream>>>(
-            d_roots, n_roots, k, m, dmat, d_code, d_dist, err);
+        auto kern = d_bits ? k_subkmers<true> : k_subkmers<false>;
+        kern<<<(unsigned)ceil_div64(n_roots, T), T, subk_smem_bytes(T, m), ctx->stream>>>(
+            d_roots, n_roots, k, m, dmat, d_bits, d_code, d_dist, d_n, err);
         PASTIS_LAUNCHED(ctx);
         prof_end(ctx);
     }
@@ -455,30 +565,47 @@ pastis_status build_as_fresh(pastis_ctx *ctx, const pastis_kmat *A, const pastis
     const int64_t ncodes = ipow24(k);
     const int32_t n = A->n_rows;
     const int64_t nnzA = A->nnz;
-    // distinct codes present in A, and their index
-    uint32_t *flags;
-    PASTIS_WS(flags, ctx, WS_SUB_ROOTS, sizeof(uint32_t) * (2 * (size_t)ncodes + 2));
-    uint32_t *root_index = flags + ncodes + 1;
-    k_present_flags<<<(unsigned)ceil_div64(ncodes, 256), 256, 0, st>>>(A->col_ptr, ncodes, flags);
+    // the products of rows and substitutes that fit the sort's indexes
+    if (nnzA * (m + 1) > 0xFFFFFFFFll) return PASTIS_ERR_UNSUPPORTED;
+    // the codes present in A: bit map, rank, and the roots in order
+    const int64_t nwords = ceil_div64(ncodes, 32), ntile = ceil_div64(ncodes, ROOT_TILE);
+    uint32_t *bits;
+    PASTIS_WS(bits, ctx, WS_SUB_ROOTS, sizeof(uint32_t) * (2 * (size_t)nwords + 2 * (size_t)ntile + 2));
+    uint32_t *before = bits + nwords, *tile_n = before + nwords, *tile_off = tile_n + ntile;
+    prof_begin(ctx, "as_roots");
+    k_present_bits<<<(unsigned)ntile, ROOT_THREADS, 0, st>>>(A->col_ptr, ncodes, bits, tile_n);
     PASTIS_LAUNCHED(ctx);
-    pastis_status s = exclusive_scan_u32(ctx, flags, root_index, ncodes);
+    prof_end(ctx);
+    pastis_status s = exclusive_scan_u32(ctx, tile_n, tile_off, ntile);
     if (s != PASTIS_OK) return s;
     uint32_t h_nroots = 0;
-    PASTIS_CUDA_TRY(cudaMemcpyAsync(&h_nroots, root_index + ncodes, 4, cudaMemcpyDeviceToHost, st));
+    PASTIS_CUDA_TRY(cudaMemcpyAsync(&h_nroots, tile_off + ntile, 4, cudaMemcpyDeviceToHost, st));
     PASTIS_CUDA_TRY(cudaStreamSynchronize(st));
     const int64_t nroots = h_nroots;
     uint32_t *roots, *sc;
     int32_t *sd;
-    PASTIS_WS(roots, ctx, WS_AS_TMP_KEY, sizeof(uint32_t) * (nroots + 1));
+    PASTIS_WS(roots, ctx, WS_AS_TMP_KEY, 2 * sizeof(uint32_t) * (nroots + 1));
+    uint32_t *sub_n = roots + nroots + 1;
     PASTIS_WS(sc, ctx, WS_SUB_CODE, sizeof(uint32_t) * (nroots + 1) * (m + 1));
     PASTIS_WS(sd, ctx, WS_SUB_DIST, sizeof(int32_t) * (nroots + 1) * (m + 1));
-    k_gather_roots<<<(unsigned)ceil_div64(ncodes, 256), 256, 0, st>>>(flags, root_index, ncodes, roots);
+    k_roots<<<(unsigned)ntile, ROOT_THREADS, 0, st>>>(bits, nwords, tile_off, before, roots);
     PASTIS_LAUNCHED(ctx);
-    s = launch_subkmers(ctx, roots, nroots, k, m, p, sc, sd);
+    s = launch_subkmers(ctx, roots, nroots, k, m, p, sc, sd, bits, sub_n);
     if (s != PASTIS_OK) return s;
-    // expand AS
-    const int64_t ne = nnzA * (m + 1);
-    if (ne > 0xFFFFFFFFll) return PASTIS_ERR_UNSUPPORTED;
+    // expand AS: the kept substitutes of every entry of A
+    uint32_t *cnt;
+    PASTIS_WS(cnt, ctx, WS_KMER_TMP, sizeof(uint32_t) * (2 * (size_t)nnzA + 2));
+    uint32_t *cnt_off = cnt + nnzA + 1;
+    if (nnzA > 0) {
+        k_as_count<<<(unsigned)ceil_div64(nnzA, 256), 256, 0, st>>>(A->row_code, nnzA, bits, before, sub_n, cnt);
+        PASTIS_LAUNCHED(ctx);
+    }
+    s = exclusive_scan_u32(ctx, cnt, cnt_off, nnzA);
+    if (s != PASTIS_OK) return s;
+    uint32_t h_ne = 0;
+    PASTIS_CUDA_TRY(cudaMemcpyAsync(&h_ne, cnt_off + nnzA, 4, cudaMemcpyDeviceToHost, st));
+    PASTIS_CUDA_TRY(cudaStreamSynchronize(st));
+    const int64_t ne = h_ne;
     uint32_t *ka, *kb;
     uint64_t *va, *vb;
     PASTIS_WS(ka, ctx, WS_SORT_KEYS_A, sizeof(uint32_t) * (ne + 1));
@@ -486,11 +613,9 @@ pastis_status build_as_fresh(pastis_ctx *ctx, const pastis_kmat *A, const pastis
     PASTIS_WS(va, ctx, WS_SORT_VALS_A, sizeof(uint64_t) * (ne + 1));
     PASTIS_WS(vb, ctx, WS_SORT_VALS_B, sizeof(uint64_t) * (ne + 1));
     if (ne > 0) {
-        int blocks = (int)ceil_div64(ne, 256);
-        if (blocks > ctx->sm_count * 32) blocks = ctx->sm_count * 32;
         prof_begin(ctx, "as_expand");
-        k_expand_as<<<blocks, 256, 0, st>>>(A->row_ptr, A->row_code, A->row_pos, n, root_index, sc, sd, m,
-                                           ka, va);
+        k_expand_as<<<(unsigned)ceil_div64(nnzA, 256), 256, 0, st>>>(A->row_ptr, A->row_code, A->row_pos, n, nnzA, bits,
+                                                                     before, sc, sd, m, cnt_off, ka, va);
         PASTIS_LAUNCHED(ctx);
         prof_end(ctx);
     }
@@ -520,17 +645,16 @@ pastis_status build_as_fresh(pastis_ctx *ctx, const pastis_kmat *A, const pastis
     PASTIS_WS(out->row_ptr, ctx, WS_AS_ROWPTR, sizeof(int64_t) * (n + 1));
     PASTIS_WS(out->row_code, ctx, WS_AS_CODE, sizeof(uint32_t) * (nnz + 1));
     PASTIS_WS(out->row_pos, ctx, WS_AS_POS, sizeof(uint16_t) * (nnz + 1));
-    PASTIS_CUDA_TRY(cudaMemsetAsync(out->col_ptr, 0, sizeof(uint32_t) * (ncodes + 1), st));
     uint32_t *rk = (sk == ka) ? kb : ka;
     uint64_t *rv = (sv == va) ? vb : va;
     if (ne > 0) {
         prof_begin(ctx, "as_compact");
         k_compact_as<<<(unsigned)ceil_div64(ne, 256), 256, 0, st>>>(sk, sv, keep, off, ne, out->col_seq,
-                                                                   out->col_pos, out->col_ptr, rk, rv);
+                                                                   out->col_pos, rk, rv);
         PASTIS_LAUNCHED(ctx);
         prof_end(ctx);
     }
-    s = exclusive_scan_u32(ctx, out->col_ptr, out->col_ptr, ncodes);
+    s = fill_col_ptr(ctx, sk, off, ne, ncodes, out->col_ptr);
     if (s != PASTIS_OK) return s;
     uint32_t *rko;
     uint64_t *rvo;

@@ -54,3 +54,23 @@ def test_tile_edges(total):
 def test_codes_at_the_ends_of_the_range(letters):
     _check(_strings([700, 3, 0, 1200], 5, letters), 4)
     _check(_strings([700, 3, 0, 1200], 6, letters), 3)
+
+
+@pytest.mark.parametrize("k,m", [(1, 10), (2, 25), (3, 7), (3, 60), (6, 25)])
+def test_substitute_candidates_where_few_or_all_codes_are_present(k, m):
+    """A S keeps the substitutes that A holds: candidates equal the oracle's where that is
+    nearly every code (short k) and nearly none (k = 6 on a small set)."""
+    import paper_2009_14467_gb300 as P
+    mat = synth.blosum62()
+    ctx = P.Context(0)
+    rng = np.random.default_rng(10 * k + m)
+    ps = synth.from_strings(_strings(list(rng.integers(0, 40 if k < 3 else 300, 30)), k + m,
+                                     "ACDEFGHIKLMNPQRSTVWYBZX*"))
+    codes = O.encode(ps.ascii)
+    params = P.Params(matrix=mat, k=k, m_subs=m)
+    A = P.build_kmers(ctx, torch.from_numpy(codes).cuda(), torch.from_numpy(ps.offsets).cuda(), k)
+    got = P.to_records(P.overlap_spgemm(ctx, A, params), P.CAND_DTYPE)
+    rp, code, pos = O.kmers(codes, ps.offsets, k)
+    want = O.candidates(rp, code, pos, k, m, mat, 1)
+    assert got.tobytes() == want.tobytes()
+    ctx.close()

@@ -8,14 +8,14 @@
 // (AS)_i . A_j and A_i . (AS)_j, and each pair keeps the orientation that shares more
 // (i -> j on ties).
 //
-// Row-wise hash SpGEMM in two kernels.
+// Row-wise SpGEMM in two steps.
 //  * Cursors: one warp per row i.  Each left entry t of the row (a k-mer of AS_i, and of
 //    A_i for the second orientation) finds where its posting list (sorted by sequence)
 //    reaches the row's first column j >= jlo; entries with a non-empty rest keep a
 //    cursor (next j, posting index, posting end).  The warp also sums the row's exact
 //    product count.
-//  * Rows: one CTA per row, a hash table in shared memory keyed by j (count and two
-//    seeds per orientation).  A row whose products could overflow the table is formed
+//  * Rows: one CTA per row.  Up to 4,096 products are sorted (k_spgemm_sort).  More go
+//    to a hash table in shared memory keyed by j (count and two seeds per orientation).  A row whose products could overflow the table is formed
 //    in column ranges [a, z), in order; each range advances every cursor up to z, so
 //    each posting entry is visited once however many ranges the row takes.  An entry
 //    inserts count += 1 and the seed t << 16 | pos_j into a two-smallest pair with
@@ -420,6 +420,191 @@ __global__ void __launch_bounds__(SPG_THREADS_MAX) k_spgemm_rows(operand F, oper
     }
 }
 
+// ---------------------------------------------------------------------------------
+// Rows of up to SORT_MAX products: all of them in shared memory as one 64-bit word each,
+// (column j, orientation, entry t, position), sorted.  A run of equal j is a candidate, its
+// orientations and in them the seeds of smallest code in order, so counts, seeds and the
+// order of the records come without a table.  The table's time is its shared-memory atomics
+// (four per product, with the wait for each result) and clearing; the sort has none and is
+// bound by its compares: bitonic, SORT_E words a thread, distances below SORT_E in
+// registers, below 32 SORT_E by shuffles, the others (3 of 66 steps for 2,048 words) through
+// shared memory.  Its steps grow with log^2 of the row, so the line is where the table
+// catches up.  Measured, 200,000 proteins' first 25,000 rows (23.1 M candidates), rows
+// kernels together: table only 3.30 ms, sort up to 1,024 products 2.73, 2,048 1.72, 4,096
+// 1.30, 8,192 1.40; (A S) of 20,000 proteins: 3.8, 3.72, 3.47, 3.24, 3.55 ms.  SORT_E 8
+// against 4 and 16: 1.12, 1.35 and 1.11 ms, with substitutes 1.52, 1.78 and 1.69.
+// ---------------------------------------------------------------------------------
+constexpr int SORT_MAX = 4096;
+constexpr int SORT_E = 8;                  // words a thread
+
+__device__ __forceinline__ void keep_order(uint64_t &a, uint64_t &b, bool up) {
+    const bool swap = (a > b) == up;
+    const uint64_t x = swap ? b : a, y = swap ? a : b;
+    a = x;
+    b = y;
+}
+
+// v[r] of thread tid is word tid * E + r.
+template <int E>
+__device__ __forceinline__ void block_bitonic(uint64_t (&v)[E], uint64_t *s) {
+    const int tid = threadIdx.x, nt = blockDim.x, n = nt * E;
+#pragma unroll
+    for (int k = 2; k <= E; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1)
+#pragma unroll
+            for (int r = 0; r < E; ++r)
+                if ((r & j) == 0) keep_order(v[r], v[r | j], k == E ? (tid & 1) == 0 : (r & k) == 0);
+    for (int k = 2 * E; k <= n; k <<= 1) {
+        const bool up = ((tid * E) & k) == 0;
+        int j = k >> 1;
+        for (; j >= 32 * E; j >>= 1) {
+            const int other = tid ^ (j / E);
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < E; ++r) s[r * nt + tid] = v[r];
+            __syncthreads();
+            const bool low = ((tid < other) == up);
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                const uint64_t o = s[r * nt + other];
+                v[r] = (o < v[r]) == low ? o : v[r];
+            }
+        }
+        for (; j >= E; j >>= 1) {
+            const int d = j / E;
+            const bool low = ((tid & d) == 0) == up;
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                const uint64_t o = __shfl_xor_sync(0xffffffffu, v[r], d);
+                v[r] = (o < v[r]) == low ? o : v[r];
+            }
+        }
+#pragma unroll
+        for (int i = E >> 1; i > 0; i >>= 1)
+#pragma unroll
+            for (int r = 0; r < E; ++r)
+                if ((r & i) == 0) keep_order(v[r], v[r | i], up);
+    }
+}
+
+template <bool SUBS>
+__global__ void __launch_bounds__(SORT_MAX / SORT_E) k_spgemm_sort(operand F, operand B, const row_item *items, int tbits,
+                                                              int32_t min_shared, cursors cur, pastis_cand *tmp_out,
+                                                              int64_t *item_count, int *item_error,
+                                                              unsigned long long *stats) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *s = (uint64_t *)smem;                       // E words a thread
+    __shared__ int s_n;
+    __shared__ uint32_t s_warp[SORT_MAX / SORT_E / 32];
+    constexpr int E = SORT_E;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int cap = nt * E, jshift = 16 + tbits + (SUBS ? 1 : 0);
+    const row_item it = items[blockIdx.x];
+    const int64_t e0 = it.ent_off;
+    if (tid == 0) s_n = 0;
+    for (int x = tid; x < cap; x += nt) s[x] = ~0ull;
+    __syncthreads();
+    // the products of every cursor
+    for (int64_t e = tid; e - tid < it.n_act; e += nt) {
+        const bool in = e < it.n_act;
+        int64_t x = 0, pe = 0;
+        uint32_t tt = 0;
+        if (in) { x = cur.x[e0 + e]; pe = cur.pe[e0 + e]; tt = cur.t[e0 + e]; }
+        const int c = (int)(pe - x);
+        int incl = c;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += y;
+        }
+        int at = 0;
+        if (lane == 31) at = atomicAdd(&s_n, incl);
+        at = __shfl_sync(0xffffffffu, at, 31) + incl - c;
+        const bool sb = SUBS && (tt & SIDE_B);
+        const int32_t *cs = sb ? B.col_seq : F.col_seq;
+        const uint16_t *cp = sb ? B.col_pos : F.col_pos;
+        const uint64_t low = ((uint64_t)(sb ? 1u : 0u) << (16 + tbits)) | ((uint64_t)(tt & ~SIDE_B) << 16);
+        for (; x < pe; ++x, ++at)
+            if (at < cap) s[at] = ((uint64_t)(uint32_t)cs[x] << jshift) | low | cp[x];
+    }
+    __syncthreads();
+    const int n = s_n;
+    if (n > cap) {                                        // cannot happen: the capacity is the row's products
+        if (tid == 0) { item_error[blockIdx.x] = 1; item_count[blockIdx.x] = 0; }
+        return;
+    }
+    uint64_t v[E];
+#pragma unroll
+    for (int r = 0; r < E; ++r) v[r] = s[r * nt + tid];          // any order will do
+    block_bitonic<E>(v, s);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < E; ++r) s[tid * E + r] = v[r];
+    __syncthreads();
+    // runs of equal j
+    const uint64_t tmask = (1ull << (16 + tbits)) - 1ull;
+    int64_t out_n = 0;
+    for (int i0 = 0; i0 < n; i0 += nt) {
+        const int i = i0 + tid;
+        bool keep = false;
+        uint32_t c0 = 0, c1 = 0;                          // entries of either orientation
+        uint64_t f0 = SEED_NONE, f1 = SEED_NONE, b0 = SEED_NONE, b1 = SEED_NONE;
+        uint64_t j = 0;
+        if (i < n) {
+            uint64_t w = s[i];
+            j = w >> jshift;
+            if (i == 0 || (s[i - 1] >> jshift) != j) {
+                for (int y = i;;) {
+                    if (SUBS && ((w >> (16 + tbits)) & 1ull)) {
+                        if (c1 == 0) b0 = w & tmask; else if (c1 == 1) b1 = w & tmask;
+                        ++c1;
+                    } else {
+                        if (c0 == 0) f0 = w & tmask; else if (c0 == 1) f1 = w & tmask;
+                        ++c0;
+                    }
+                    if (++y >= n) break;
+                    w = s[y];
+                    if ((w >> jshift) != j) break;
+                }
+                keep = (int64_t)max(c0, c1) >= (int64_t)min_shared;
+            }
+        }
+        const unsigned b = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) s_warp[warp] = __popc(b);
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+        for (int w = 0; w < (nt >> 5); ++w) {
+            const uint32_t q = s_warp[w];
+            before += w < warp ? q : 0u;
+            total += q;
+        }
+        if (keep && out_n + total <= it.out_cap) {
+            pastis_cand rec;
+            rec.i = it.i;
+            rec.j = (int32_t)j;
+            const bool use_b = SUBS && c1 > c0;
+            rec.count = use_b ? c1 : c0;
+            const int64_t rb = use_b ? B.row_ptr[it.i] : F.row_ptr[it.i];
+            const uint16_t *lpos = use_b ? B.row_pos : F.row_pos;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint64_t w = use_b ? (q ? b1 : b0) : (q ? f1 : f0);
+                rec.qpos[q] = w == SEED_NONE ? (uint16_t)0xFFFF : lpos[rb + (int64_t)(w >> 16)];
+                rec.tpos[q] = w == SEED_NONE ? (uint16_t)0xFFFF : (uint16_t)(w & 0xFFFF);
+            }
+            tmp_out[it.out_off + out_n + before + __popc(b & ((1u << lane) - 1u))] = rec;
+        }
+        out_n += total;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        if (out_n > it.out_cap) { item_error[blockIdx.x] = 1; out_n = 0; }   // cannot happen either
+        item_count[blockIdx.x] = out_n;
+        if (stats) atomicAdd(&stats[2], (unsigned long long)out_n);
+    }
+}
+
 __global__ void k_concat(const pastis_cand *tmp, const int64_t *src_off, const int64_t *dst_off, const int64_t *cnt,
                          int64_t n_items, pastis_cand *out) {
     // one warp per item
@@ -566,6 +751,15 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
     while (tmax > 64 && table_bytes(tmax, subs) + 64 > ctx->smem_optin) tmax >>= 1;
     int tl_max = 0;
     while ((1 << tl_max) < tmax) ++tl_max;
+    // rows whose products can be sorted as 64-bit words in shared memory (bins SORT_BIN + the
+    // logarithm of the words), where the word has room for column, orientation and entry
+    constexpr int SORT_BIN = 32;
+    int64_t max_ent = 0;
+    for (int64_t r = 0; r < ni; ++r) max_ent = std::max(max_ent, (r + 1 < ni ? ent_off[r + 1] : n_ent) - ent_off[r]);
+    int tbits = 1, jbits = 1;
+    while ((max_ent >> tbits) != 0) ++tbits;
+    while (((int64_t)n_cols >> jbits) != 0) ++jbits;
+    const bool sortable = 16 + tbits + (subs ? 1 : 0) + jbits <= 63;
     struct plan_row { row_item it; int tlog; int64_t order; };
     std::vector<plan_row> plan;
     plan.reserve((size_t)ni);
@@ -581,7 +775,12 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
         p.it.n_act = nact[r];
         p.it.out_cap = est;
         p.order = r;
-        if (est * 4 <= (int64_t)tmax * 3) {
+        if (sortable && nprod[r] <= SORT_MAX) {
+            int tl = 8;                          // a warp's words
+            while ((1ll << tl) < nprod[r]) ++tl;
+            p.tlog = SORT_BIN + tl;
+            p.it.pieces = 1;
+        } else if (est * 4 <= (int64_t)tmax * 3) {
             int tl = 6;
             while ((1ll << tl) * 3 < est * 4) ++tl;
             p.tlog = tl;
@@ -613,13 +812,18 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
         while (x0 < np) {
             int64_t x1 = x0;
             while (x1 < np && plan[x1].tlog == plan[x0].tlog) ++x1;
-            const int tsize = 1 << plan[x0].tlog;
-            const size_t shm = table_bytes(tsize, subs);
+            const bool sorted = plan[x0].tlog >= SORT_BIN;
+            const int tsize = 1 << (sorted ? plan[x0].tlog - SORT_BIN : plan[x0].tlog);
+            const size_t shm = sorted ? (size_t)tsize * 8 : table_bytes(tsize, subs);
             for (int64_t g0 = x0; g0 < x1; g0 += 65535) {
                 const int64_t g1 = std::min<int64_t>(x1, g0 + 65535);
                 prof_begin(ctx, "spgemm_rows");
-                const int nth = spg_threads_for(tsize);
-                if (subs)
+                const int nth = sorted ? tsize / SORT_E : spg_threads_for(tsize);
+                if (sorted) {
+                    auto kern = subs ? k_spgemm_sort<true> : k_spgemm_sort<false>;
+                    kern<<<(unsigned)(g1 - g0), nth, shm, st>>>(F, Bop, d_items + g0, tbits, params->min_shared, cur, tmp,
+                                                                d_cnt + g0, d_err + g0, stats);
+                } else if (subs)
                     k_spgemm_rows<true><<<(unsigned)(g1 - g0), nth, shm, st>>>(
                         F, Bop, d_items + g0, tsize, params->min_shared, self ? 1 : 0, n_cols, cur, tmp, d_cnt + g0,
                         d_err + g0, stats);

@@ -753,14 +753,14 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
     while ((1 << tl_max) < tmax) ++tl_max;
     // rows whose products can be sorted as 64-bit words in shared memory (bins SORT_BIN + the
     // logarithm of the words), where the word has room for column, orientation and entry
-    constexpr int SORT_BIN = 32;
+    constexpr int SORT_BIN = 32, PLAN_BINS = 64;
     int64_t max_ent = 0;
     for (int64_t r = 0; r < ni; ++r) max_ent = std::max(max_ent, (r + 1 < ni ? ent_off[r + 1] : n_ent) - ent_off[r]);
     int tbits = 1, jbits = 1;
     while ((max_ent >> tbits) != 0) ++tbits;
     while (((int64_t)n_cols >> jbits) != 0) ++jbits;
     const bool sortable = 16 + tbits + (subs ? 1 : 0) + jbits <= 63;
-    struct plan_row { row_item it; int tlog; int64_t order; };
+    struct plan_row { row_item it; int tlog; };
     std::vector<plan_row> plan;
     plan.reserve((size_t)ni);
     int64_t tmp_total = 0;
@@ -774,7 +774,6 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
         p.it.ent_off = ent_off[r];
         p.it.n_act = nact[r];
         p.it.out_cap = est;
-        p.order = r;
         if (sortable && nprod[r] <= SORT_MAX) {
             int tl = 8;                          // a warp's words
             while ((1ll << tl) < nprod[r]) ++tl;
@@ -797,9 +796,18 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
     int64_t total = 0;
     pastis_cand *result = nullptr;
     if (np > 0) {
-        std::stable_sort(plan.begin(), plan.end(), [](const plan_row &a, const plan_row &b) { return a.tlog < b.tlog; });
+        // items by kernel and table size, in row order within each: place[x] = item of row x
+        int64_t bin_at[PLAN_BINS + 1] = {0};
+        for (const plan_row &p : plan) ++bin_at[p.tlog + 1];
+        for (int b = 0; b < PLAN_BINS; ++b) bin_at[b + 1] += bin_at[b];
+        int64_t next[PLAN_BINS];
+        std::copy(bin_at, bin_at + PLAN_BINS, next);
         std::vector<row_item> wi((size_t)np);
-        for (int64_t x = 0; x < np; ++x) wi[x] = plan[x].it;
+        std::vector<int64_t> place((size_t)np);
+        for (int64_t x = 0; x < np; ++x) {
+            place[x] = next[plan[x].tlog]++;
+            wi[place[x]] = plan[x].it;
+        }
         row_item *d_items;
         PASTIS_WS(d_items, ctx, WS_SPG_BIN, sizeof(row_item) * np + (sizeof(int64_t) + sizeof(int)) * np + 64);
         int64_t *d_cnt = (int64_t *)(d_items + np);
@@ -808,12 +816,10 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
         PASTIS_WS(tmp, ctx, WS_SPG_TMP, sizeof(pastis_cand) * (size_t)(tmp_total + 1));
         PASTIS_CUDA_TRY(cudaMemcpyAsync(d_items, wi.data(), sizeof(row_item) * np, cudaMemcpyHostToDevice, st));
         PASTIS_CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int) * np, st));
-        int64_t x0 = 0;
-        while (x0 < np) {
-            int64_t x1 = x0;
-            while (x1 < np && plan[x1].tlog == plan[x0].tlog) ++x1;
-            const bool sorted = plan[x0].tlog >= SORT_BIN;
-            const int tsize = 1 << (sorted ? plan[x0].tlog - SORT_BIN : plan[x0].tlog);
+        for (int bin = 0; bin < PLAN_BINS; ++bin) {
+            const int64_t x0 = bin_at[bin], x1 = bin_at[bin + 1];
+            const bool sorted = bin >= SORT_BIN;
+            const int tsize = 1 << (sorted ? bin - SORT_BIN : bin);
             const size_t shm = sorted ? (size_t)tsize * 8 : table_bytes(tsize, subs);
             for (int64_t g0 = x0; g0 < x1; g0 += 65535) {
                 const int64_t g1 = std::min<int64_t>(x1, g0 + 65535);
@@ -834,7 +840,6 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
                 PASTIS_LAUNCHED(ctx);
                 prof_end(ctx);
             }
-            x0 = x1;
         }
         std::vector<int64_t> hc((size_t)np);
         std::vector<int> he((size_t)np);
@@ -842,19 +847,18 @@ static pastis_status overlap_impl(pastis_ctx *ctx, const pastis_kmat *A, const p
         PASTIS_CUDA_TRY(cudaMemcpyAsync(he.data(), d_err, sizeof(int) * np, cudaMemcpyDeviceToHost, st));
         PASTIS_CUDA_TRY(cudaStreamSynchronize(st));
         // slices in row order
-        std::vector<int64_t> ord((size_t)np);
-        for (int64_t x = 0; x < np; ++x) {
-            if (he[x]) return PASTIS_ERR_INTERNAL;
-            ord[x] = x;
-        }
-        std::sort(ord.begin(), ord.end(), [&](int64_t a, int64_t b) { return plan[a].order < plan[b].order; });
         std::vector<int64_t> src, dst, cnt;
-        for (int64_t x : ord) {
-            if (hc[x] == 0) continue;
+        src.reserve((size_t)np);
+        dst.reserve((size_t)np);
+        cnt.reserve((size_t)np);
+        for (int64_t x = 0; x < np; ++x) {
+            const int64_t y = place[x];
+            if (he[y]) return PASTIS_ERR_INTERNAL;
+            if (hc[y] == 0) continue;
             src.push_back(plan[x].it.out_off);
             dst.push_back(total);
-            cnt.push_back(hc[x]);
-            total += hc[x];
+            cnt.push_back(hc[y]);
+            total += hc[y];
         }
         PASTIS_WS(result, ctx, WS_SPG_RESULT, sizeof(pastis_cand) * (size_t)(total + 1));
         const int64_t nk = (int64_t)src.size();

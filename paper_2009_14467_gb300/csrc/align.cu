@@ -351,7 +351,11 @@ __device__ bool xd_diag_warp(const uint8_t *q, int A, int qs, const uint8_t *t, 
 // Measured on 2 M exact candidates of 200,000 proteins: first phase 63.8 ms with separate
 // range and limit masks, dead E and F cleared, and the best score reduced in every step,
 // 53.1 ms so; second phase 14.5 ms with one 32-bit word of statistics per cell, 11.9 ms so;
-// 300,000 family-rich pairs with carries throughout 25.8 -> 20.6 ms.
+// 300,000 family-rich pairs with carries throughout 25.8 -> 20.6 ms.  A window that leaves
+// its range is centred to the nearest lane (16 diagonals with four extensions a warp): the
+// 32-bit kernel's share was 4.1 and 1.2 ms with the shift cut towards zero and is 1.9 and
+// 0.9 ms so.  Shifting by single registers as well leaves 1.1 and 0.6 ms there but takes 3.3
+// and 0.6 ms more here.
 // ---------------------------------------------------------------------------------
 constexpr int XD16_NEG = -32512;                 // 0x8100
 constexpr uint32_t XD16_NEG2 = (uint32_t)(XD16_NEG & 0xffff) * 0x10001u;   // 0x81008100
@@ -465,7 +469,10 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
     }
     if (P == 1 && __any_sync(0xffffffffu, move)) {
         if (move) {
-            const int sh = ((kmin + kmax) / 2 - (x.kbase + 64)) / WD;      // whole lanes, centring the range
+            // the range's centre to the nearest whole lane: up to 112 diagonals fit with four
+            // extensions a warp
+            const int by = ((kmin + kmax) >> 1) - (x.kbase + 64) + WD / 2;
+            const int sh = by >= 0 ? by / WD : -((WD - 1 - by) / WD);
             x.kbase += WD * sh;
             if (kmin < x.kbase || kmax > x.kbase + 127) {
                 defer = true;

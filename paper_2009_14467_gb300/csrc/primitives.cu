@@ -388,12 +388,32 @@ __global__ void __launch_bounds__(CP_THREADS) k_fill_col_ptr(const uint32_t *__r
     }
 }
 
+// The same for few codes, a thread each: one binary search of the sorted keys.
+__global__ void k_find_col_ptr(const uint32_t *__restrict__ keys, const uint32_t *__restrict__ keep_off, int64_t n,
+                               int64_t ncodes, uint32_t *__restrict__ col_ptr) {
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c > ncodes) return;
+    int64_t a = 0, b = n;
+    while (a < b) {
+        const int64_t m = (a + b) >> 1;
+        if ((int64_t)keys[m] < c) a = m + 1; else b = m;
+    }
+    col_ptr[c] = keep_off[a];
+}
+
 }  // namespace
 
 pastis_status fill_col_ptr(pastis_ctx *c, const uint32_t *keys, const uint32_t *keep_off, int64_t n, int64_t ncodes,
                            uint32_t *col_ptr) {
     prof_begin(c, "col_ptr");
-    k_fill_col_ptr<<<(unsigned)ceil_div64(ncodes + 1, CP_TILE), CP_THREADS, 0, c->stream>>>(keys, keep_off, n, ncodes,
+    // Too few tiles to fill the SMs (k <= 4), each with a long stretch of keys: one search per
+    // code instead.  7.6 M entries over 24^4 codes: 17 us so, 1,139 us in 41 tiles; over 24^5
+    // codes (972 tiles) the two are close, 168 and 196 us, and from there on the searches
+    // grow with the codes.
+    if (ceil_div64(ncodes + 1, CP_TILE) < 2 * (int64_t)c->sm_count)
+        k_find_col_ptr<<<(unsigned)ceil_div64(ncodes + 1, 256), 256, 0, c->stream>>>(keys, keep_off, n, ncodes, col_ptr);
+    else
+        k_fill_col_ptr<<<(unsigned)ceil_div64(ncodes + 1, CP_TILE), CP_THREADS, 0, c->stream>>>(keys, keep_off, n, ncodes,
                                                                                            col_ptr);
     PASTIS_LAUNCHED(c);
     prof_end(c);

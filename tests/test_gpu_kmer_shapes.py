@@ -1,6 +1,7 @@
 """GPU k-mer matrices against the oracle at the edges of the kernels that build them: the
 windows' tiles (4,096 positions, up to 1,024 sequences each before offsets are read from
-memory), the radix sort's tiles (2,048 items) and the column pointers' (8,192 codes).
+memory), the radix sort's tiles (2,048 items) and the column pointers' (8,192 codes from
+k = 5 on, one search per code below).
 Whole numbers, so equality."""
 import numpy as np
 import pytest
@@ -38,7 +39,7 @@ def _strings(lengths, seed, letters="ACDEFGHIKLMNPQRSTVWY"):
     return ["".join(rng.choice(list(letters), size=n)) for n in lengths]
 
 
-@pytest.mark.parametrize("k", [1, 2, 4])
+@pytest.mark.parametrize("k", [1, 2, 4, 5])
 def test_thousands_of_tiny_sequences(k):
     rng = np.random.default_rng(k)
     _check(_strings(rng.integers(0, 4, 9000), k), k)
@@ -47,13 +48,15 @@ def test_thousands_of_tiny_sequences(k):
 @pytest.mark.parametrize("total", [1, 2, 2047, 2048, 2049, 4095, 4096, 4097, 8191, 8193, 20000])
 def test_tile_edges(total):
     _check(_strings([total], total), 3)
-    _check(_strings([total // 3, 0, total - total // 3, 5], total), 3, )
+    _check(_strings([total // 3, 0, total - total // 3, 5], total), 3)
+    _check(_strings([total], total), 5)
 
 
 @pytest.mark.parametrize("letters", ["A", "*", "A*", "ACDEFGHIKLMNPQRSTVWYBZX*"])
 def test_codes_at_the_ends_of_the_range(letters):
     _check(_strings([700, 3, 0, 1200], 5, letters), 4)
     _check(_strings([700, 3, 0, 1200], 6, letters), 3)
+    _check(_strings([700, 3, 0, 1200], 7, letters), 5)
 
 
 @pytest.mark.parametrize("k,m", [(1, 10), (2, 25), (3, 7), (3, 60), (6, 25)])

@@ -488,6 +488,16 @@ __device__ __forceinline__ void block_bitonic(uint64_t (&v)[E], uint64_t *s) {
     }
 }
 
+// The end of the run of key in the sorted words s[0, n) that starts at i (i when it has
+// none): steps that double, then halve, as most runs are short.
+__device__ __forceinline__ int run_end(const uint64_t *s, int i, int n, int shift, uint64_t key) {
+    int a = i, step = 1;                                  // everything before a is in the run
+    while (a + step <= n && (s[a + step - 1] >> shift) == key) { a += step; step <<= 1; }
+    while ((step >>= 1) > 0)
+        if (a + step <= n && (s[a + step - 1] >> shift) == key) a += step;
+    return a;
+}
+
 template <bool SUBS>
 __global__ void __launch_bounds__(SORT_MAX / SORT_E) k_spgemm_sort(operand F, operand B, const row_item *items, int tbits,
                                                               int32_t min_shared, cursors cur, pastis_cand *tmp_out,
@@ -549,24 +559,14 @@ __global__ void __launch_bounds__(SORT_MAX / SORT_E) k_spgemm_sort(operand F, op
         const int i = i0 + tid;
         bool keep = false;
         uint32_t c0 = 0, c1 = 0;                          // entries of either orientation
-        uint64_t f0 = SEED_NONE, f1 = SEED_NONE, b0 = SEED_NONE, b1 = SEED_NONE;
         uint64_t j = 0;
         if (i < n) {
-            uint64_t w = s[i];
-            j = w >> jshift;
+            j = s[i] >> jshift;
             if (i == 0 || (s[i - 1] >> jshift) != j) {
-                for (int y = i;;) {
-                    if (SUBS && ((w >> (16 + tbits)) & 1ull)) {
-                        if (c1 == 0) b0 = w & tmask; else if (c1 == 1) b1 = w & tmask;
-                        ++c1;
-                    } else {
-                        if (c0 == 0) f0 = w & tmask; else if (c0 == 1) f1 = w & tmask;
-                        ++c0;
-                    }
-                    if (++y >= n) break;
-                    w = s[y];
-                    if ((w >> jshift) != j) break;
-                }
+                const int y = SUBS ? run_end(s, i, n, 16 + tbits, j << 1) : i;
+                const int z = run_end(s, y, n, jshift, j);
+                c0 = SUBS ? (uint32_t)(y - i) : (uint32_t)(z - i);
+                c1 = SUBS ? (uint32_t)(z - y) : 0u;
                 keep = (int64_t)max(c0, c1) >= (int64_t)min_shared;
             }
         }
@@ -587,11 +587,13 @@ __global__ void __launch_bounds__(SORT_MAX / SORT_E) k_spgemm_sort(operand F, op
             rec.count = use_b ? c1 : c0;
             const int64_t rb = use_b ? B.row_ptr[it.i] : F.row_ptr[it.i];
             const uint16_t *lpos = use_b ? B.row_pos : F.row_pos;
+            const int first = use_b ? i + (int)c0 : i;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                const uint64_t w = use_b ? (q ? b1 : b0) : (q ? f1 : f0);
-                rec.qpos[q] = w == SEED_NONE ? (uint16_t)0xFFFF : lpos[rb + (int64_t)(w >> 16)];
-                rec.tpos[q] = w == SEED_NONE ? (uint16_t)0xFFFF : (uint16_t)(w & 0xFFFF);
+                const bool has = q < (int)rec.count;
+                const uint64_t w = has ? s[first + q] & tmask : 0ull;
+                rec.qpos[q] = has ? lpos[rb + (int64_t)(w >> 16)] : (uint16_t)0xFFFF;
+                rec.tpos[q] = has ? (uint16_t)(w & 0xFFFF) : (uint16_t)0xFFFF;
             }
             tmp_out[it.out_off + out_n + before + __popc(b & ((1u << lane) - 1u))] = rec;
         }

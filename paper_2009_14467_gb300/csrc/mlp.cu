@@ -84,7 +84,7 @@ constexpr int TM = 64;                               // rows of a tile
 constexpr int MLP_GROUPS = 2;                        // groups of eight warps, a tile each
 constexpr int LDH = HID + 8, LDX = FEAT + 8;         // row pitches in shared memory
 constexpr int GROUP = 256, MLP_THREADS = MLP_GROUPS * GROUP;
-constexpr int PART = 3 * HID + 2;                    // a CTA's partial sums: g_b1, g_b2, g_w3, g_b3, loss
+constexpr int PART = 3 * HID;                        // a CTA's partial sums: g_b1, g_b2, g_w3
 constexpr size_t MLP_SMEM = sizeof(__nv_bfloat16) * ((size_t)HID * LDH + FEAT * LDH + MLP_GROUPS * (TM * LDH + TM * LDX)) +
                             sizeof(float) * 3 * HID;
 
@@ -161,12 +161,13 @@ struct mlp_train_io {           // training only
     const float *y;
     float pos_weight;
     __nv_bfloat16 *h1, *dh1, *dh2;   // n x 256 each, for the gradients of W1 and W2
+    float *dz, *lrow;           // per row: the gradient at the logit, the loss term
     float *part;                // PART floats per CTA
 };
 
-// z[r] = the logit of row r.  TRAIN: also the weighted logistic loss, dz = w * (sigmoid(z)
-// - y) / n, the gradients dh2 = dz * w3 where layer 2 is active and dh1 = dh2 W2^T where
-// layer 1 is, and the gradients of the biases and W3 as partial sums per CTA (fixed order,
+// z[r] = the logit of row r.  TRAIN: the weighted logistic loss's terms and dz = w *
+// (sigmoid(z) - y) / n instead, the gradients dh2 = dz * w3 where layer 2 is active and dh1 = dh2 W2^T where
+// layer 1 is, and the gradients of W3 and its layers' biases as partial sums per CTA (fixed order,
 // so a training step is deterministic).  Measured on 10^6 rows: 3.99 ms with
 // one 64 x 64 tile and 2-byte loads a CTA and h1, h2 through memory, 0.355 ms so (137 GF:
 // 0.6 of the rate mma.sync reaches alone); a training step of 65,536 rows 28.1 ms with the
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bf
     const float b3 = net.b3[0];
     const uint32_t u_h = smem_u32(s_h), u_w1 = smem_u32(s_w1), u_w2 = smem_u32(s_w2), u_x = smem_u32(s_x);
     // TRAIN: sums kept over the CTA's tiles
-    float gw3[8], gb2[8], gb1[16], gb3 = 0.f, loss = 0.f;
+    float gw3[8], gb2[8], gb1[16];
     if constexpr (TRAIN) {
 #pragma unroll
         for (int t = 0; t < 8; ++t) { gw3[t] = 0.f; gb2[t] = 0.f; }
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bf
 #pragma unroll
             for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
             const float zz = s + b3;
-            if (r0 + row < n && lane == 0) z[r0 + row] = zz;
+            if (!TRAIN && r0 + row < n && lane == 0) z[r0 + row] = zz;
             if constexpr (TRAIN) {
                 float d = 0.f;
                 if (r0 + row < n) {
@@ -292,8 +293,10 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bf
                     const float sg = 1.f / (1.f + __expf(-zz));
                     d = w * (sg - yy) / (float)n;
                     const float sp = zz > 0.f ? zz + log1pf(__expf(-zz)) : log1pf(__expf(zz));
-                    gb3 += d;
-                    loss += w * (sp - yy * zz) / (float)n;
+                    if (lane == 0) {
+                        tr.dz[r0 + row] = d;
+                        tr.lrow[r0 + row] = w * (sp - yy * zz) / (float)n;
+                    }
                 }
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
@@ -364,11 +367,6 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bf
             v += __shfl_xor_sync(0xffffffffu, v, 16);
             if (gid == 0) s_red[(2 * W + group * 2 + mw) * HID + nw * 64 + (t >> 1) * 8 + tig * 2 + (t & 1)] = v;
         }
-        float *s_one = s_red + (2 * W + 2 * MLP_GROUPS) * HID;
-        if (lane == 0) {
-            s_one[aw] = gb3;
-            s_one[W + aw] = loss;
-        }
         __syncthreads();
         if (group == 0) {
             float a = 0.f, b = 0.f, c = 0.f;
@@ -377,11 +375,6 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bf
             part[tid] = c;
             part[HID + tid] = a;
             part[2 * HID + tid] = b;
-            if (tid < 2) {
-                float v = 0.f;
-                for (int w = 0; w < W; ++w) v += s_one[tid * W + w];
-                part[3 * HID + tid] = v;
-            }
         }
     }
 }
@@ -399,15 +392,48 @@ constexpr int WG_PROD = 128, WG_THREADS = WG_PROD + 256;   // four warps of prod
 constexpr int WG_STAGE = 2 * WG_ROWS * LDG;              // bf16 values of a stage
 constexpr size_t WG_SMEM = sizeof(__nv_bfloat16) * WG_STAGES * WG_STAGE;
 
+constexpr int WG_CTAS = 64 + 8 + 1;
+
+// The sums of dz (W3's bias) and of the loss terms over the rows, by the last CTA beside the
+// chains: every 256th row to a thread, then a tree, so their rounding does not depend on
+// the number of SMs.
+__device__ void row_sums(const float *__restrict__ dz, const float *__restrict__ lrow, int64_t n, float *g_b3,
+                         float *loss, float *s) {
+    const int t = threadIdx.x;
+    if (t < 256) {
+        float a = 0.f, b = 0.f;
+#pragma unroll 8
+        for (int64_t r = t; r < n; r += 256) { a += dz[r]; b += lrow[r]; }
+        s[t] = a;
+        s[256 + t] = b;
+    }
+    __syncthreads();
+    for (int d = 128; d > 0; d >>= 1) {
+        if (t < d) { s[t] += s[t + d]; s[256 + t] += s[256 + t + d]; }
+        __syncthreads();
+    }
+    if (t == 0) {
+        *g_b3 = s[0];
+        if (loss) *loss = s[256];
+    }
+}
+
 __global__ void __launch_bounds__(WG_THREADS) k_mlp_wgrad(const __nv_bfloat16 *__restrict__ x,
                                                           const __nv_bfloat16 *__restrict__ h1,
                                                           const __nv_bfloat16 *__restrict__ dh1,
                                                           const __nv_bfloat16 *__restrict__ dh2, int64_t n,
-                                                          float *__restrict__ g_w1, float *__restrict__ g_w2) {
+                                                          const float *__restrict__ dz,
+                                                          const float *__restrict__ lrow, float *__restrict__ g_w1,
+                                                          float *__restrict__ g_w2, float *__restrict__ g_b3,
+                                                          float *__restrict__ loss) {
     extern __shared__ __align__(16) unsigned char mlp_smem[];
     __nv_bfloat16 *s = reinterpret_cast<__nv_bfloat16 *>(mlp_smem);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int mw = (warp >> 1) & 1, nw = warp & 1;       // a product warp's 16 x 16 entries
+    if (blockIdx.x == WG_CTAS - 1) {
+        row_sums(dz, lrow, n, g_b3, loss, reinterpret_cast<float *>(mlp_smem));
+        return;
+    }
     const bool first = blockIdx.x >= 64;                 // W1
     const int i0 = first ? 0 : (blockIdx.x >> 3) * WG_COLS, o0 = (blockIdx.x & 7) * WG_COLS;
     const int stages = (int)((n + WG_ROWS - 1) / WG_ROWS);
@@ -491,13 +517,13 @@ __global__ void __launch_bounds__(WG_THREADS) k_mlp_wgrad(const __nv_bfloat16 *_
                 acc[t][q];
 }
 
-// Every parameter's Adam step on its float32 master, with the gradients of the biases and
-// W3 summed here from the CTAs' partial sums (in order); refreshes the bf16 copies.  The
-// last thread sums the loss.
+// Every parameter's Adam step on its float32 master, with the gradients of W3 and of the
+// biases of layers 1 and 2 summed here from the CTAs' partial sums (in order); refreshes the
+// bf16 copies.
 struct adam_args {
     float *w1, *b1, *w2, *b2, *w3, *b3;
     __nv_bfloat16 *w1b, *w2b, *w3b;
-    float *grad, *m, *v, *loss;
+    float *grad, *m, *v;
     float lr, beta1, beta2, eps, c1, c2;
 };
 
@@ -505,16 +531,15 @@ __global__ void __launch_bounds__(256) k_mlp_adam(adam_args a, const float *__re
     constexpr int NW1 = FEAT * HID, NW2 = HID * HID, O1 = NW1, O2 = O1 + HID, O3 = O2 + NW2, O4 = O3 + HID,
                   O5 = O4 + HID, N = O5 + 1;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x > N || (x == N && !a.loss)) return;
+    if (x >= N) return;
     float g;
-    if (x < O1 || (x >= O2 && x < O3)) {
+    if (x < O1 || (x >= O2 && x < O3) || x == O5) {
         g = a.grad[x];
     } else {
-        const float *p = part + (x < O2 ? x - O1 : x - O3 + HID);     // b1, then b2, w3, b3, loss
+        const float *p = part + (x < O2 ? x - O1 : x - O3 + HID);     // b1, then b2, w3
         g = 0.f;
 #pragma unroll 8
         for (int q = 0; q < n_part; ++q) g += p[q * PART];
-        if (x == N) { *a.loss = g; return; }
         a.grad[x] = g;
     }
     float *w;
@@ -611,38 +636,40 @@ extern "C" pastis_status pastis_mlp_train_step(pastis_ctx *ctx, pastis_mlp *net,
                                                int64_t n, float lr, float pos_weight, float *d_loss) {
     if (!ctx || !net || n <= 0 || n > (1 << 22) || !d_x || !d_y) return PASTIS_ERR_INVALID_ARG;
     cudaStream_t st = ctx->stream;
-    // scratch: h1, dh1 and dh2 (bf16 n x 256), the logits, and the partial sums of the gradients
+    // scratch: h1, dh1 and dh2 (bf16 n x 256), dz and the loss terms, the partial sums of the gradients
     const int grid = (int)std::min<int64_t>(ceil_div64(n, TM), ctx->sm_count);
     const size_t act = (size_t)n * HID * 2, zb = ((size_t)n * 4 + 255) & ~(size_t)255;
     const size_t pb = ((size_t)grid * PART * 4 + 255) & ~(size_t)255;
     char *b;
-    PASTIS_WS(b, ctx, WS_MLP, 3 * act + zb + pb);
+    PASTIS_WS(b, ctx, WS_MLP, 3 * act + 2 * zb + pb);
     mlp_train_io tr;
     tr.y = d_y;
     tr.pos_weight = pos_weight;
     tr.h1 = (__nv_bfloat16 *)b;
     tr.dh1 = (__nv_bfloat16 *)(b + act);
     tr.dh2 = (__nv_bfloat16 *)(b + 2 * act);
-    float *z = (float *)(b + 3 * act);
-    tr.part = (float *)(b + 3 * act + zb);
+    tr.dz = (float *)(b + 3 * act);
+    tr.lrow = (float *)(b + 3 * act + zb);
+    tr.part = (float *)(b + 3 * act + 2 * zb);
     prof_begin(ctx, "mlp_train");
-    k_mlp<true><<<grid, MLP_THREADS, MLP_SMEM, st>>>(mlp_weights(net), (const __nv_bfloat16 *)d_x, n, z, tr);
+    k_mlp<true><<<grid, MLP_THREADS, MLP_SMEM, st>>>(mlp_weights(net), (const __nv_bfloat16 *)d_x, n, nullptr, tr);
     PASTIS_LAUNCHED(ctx);
     prof_end(ctx);
     prof_begin(ctx, "mlp_wgrad");
-    k_mlp_wgrad<<<64 + 8, WG_THREADS, WG_SMEM, st>>>((const __nv_bfloat16 *)d_x, tr.h1, tr.dh1, tr.dh2, n, net->grad,
-                                                    net->grad + FEAT * HID + HID);
+    k_mlp_wgrad<<<WG_CTAS, WG_THREADS, WG_SMEM, st>>>((const __nv_bfloat16 *)d_x, tr.h1, tr.dh1, tr.dh2, n, tr.dz,
+                                                     tr.lrow, net->grad, net->grad + FEAT * HID + HID,
+                                                     net->grad + FEAT * HID + HID * HID + 3 * HID, d_loss);
     PASTIS_LAUNCHED(ctx);
     prof_end(ctx);
     net->step += 1;
     adam_args a;
     a.w1 = net->w1; a.b1 = net->b1; a.w2 = net->w2; a.b2 = net->b2; a.w3 = net->w3; a.b3 = net->b3;
     a.w1b = (__nv_bfloat16 *)net->w1b; a.w2b = (__nv_bfloat16 *)net->w2b; a.w3b = (__nv_bfloat16 *)net->w3b;
-    a.grad = net->grad; a.m = net->adam_m; a.v = net->adam_v; a.loss = d_loss;
+    a.grad = net->grad; a.m = net->adam_m; a.v = net->adam_v;
     a.lr = lr; a.beta1 = 0.9f; a.beta2 = 0.999f; a.eps = 1e-8f;
     a.c1 = 1.f - powf(a.beta1, (float)net->step);
     a.c2 = 1.f - powf(a.beta2, (float)net->step);
-    const int np = FEAT * HID + HID * HID + 3 * HID + 2;
+    const int np = FEAT * HID + HID * HID + 3 * HID + 1;
     prof_begin(ctx, "mlp_adam");
     k_mlp_adam<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(a, tr.part, grid);
     PASTIS_LAUNCHED(ctx);

@@ -171,9 +171,8 @@ int32_t pastis_ctx_profile_read(pastis_ctx *ctx, char *buf, int32_t len);
 /* Work counters accumulated while profiling is on (cleared when it is enabled), for the
  * roofline of the overlap product: h_out[0] = posting entries visited (products),
  * [1] = left-operand entries of the rows formed (each once per row; of A S those kept: the
- * substitutes that A holds), [2] = candidate
- * records written, [3] = radix-sort element passes of the k-mer matrix builds (A and AS:
- * elements sorted x 8-bit digit passes).  Entries past the fourth are 0.  Synchronises
+ * substitutes that A holds), [2] = candidate records written, [3] = radix-sort element
+ * passes of the k-mer matrix builds (A and AS: elements sorted x 8-bit digit passes).  Entries past the fourth are 0.  Synchronises
  * the stream.                                                                             */
 #define PASTIS_STATS 4
 pastis_status pastis_ctx_stats(pastis_ctx *ctx, int64_t *h_out, int32_t n);
@@ -307,12 +306,13 @@ pastis_status pastis_align_pairs_qt(pastis_ctx *ctx, const uint8_t *d_qcodes, co
                                     const pastis_params *params, pastis_aln *d_out, int64_t *d_cells);
 
 /* ---- batching: the Smith-Waterman tile layout and its tuner -----------------------
- * Pass 1 of PASTIS_SW / PASTIS_SW_SCORE computes a query of m residues in stripes of
- * 32 lanes x LR rows (LR 2..16), two pairs per warp in the 16-bit halves of every
- * register.  By default it takes as few stripes as 16 rows per lane allow; a layout
- * sets, per query-length bin (bin = (m-1) / 32, the last bin taking every longer
- * query), either 0..PASTIS_SW_MAX_EXTRA extra stripes, which pad fewer rows but sweep
- * the target more often, or PASTIS_SW_INT32: the bin's pairs take one pair per warp in
+ * Pass 1 of PASTIS_SW / PASTIS_SW_SCORE computes a query of m residues on groups of 8, 16
+ * or 32 lanes with 2 to 32 rows a lane (an even number), two pairs per group in the
+ * 16-bit halves of every register: by default the lanes and rows that cost least, and
+ * stripes of 1,024 rows for a longer query.  A layout sets, per query-length bin
+ * (bin = (m-1) / 32, the last bin taking every longer query), either
+ * 0..PASTIS_SW_MAX_EXTRA stripes more than a query needs, of 32 lanes, which pad fewer
+ * rows but sweep the target more often, or PASTIS_SW_INT32: the bin's pairs take one pair per warp in
  * 32-bit lanes (the whole-matrix path that also serves pairs whose scores could
  * overflow 16 bits).  The layout is a speed choice only: every output of every entry
  * point is the same under every layout.                                             */

@@ -1,5 +1,5 @@
 // Device primitives used by the k-mer and candidate stages: a reduce-then-scan exclusive
-// prefix sum and a stable LSD radix sort (8-bit digits) of (uint32 key, uint64 value).
+// prefix sum and a stable LSD radix sort (digits of 5 to 8 bits) of (uint32 key, uint64 value).
 #include "internal.cuh"
 
 namespace {
@@ -128,7 +128,7 @@ pastis_status exclusive_scan_i64(pastis_ctx *c, const int64_t *in, int64_t *out,
 }
 
 // ---------------------------------------------------------------------------------
-// Stable LSD radix sort.  Per 8-bit digit: a tile histogram, a scan of the
+// Stable LSD radix sort.  Per digit: a tile histogram, a scan of the
 // (digit, tile) counts in digit-major order, then a scatter in which every warp ranks
 // its items in input order, so equal digits keep input order.
 // ---------------------------------------------------------------------------------
@@ -139,43 +139,49 @@ constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_ITEMS = 8;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;   // each warp owns 256 consecutive items
 
+template <int BITS>
 __global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint32_t *keys, int64_t n, int shift,
                                                         uint32_t *hist, int64_t nb) {
-    __shared__ uint32_t s_h[256];
-    s_h[threadIdx.x] = 0;
+    constexpr uint32_t D = 1u << BITS;
+    __shared__ uint32_t s_h[D];
+    if (threadIdx.x < D) s_h[threadIdx.x] = 0;
     __syncthreads();
     int64_t base = (int64_t)blockIdx.x * RS_TILE;
 #pragma unroll 4
     for (int it = 0; it < RS_ITEMS; ++it) {
         int64_t x = base + (int64_t)it * RS_THREADS + threadIdx.x;
-        if (x < n) atomicAdd(&s_h[(keys[x] >> shift) & 255u], 1u);
+        if (x < n) atomicAdd(&s_h[(keys[x] >> shift) & (D - 1)], 1u);
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * nb + blockIdx.x] = s_h[threadIdx.x];
+    if (threadIdx.x < D) hist[(int64_t)threadIdx.x * nb + blockIdx.x] = s_h[threadIdx.x];
 }
 
 // The tile's items are first placed in shared memory in their sorted order (digit, then
 // input order), then written out in that order, so consecutive threads write
 // consecutive positions of each digit's run in the output.  The ranks of the first sweep
-// are kept, so each item's peers are found once, by eight ballots.  Seven passes over the
-// 35 M windows of 100,000 proteins: 3.10 ms with __match_any_sync in two sweeps and 16 items
-// a thread, 1.64 ms so (3.6 TB/s).
-constexpr size_t RS_SCATTER_SMEM = sizeof(uint64_t) * RS_TILE + sizeof(uint32_t) * RS_TILE +
-                                   sizeof(uint32_t) * (2 * RS_WARPS * 256 + 2 * 256 + RS_WARPS);
+// are kept, so each item's peers are found once, by a ballot per bit of the digit.  Seven
+// passes over the 35 M windows of 100,000 proteins: 3.10 ms with __match_any_sync in two sweeps
+// and 16 items a thread, 1.64 ms so, 1.53 ms (3.9 TB/s) in digits of 7 and 6 bits.
+constexpr size_t rs_scatter_smem(int bits) {
+    return sizeof(uint64_t) * RS_TILE + sizeof(uint32_t) * RS_TILE +
+           sizeof(uint32_t) * ((size_t)2 * (RS_WARPS + 1) * ((size_t)1 << bits) + RS_WARPS);
+}
 
+template <int BITS>
 __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t *keys, const uint64_t *vals,
                                                            int64_t n, int shift, const uint32_t *offs,
                                                            int64_t nb, uint32_t *okeys, uint64_t *ovals) {
+    constexpr uint32_t D = 1u << BITS;
     extern __shared__ __align__(16) unsigned char rs_smem[];
     uint64_t *s_v = reinterpret_cast<uint64_t *>(rs_smem);
     uint32_t *s_k = reinterpret_cast<uint32_t *>(s_v + RS_TILE);
     uint32_t *s_cnt = s_k + RS_TILE;                 // [warp][digit]: counts
-    uint32_t *s_base = s_cnt + RS_WARPS * 256;       // [warp][digit]: start within the digit's run
-    uint32_t *s_tstart = s_base + RS_WARPS * 256;    // [digit]: start of the digit's run in the tile
-    uint32_t *s_gbase = s_tstart + 256;              // [digit]: its start in the output
-    uint32_t *s_wsum = s_gbase + 256;                // [warp]: scan carries
+    uint32_t *s_base = s_cnt + RS_WARPS * D;       // [warp][digit]: start within the digit's run
+    uint32_t *s_tstart = s_base + RS_WARPS * D;    // [digit]: start of the digit's run in the tile
+    uint32_t *s_gbase = s_tstart + D;              // [digit]: its start in the output
+    uint32_t *s_wsum = s_gbase + D;                // [warp]: scan carries
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int d = threadIdx.x; d < 256 * RS_WARPS; d += RS_THREADS) s_cnt[d] = 0;
+    for (int d = threadIdx.x; d < (int)D * RS_WARPS; d += RS_THREADS) s_cnt[d] = 0;
     __syncthreads();
     const int64_t tile0 = (int64_t)blockIdx.x * RS_TILE;
     const int64_t base = tile0 + (int64_t)warp * (RS_ITEMS * 32);
@@ -195,17 +201,17 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t *keys,
 #pragma unroll
     for (int it = 0; it < RS_ITEMS; ++it) {
         const bool ok = base + it * 32 + lane < n;
-        const uint32_t d = ok ? ((k[it] >> shift) & 255u) : 256u;
+        const uint32_t d = ok ? ((k[it] >> shift) & (D - 1)) : 0u;
         unsigned peers = __ballot_sync(0xffffffffu, ok);      // lanes with the same digit, by its bits
         peers = ok ? peers : 0u;
 #pragma unroll
-        for (int bit = 0; bit < 8; ++bit) {
+        for (int bit = 0; bit < BITS; ++bit) {
             const unsigned set = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
             peers &= ((d >> bit) & 1u) ? set : ~set;
         }
-        const uint32_t before = ok ? s_cnt[warp * 256 + d] : 0u;
+        const uint32_t before = ok ? s_cnt[warp * D + d] : 0u;
         __syncwarp();
-        if (ok && lane == __ffs(peers) - 1) s_cnt[warp * 256 + d] = before + __popc(peers);
+        if (ok && lane == __ffs(peers) - 1) s_cnt[warp * D + d] = before + __popc(peers);
         __syncwarp();
         const uint32_t r = before + __popc(peers & lt_mask);
         rank[it >> 1] = (it & 1) ? rank[it >> 1] | (r << 16) : r;
@@ -213,12 +219,13 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t *keys,
     __syncthreads();
     // per digit: the warps' starts within its run, its total, and the runs' starts in the
     // tile (an exclusive scan over the digits)
-    const int d0 = threadIdx.x;                      // RS_THREADS == 256 digits
+    const int d0 = threadIdx.x;                      // at most RS_THREADS digits
     uint32_t tot = 0;
-    for (int w = 0; w < RS_WARPS; ++w) {
-        s_base[w * 256 + d0] = tot;
-        tot += s_cnt[w * 256 + d0];
-    }
+    if (d0 < (int)D)
+        for (int w = 0; w < RS_WARPS; ++w) {
+            s_base[w * D + d0] = tot;
+            tot += s_cnt[w * D + d0];
+        }
     uint32_t incl = tot;
 #pragma unroll
     for (int x = 1; x < 32; x <<= 1) {
@@ -226,18 +233,18 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t *keys,
         if (lane >= x) incl += y;
     }
     if (lane == 31) s_wsum[warp] = incl;
-    s_gbase[d0] = offs[(int64_t)d0 * nb + blockIdx.x];
+    if (d0 < (int)D) s_gbase[d0] = offs[(int64_t)d0 * nb + blockIdx.x];
     __syncthreads();
     uint32_t wpre = 0;
     for (int w = 0; w < warp; ++w) wpre += s_wsum[w];
-    s_tstart[d0] = wpre + incl - tot;
+    if (d0 < (int)D) s_tstart[d0] = wpre + incl - tot;
     __syncthreads();
     // each item to its place in the tile's sorted order
 #pragma unroll
     for (int it = 0; it < RS_ITEMS; ++it) {
         if (base + it * 32 + lane < n) {
-            const uint32_t d = (k[it] >> shift) & 255u;
-            const uint32_t lp = s_tstart[d] + s_base[warp * 256 + d] + ((rank[it >> 1] >> (16 * (it & 1))) & 0xFFFFu);
+            const uint32_t d = (k[it] >> shift) & (D - 1);
+            const uint32_t lp = s_tstart[d] + s_base[warp * D + d] + ((rank[it >> 1] >> (16 * (it & 1))) & 0xFFFFu);
             s_k[lp] = k[it];
             s_v[lp] = v[it];
         }
@@ -247,15 +254,36 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t *keys,
     const int tile_n = (int)min((int64_t)RS_TILE, n - tile0);
     for (int x = threadIdx.x; x < tile_n; x += RS_THREADS) {
         const uint32_t key = s_k[x];
-        const uint32_t d = (key >> shift) & 255u;
+        const uint32_t d = (key >> shift) & (D - 1);
         const uint32_t pos = s_gbase[d] + ((uint32_t)x - s_tstart[d]);
         okeys[pos] = key;
         ovals[pos] = s_v[x];
     }
 }
 
+template <int BITS>
+pastis_status rs_pass(pastis_ctx *c, const uint32_t *ik, const uint64_t *iv, int64_t n, int shift, uint32_t *hist,
+                      uint32_t *offs, int64_t nb, uint32_t *ok, uint64_t *ov) {
+    prof_begin(c, "radix_hist");
+    k_rs_hist<BITS><<<(unsigned)nb, RS_THREADS, 0, c->stream>>>(ik, n, shift, hist, nb);
+    PASTIS_LAUNCHED(c);
+    prof_end(c);
+    pastis_status st = exclusive_scan_u32(c, hist, offs, nb << BITS);
+    if (st != PASTIS_OK) return st;
+    prof_begin(c, "radix_scatter");
+    k_rs_scatter<BITS><<<(unsigned)nb, RS_THREADS, rs_scatter_smem(BITS), c->stream>>>(ik, iv, n, shift, offs, nb, ok,
+                                                                                      ov);
+    PASTIS_LAUNCHED(c);
+    prof_end(c);
+    return PASTIS_OK;
+}
+
 }  // namespace
 
+// Keys below 2^key_bits.  As many passes as 8-bit digits need, of digits as equal as they
+// come (28 bits: four of 7, not three of 8 and one of 4): fewer ballots and counters, and
+// longer runs in each tile's writes.  The seven passes over 35 M windows (28 bits, then the 17 of
+// the sequences) with their counts and scans: 2.53 ms in digits of 8 bits, 2.23 ms so.
 pastis_status radix_sort_u32_u64(pastis_ctx *c, uint32_t *keys, uint64_t *vals, uint32_t *keys_alt,
                                  uint64_t *vals_alt, int64_t n, int key_bits, uint32_t **keys_out,
                                  uint64_t **vals_out) {
@@ -270,17 +298,11 @@ pastis_status radix_sort_u32_u64(pastis_ctx *c, uint32_t *keys, uint64_t *vals, 
     uint32_t *ik = keys, *ok = keys_alt;
     uint64_t *iv = vals, *ov = vals_alt;
     if (c->prof_on) c->sort_passes += n * (int64_t)((key_bits + 7) / 8);
-    for (int shift = 0; shift < key_bits; shift += 8) {
-        prof_begin(c, "radix_hist");
-        k_rs_hist<<<(unsigned)nb, RS_THREADS, 0, c->stream>>>(ik, n, shift, hist, nb);
-        PASTIS_LAUNCHED(c);
-        prof_end(c);
-        pastis_status st = exclusive_scan_u32(c, hist, offs, 256 * nb);
+    const int passes = (key_bits + 7) / 8, bits = std::max(5, (key_bits + passes - 1) / passes);
+    for (int x = 0; x < passes; ++x) {
+        auto pass = bits == 5 ? rs_pass<5> : bits == 6 ? rs_pass<6> : bits == 7 ? rs_pass<7> : rs_pass<8>;
+        pastis_status st = pass(c, ik, iv, n, x * bits, hist, offs, nb, ok, ov);
         if (st != PASTIS_OK) return st;
-        prof_begin(c, "radix_scatter");
-        k_rs_scatter<<<(unsigned)nb, RS_THREADS, RS_SCATTER_SMEM, c->stream>>>(ik, iv, n, shift, offs, nb, ok, ov);
-        PASTIS_LAUNCHED(c);
-        prof_end(c);
         uint32_t *tk = ik; ik = ok; ok = tk;
         uint64_t *tv = iv; iv = ov; ov = tv;
     }
@@ -421,5 +443,5 @@ pastis_status fill_col_ptr(pastis_ctx *c, const uint32_t *keys, const uint32_t *
 }
 
 cudaError_t radix_set_smem_limit() {
-    return cudaFuncSetAttribute(k_rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SCATTER_SMEM);
+    return cudaFuncSetAttribute(k_rs_scatter<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs_scatter_smem(8));
 }

@@ -171,7 +171,7 @@ struct mlp_train_io {           // training only
 // so a training step is deterministic).  Measured on 10^6 rows: 3.99 ms with
 // one 64 x 64 tile and 2-byte loads a CTA and h1, h2 through memory, 0.355 ms so (137 GF:
 // 0.6 of the rate mma.sync reaches alone); a training step of 65,536 rows 28.1 ms with the
-// column sums in one CTA each, 0.39 ms so.
+// column sums in one CTA each, 0.35 ms so.
 template <bool TRAIN>
 __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bfloat16 *__restrict__ x, int64_t n,
                                                         float *__restrict__ z, mlp_train_io tr) {
@@ -380,14 +380,16 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bf
 }
 
 // The gradients of W2 (h1^T dh2) and W1 (x^T dh1): every entry is one chain of mma.sync over
-// the rows, 16 at a time in order, so what bounds it is the latency of 65,536 / 16
-// dependent products; the chains run side by side, 32 inputs x 32 outputs a CTA (two
-// chains a warp), 64 CTAs for W2 and 8 for W1, each reading only its columns through a
-// ring of cp.async stages.  Tiles of 64 x 64 with 2-byte loads took 16.8 ms of a 65,536-row
-// step, 0.23 ms so; chains split over the rows and added up would be faster still, but the
-// sums would differ from these by more than a re-ordering (3e-4: the tensor core truncates
-// what it aligns to a long chain's accumulator).
-constexpr int WG_ROWS = 64, WG_STAGES = 6, WG_COLS = 32, LDG = WG_COLS + 8;
+// the rows, 16 at a time in order, so what bounds it is the time of a step through the
+// 4,096 of a 65,536-row batch: the fragments of a stage are read from the ring of cp.async stages
+// while the products of the one before run.  The chains run side by side, 32 inputs x 32
+// outputs a CTA (two chains a warp), 64 CTAs for W2 and 8 for W1, each reading only its
+// columns.  Tiles of 64 x 64 with 2-byte loads took 16.8 ms of a 65,536-row step, 0.23 ms with
+// read and product one after the other, 0.197 ms so (stages of 128 rows 0.210, rings of 5, 14
+// and 20 stages 0.266, 0.208 and 0.208); chains split over the rows and added up would be
+// faster still, but the sums would differ from these by more than a re-ordering (3e-4: the
+// tensor core truncates what it aligns to a long chain's accumulator).
+constexpr int WG_ROWS = 64, WG_STAGES = 8, WG_COLS = 32, LDG = WG_COLS + 8;
 constexpr int WG_PROD = 128, WG_THREADS = WG_PROD + 256;   // four warps of products, then eight that fetch
 constexpr int WG_STAGE = 2 * WG_ROWS * LDG;              // bf16 values of a stage
 constexpr size_t WG_SMEM = sizeof(__nv_bfloat16) * WG_STAGES * WG_STAGE;
@@ -418,7 +420,7 @@ __device__ void row_sums(const float *__restrict__ dz, const float *__restrict__
     }
 }
 
-__global__ void __launch_bounds__(WG_THREADS) k_mlp_wgrad(const __nv_bfloat16 *__restrict__ x,
+__global__ void __launch_bounds__(WG_THREADS, 1) k_mlp_wgrad(const __nv_bfloat16 *__restrict__ x,
                                                           const __nv_bfloat16 *__restrict__ h1,
                                                           const __nv_bfloat16 *__restrict__ dh1,
                                                           const __nv_bfloat16 *__restrict__ dh2, int64_t n,
@@ -451,21 +453,20 @@ __global__ void __launch_bounds__(WG_THREADS) k_mlp_wgrad(const __nv_bfloat16 *_
         int left = (int)n - row0;                        // rows from this thread's next one on
         int put = 0;                                     // ring slot of the next fetch
         auto fetch = [&]() {
-            if (left > 0 && mine) {
+            if (mine) {
                 __nv_bfloat16 *d = dst + put * WG_STAGE;
                 const uint32_t d32 = smem_u32(d);
-                if (aligned && left > 32) {
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d32), "l"(src));
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d32 + 32 * LDG * 2), "l"(src + 32 * ld));
-                } else {
-                    *reinterpret_cast<uint4 *>(d) = load8(src, aligned);
-                    *reinterpret_cast<uint4 *>(d + 32 * LDG) =
-                        left > 32 ? load8(src + 32 * ld, aligned) : make_uint4(0u, 0u, 0u, 0u);
+                if (aligned && left > WG_ROWS - 32) {
+#pragma unroll
+                    for (int u = 0; u < WG_ROWS / 32; ++u)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d32 + u * 32 * LDG * 2),
+                                     "l"(src + u * 32 * ld));
+                } else {                                 // rows past the batch are zero
+#pragma unroll
+                    for (int u = 0; u < WG_ROWS / 32; ++u)
+                        *reinterpret_cast<uint4 *>(d + u * 32 * LDG) =
+                            left > u * 32 ? load8(src + u * 32 * ld, aligned) : make_uint4(0u, 0u, 0u, 0u);
                 }
-            } else if (mine) {                           // rows past the batch are zero
-                __nv_bfloat16 *d = dst + put * WG_STAGE;
-                *reinterpret_cast<uint4 *>(d) = make_uint4(0u, 0u, 0u, 0u);
-                *reinterpret_cast<uint4 *>(d + 32 * LDG) = make_uint4(0u, 0u, 0u, 0u);
             }
             src += (int64_t)WG_ROWS * ld;
             left -= WG_ROWS;
@@ -473,10 +474,10 @@ __global__ void __launch_bounds__(WG_THREADS) k_mlp_wgrad(const __nv_bfloat16 *_
             asm volatile("cp.async.commit_group;");
         };
 #pragma unroll
-        for (int st = 0; st < WG_STAGES - 1; ++st) fetch();
+        for (int st = 0; st < WG_STAGES - 2; ++st) fetch();
         for (int st = 0; st < stages; ++st) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(WG_STAGES - 2));
-            __syncthreads();                             // stage st is here, and stage st - 1 is read
+            asm volatile("cp.async.wait_group %0;" ::"n"(WG_STAGES - 3));
+            __syncthreads();                             // stage st is here, and stage st - 2 is used
             fetch();
         }
         asm volatile("cp.async.wait_group 0;");
@@ -486,26 +487,44 @@ __global__ void __launch_bounds__(WG_THREADS) k_mlp_wgrad(const __nv_bfloat16 *_
     const uint32_t a_at = smem_u32(s) + (uint32_t)((((lane & 7) + (q >> 1) * 8) * LDG + mw * 16 + (q & 1) * 8) * 2);
     const uint32_t b_at = smem_u32(s) + (uint32_t)((WG_ROWS * LDG + (lane & 15) * LDG + nw * 16 + (lane >> 4) * 8) * 2);
     uint32_t at = 0;                                     // byte offset of the stage in the ring
-    int rows = (int)n;                                   // rows from this stage on
-    for (int st = 0; st < stages; ++st) {
+    int rows = (int)n;                                   // rows from the stage to multiply on
+    const bool works = !(first && mw == 1);              // W1 has 16 inputs
+    // the fragments of a stage are read while the products of the one before run
+    uint32_t fa[2][WG_ROWS / 16][4], fb[2][WG_ROWS / 16][4];
+    auto read = [&](uint32_t (&a)[WG_ROWS / 16][4], uint32_t (&b)[WG_ROWS / 16][4]) {
         __syncthreads();
-        if (!(first && mw == 1)) {                       // W1 has 16 inputs
-            uint32_t a[WG_ROWS / 16][4], b[WG_ROWS / 16][4];
+        if (works)
 #pragma unroll
             for (int k = 0; k < WG_ROWS / 16; ++k) {
                 ldsm4t(a[k], a_at + at + k * 16 * LDG * 2);
                 ldsm4t(b[k], b_at + at + k * 16 * LDG * 2);
             }
+        at = at + WG_STAGE * 2 == WG_STAGES * WG_STAGE * 2 ? 0u : at + WG_STAGE * 2;
+    };
+    auto multiply = [&](uint32_t (&a)[WG_ROWS / 16][4], uint32_t (&b)[WG_ROWS / 16][4]) {
+        if (works)
 #pragma unroll
-            for (int k = 0; k < WG_ROWS / 16; ++k) {
+            for (int k = 0; k < WG_ROWS / 16; ++k)
                 if (k * 16 < rows) {
                     mma16816(acc[0], a[k], b[k][0], b[k][1]);
                     mma16816(acc[1], a[k], b[k][2], b[k][3]);
                 }
-            }
-        }
         rows -= WG_ROWS;
-        at = at + WG_STAGE * 2 == WG_STAGES * WG_STAGE * 2 ? 0u : at + WG_STAGE * 2;
+    };
+    read(fa[0], fb[0]);
+    int st = 1;
+    for (; st + 1 < stages; st += 2) {
+        read(fa[1], fb[1]);
+        multiply(fa[0], fb[0]);
+        read(fa[0], fb[0]);
+        multiply(fa[1], fb[1]);
+    }
+    if (st < stages) {
+        read(fa[1], fb[1]);
+        multiply(fa[0], fb[0]);
+        multiply(fa[1], fb[1]);
+    } else {
+        multiply(fa[0], fb[0]);
     }
     if (first && mw == 1) return;
     float *out = first ? g_w1 : g_w2;

@@ -428,11 +428,11 @@ __global__ void k_find_col_ptr(const uint32_t *__restrict__ keys, const uint32_t
 pastis_status fill_col_ptr(pastis_ctx *c, const uint32_t *keys, const uint32_t *keep_off, int64_t n, int64_t ncodes,
                            uint32_t *col_ptr) {
     prof_begin(c, "col_ptr");
-    // Too few tiles to fill the SMs (k <= 4), each with a long stretch of keys: one search per
-    // code instead.  7.6 M entries over 24^4 codes: 17 us so, 1,139 us in 41 tiles; over 24^5
-    // codes (972 tiles) the two are close, 168 and 196 us, and from there on the searches
-    // grow with the codes.
-    if (ceil_div64(ncodes + 1, CP_TILE) < 2 * (int64_t)c->sm_count)
+    // Too few tiles to fill the SMs (k <= 4), or more entries than codes, so that a tile has a
+    // long stretch of keys: one search per code instead.  7.6 M entries over 24^4 codes: 17 us
+    // so, 1,139 us in 41 tiles; over the 8 M codes of k = 5 the searches take 188 us with 20 M
+    // entries, the tiles 433, and with 7.6 M (tiles) 168 and 196.
+    if (n > ncodes || ceil_div64(ncodes + 1, CP_TILE) < 2 * (int64_t)c->sm_count)
         k_find_col_ptr<<<(unsigned)ceil_div64(ncodes + 1, 256), 256, 0, c->stream>>>(keys, keep_off, n, ncodes, col_ptr);
     else
         k_fill_col_ptr<<<(unsigned)ceil_div64(ncodes + 1, CP_TILE), CP_THREADS, 0, c->stream>>>(keys, keep_off, n, ncodes,

@@ -268,10 +268,14 @@ __device__ __forceinline__ uint32_t column2(const uint8_t *__restrict__ pa, cons
 // row; a later column of the same row never replaces an earlier one), then the group's:
 // its best and the first lane holding it.  Returns the value a cell of this lane must
 // exceed to matter: the group's best for the lanes behind the holder, whose rows are
-// larger, one less for the holder and the lanes before it.
+// larger, one less for the holder and the lanes before it, and never less than `none`, what
+// a cell of H = 0 holds.  (A half without a pair has no other cells: one less than those,
+// every later column called for this function, and the last grab of a run of 17 or 18 pairs took
+// a third longer: 10^6 cells a ms 990 at 60 residues and 18 pairs a query, 1,395 so; 1,623 and
+// 2,138 at 120.)
 template <int G, int LR, bool HI>
 __device__ __forceinline__ int note_best(const uint32_t (&Ho)[LR], bool mine, int row0, int j, int lg, uint32_t sh16,
-                                         int &bv, int &brow, int &bcol) {
+                                         int none, int &bv, int &brow, int &bcol) {
     int kk = (int)0x80000000;
 #pragma unroll
     for (int r = 0; r < LR; ++r) {
@@ -283,7 +287,7 @@ __device__ __forceinline__ int note_best(const uint32_t (&Ho)[LR], bool mine, in
     int gk = bv * 64 + (63 - lg);
     for (int d = G >> 1; d > 0; d >>= 1) gk = max(gk, __shfl_xor_sync(0xffffffffu, gk, d));
     const int holder = 63 - (gk & 63);
-    return (gk >> 6) - (lg > holder ? 0 : 1);
+    return max((gk >> 6) - (lg > holder ? 0 : 1), none);
 }
 
 // One group's two pairs in pass 1: targets, columns and the outputs.
@@ -374,11 +378,12 @@ __device__ __noinline__ void score_group(const uint8_t *__restrict__ prof, const
                 const uint32_t over = cm ^ tm;
                 if (__builtin_expect(__any_sync(0xffffffffu, over != 0u), 0)) {
                     if (__any_sync(0xffffffffu, (over & 0xFFFFu) != 0u)) {
-                        const int t = note_best<G, LR, false>(Ho, (over & 0xFFFFu) != 0u, row0, j, lg, sh16, vA, iA, jA);
+                        const int t = note_best<G, LR, false>(Ho, (over & 0xFFFFu) != 0u, row0, j, lg, sh16, -o, vA, iA,
+                                                              jA);
                         tm = (tm & 0xFFFF0000u) | ((uint32_t)t & 0xFFFFu);
                     }
                     if (__any_sync(0xffffffffu, (over >> 16) != 0u)) {
-                        const int t = note_best<G, LR, true>(Ho, (over >> 16) != 0u, row0, j, lg, sh16, vB, iB, jB);
+                        const int t = note_best<G, LR, true>(Ho, (over >> 16) != 0u, row0, j, lg, sh16, -o, vB, iB, jB);
                         tm = (tm & 0xFFFFu) | ((uint32_t)t << 16);
                     }
                 }

@@ -5,26 +5,36 @@
 
 #include "internal.cuh"
 
+static void ws_free(pastis_ctx *c, int s) {
+    cudaStreamSynchronize(c->stream);
+    cudaFree(c->ws[s]);
+    c->ws[s] = nullptr;
+    c->ws_bytes[s] = 0;
+}
+
 void *ws_get(pastis_ctx *c, int s, size_t bytes) {
     if (bytes == 0) bytes = 16;
     if (c->ws_bytes[s] >= bytes) return c->ws[s];
-    if (c->ws[s]) {
-        cudaStreamSynchronize(c->stream);
-        cudaFree(c->ws[s]);
-        c->ws[s] = nullptr;
-        c->ws_bytes[s] = 0;
+    if (c->ws[s]) ws_free(c, s);
+    for (;;) {
+        size_t grow = bytes + bytes / 8;        // headroom against repeated regrowth
+        grow = (grow + 255) & ~(size_t)255;
+        void *p = nullptr;
+        if (cudaMalloc(&p, grow) != cudaSuccess) {
+            cudaGetLastError();
+            if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); p = nullptr; }
+            grow = bytes;
+        }
+        if (p) {
+            c->ws[s] = p;
+            c->ws_bytes[s] = grow;
+            return p;
+        }
+        // the bands are optional and taken last in the call that uses them: what an earlier
+        // call left there goes to a buffer that has to be had
+        if (s == WS_ALN_BAND || !c->ws[WS_ALN_BAND]) return nullptr;
+        ws_free(c, WS_ALN_BAND);
     }
-    size_t grow = bytes + bytes / 8;            // headroom against repeated regrowth
-    grow = (grow + 255) & ~(size_t)255;
-    void *p = nullptr;
-    if (cudaMalloc(&p, grow) != cudaSuccess) {
-        cudaGetLastError();
-        if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-        grow = bytes;
-    }
-    c->ws[s] = p;
-    c->ws_bytes[s] = grow;
-    return p;
 }
 
 extern "C" pastis_status pastis_ctx_create(pastis_ctx **ctx, int device, void *stream) {

@@ -1497,16 +1497,6 @@ pastis_status sw_align(pastis_ctx *ctx, const uint8_t *d_qcodes, const int64_t *
     }
     int16_t *bm_all;
     PASTIS_WS(bm_all, ctx, WS_ALN_BOUND, sizeof(int16_t) * (size_t)h_bm + 16);
-    // pass 2's column ranges per 8 rows; without room for them pass 3 takes the rectangles
-    uint32_t *band = nullptr;
-    if (p->mode != PASTIS_SW_SCORE) {
-        const size_t bytes = sizeof(uint32_t) * ((size_t)(h_bm >> 2) + (size_t)n_pairs + 2);
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (dn) PASTIS_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
-        // a capture allocates nothing: what its sizing run could not have, it goes without
-        if (cap == cudaStreamCaptureStatusNone || ctx->ws_bytes[WS_ALN_BAND] >= bytes)
-            band = (uint32_t *)ws_get(ctx, WS_ALN_BAND, bytes);
-    }
     uint32_t *list = (uint32_t *)bm_cnt;       // the counts have served: two lists of pairs
 
     sw_score_out *res;
@@ -1531,6 +1521,18 @@ pastis_status sw_align(pastis_ctx *ctx, const uint8_t *d_qcodes, const int64_t *
     const size_t scr3 = sizeof(stripe3_cell) * (size_t)blocks3 * SW_WARPS * 2 * sstride;
     void *scratch;
     PASTIS_WS(scratch, ctx, WS_ALN_SCRATCH, std::max(scr1, scr3));
+    // pass 2's column ranges per 8 rows; without room for them pass 3 takes the rectangles.
+    // Taken last, so that they never have the room that a buffer needed above would take
+    // (ws_get gives them up where a later call needs it).
+    uint32_t *band = nullptr;
+    if (p->mode != PASTIS_SW_SCORE) {
+        const size_t bytes = sizeof(uint32_t) * ((size_t)(h_bm >> 2) + (size_t)n_pairs + 2);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (dn) PASTIS_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+        // a capture allocates nothing: what its sizing run could not have, it goes without
+        if (cap == cudaStreamCaptureStatusNone || ctx->ws_bytes[WS_ALN_BAND] >= bytes)
+            band = (uint32_t *)ws_get(ctx, WS_ALN_BAND, bytes);
+    }
     prof_begin(ctx, "sw_pass1");
     k_sw_score<<<blocks1, SW_THREADS, shm1, st>>>(d_qcodes, d_qoffsets, d_tcodes, d_toffsets, d_pairs, seg_start,
                                                   sflags, (int64_t)h_nseg, dmat,

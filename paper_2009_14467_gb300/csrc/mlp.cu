@@ -84,7 +84,8 @@ constexpr int TM = 64;                               // rows of a tile
 constexpr int MLP_GROUPS = 2;                        // groups of eight warps, a tile each
 constexpr int LDH = HID + 8, LDX = FEAT + 8;         // row pitches in shared memory
 constexpr int GROUP = 256, MLP_THREADS = MLP_GROUPS * GROUP;
-constexpr int PART = 3 * HID;                        // a CTA's partial sums: g_b1, g_b2, g_w3
+constexpr int PART = 3 * HID;                        // a slot's partial sums: g_b1, g_b2, g_w3
+constexpr int MLP_SLOTS = 152;                       // slots at most, a CTA each where there are as many SMs
 constexpr size_t MLP_SMEM = sizeof(__nv_bfloat16) * ((size_t)HID * LDH + FEAT * LDH + MLP_GROUPS * (TM * LDH + TM * LDX)) +
                             sizeof(float) * 3 * HID;
 
@@ -162,13 +163,15 @@ struct mlp_train_io {           // training only
     float pos_weight;
     __nv_bfloat16 *h1, *dh1, *dh2;   // n x 256 each, for the gradients of W1 and W2
     float *dz, *lrow;           // per row: the gradient at the logit, the loss term
-    float *part;                // PART floats per CTA
+    float *part;                // PART floats per slot
+    int slots;
 };
 
 // z[r] = the logit of row r.  TRAIN: the weighted logistic loss's terms and dz = w *
 // (sigmoid(z) - y) / n instead, the gradients dh2 = dz * w3 where layer 2 is active and dh1 = dh2 W2^T where
-// layer 1 is, and the gradients of W3 and its layers' biases as partial sums per CTA (fixed order,
-// so a training step is deterministic).  Measured on 10^6 rows: 3.99 ms with
+// layer 1 is, and the gradients of W3 and its layers' biases as partial sums per slot: the tiles go
+// to min(tiles, MLP_SLOTS) slots in turn, whatever the number of CTAs, and k_mlp_adam adds the
+// slots in order, so a training step gives the same bits on any number of SMs.  Measured on 10^6 rows: 3.99 ms with
 // one 64 x 64 tile and 2-byte loads a CTA and h1, h2 through memory, 0.355 ms so (137 GF:
 // 0.6 of the rate mma.sync reaches alone); a training step of 65,536 rows 28.1 ms with the
 // column sums in one CTA each, 0.35 ms so.
@@ -201,180 +204,184 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bf
     __syncthreads();
     const float b3 = net.b3[0];
     const uint32_t u_h = smem_u32(s_h), u_w1 = smem_u32(s_w1), u_w2 = smem_u32(s_w2), u_x = smem_u32(s_x);
-    // TRAIN: sums kept over the CTA's tiles
-    float gw3[8], gb2[8], gb1[16];
-    if constexpr (TRAIN) {
-#pragma unroll
-        for (int t = 0; t < 8; ++t) { gw3[t] = 0.f; gb2[t] = 0.f; }
-#pragma unroll
-        for (int t = 0; t < 16; ++t) gb1[t] = 0.f;
-    }
     const int64_t tiles = (n + TM - 1) / TM;
     const int xr = tid >> 1, xc = (tid & 1) * 8;         // 128 threads load 8 features of a tile each
     auto load_x = [&](int64_t tile) {
         const int64_t r = tile * TM + xr;
         return xr < TM && tile < tiles && r < n ? load8(x + r * FEAT + xc, xal) : make_uint4(0u, 0u, 0u, 0u);
     };
-    const int64_t step = (int64_t)gridDim.x * MLP_GROUPS, tile0 = (int64_t)group * gridDim.x + blockIdx.x;
-    uint4 xv = load_x(tile0);
-    for (int64_t tile = tile0; tile < tiles; tile += step) {
-        const int64_t r0 = tile * TM;
-        if (xr < TM) *reinterpret_cast<uint4 *>(s_x + xr * LDX + xc) = xv;
-        sync();                                          // x here; the group is done with its last tile
-        xv = load_x(tile + step);
-        // layer 1: one k step
-        uint32_t act[2] = {0u, 0u};                      // TRAIN: which of the warp's fragment values are active
-        {
-            uint32_t a[2][4];
-            ldsm4(a[0], u_x + (uint32_t)(((mw * 32 + (lane & 15)) * LDX + (lane >> 4) * 8) * 2));
-            ldsm4(a[1], u_x + (uint32_t)(((mw * 32 + 16 + (lane & 15)) * LDX + (lane >> 4) * 8) * 2));
+    const int slots = TRAIN ? tr.slots : (int)gridDim.x;
+    for (int slot = blockIdx.x; slot < slots; slot += gridDim.x) {
+        // TRAIN: sums kept over the slot's tiles
+        float gw3[8], gb2[8], gb1[16];
+        if constexpr (TRAIN) {
 #pragma unroll
-            for (int t = 0; t < 8; t += 2) {
-                uint32_t b[4];
-                ldsm4t(b, u_w1 + (uint32_t)(((lane & 15) * LDH + nw * 64 + t * 8 + (lane >> 4) * 8) * 2));
+            for (int t = 0; t < 8; ++t) { gw3[t] = 0.f; gb2[t] = 0.f; }
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        float c[4] = {0.f, 0.f, 0.f, 0.f};
-                        mma16816(c, a[i], b[2 * u], b[2 * u + 1]);
-                        const int col = nw * 64 + (t + u) * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
-                        const uint32_t lo = bias_relu2(c[0], c[1], s_b1 + col), hi = bias_relu2(c[2], c[3], s_b1 + col);
-                        *reinterpret_cast<uint32_t *>(s_h + row * LDH + col) = lo;
-                        *reinterpret_cast<uint32_t *>(s_h + (row + 8) * LDH + col) = hi;
-                        if constexpr (TRAIN) {           // stored halves are never negative: non-zero is active
-                            const uint32_t m = ((lo & 0x7FFFu) ? 1u : 0u) | ((lo & 0x7FFF0000u) ? 2u : 0u) |
-                                               ((hi & 0x7FFFu) ? 4u : 0u) | ((hi & 0x7FFF0000u) ? 8u : 0u);
-                            act[i] |= m << (4 * (t + u));
-                        }
-                    }
-            }
+            for (int t = 0; t < 16; ++t) gb1[t] = 0.f;
         }
-        sync();
-        if constexpr (TRAIN)
-            for (int i = tid; i < TM * (HID / 8); i += GROUP) {
-                const int64_t r = r0 + (i >> 5);
-                if (r < n)
-                    *reinterpret_cast<uint4 *>(tr.h1 + r * HID + (i & 31) * 8) =
-                        *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
-            }
-        float acc[2][8][4];
-        tile_product<false>(acc, u_h, u_w2, mw, nw, lane);
-        sync();                                 // h1 is read: h2 takes its place
+        const int64_t step = (int64_t)slots * MLP_GROUPS, tile0 = (int64_t)group * slots + slot;
+        uint4 xv = load_x(tile0);
+        for (int64_t tile = tile0; tile < tiles; tile += step) {
+            const int64_t r0 = tile * TM;
+            if (xr < TM) *reinterpret_cast<uint4 *>(s_x + xr * LDX + xc) = xv;
+            sync();                                          // x here; the group is done with its last tile
+            xv = load_x(tile + step);
+            // layer 1: one k step
+            uint32_t act[2] = {0u, 0u};                      // TRAIN: which of the warp's fragment values are active
+            {
+                uint32_t a[2][4];
+                ldsm4(a[0], u_x + (uint32_t)(((mw * 32 + (lane & 15)) * LDX + (lane >> 4) * 8) * 2));
+                ldsm4(a[1], u_x + (uint32_t)(((mw * 32 + 16 + (lane & 15)) * LDX + (lane >> 4) * 8) * 2));
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+                for (int t = 0; t < 8; t += 2) {
+                    uint32_t b[4];
+                    ldsm4t(b, u_w1 + (uint32_t)(((lane & 15) * LDH + nw * 64 + t * 8 + (lane >> 4) * 8) * 2));
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const int col = nw * 64 + t * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
-                *reinterpret_cast<uint32_t *>(s_h + row * LDH + col) = bias_relu2(acc[i][t][0], acc[i][t][1], s_b2 + col);
-                *reinterpret_cast<uint32_t *>(s_h + (row + 8) * LDH + col) =
-                    bias_relu2(acc[i][t][2], acc[i][t][3], s_b2 + col);
-            }
-        sync();
-        // the head: a warp takes 16 rows, a lane every 32nd column
-#pragma unroll 2
-        for (int q = 0; q < TM / 8; ++q) {
-            const int row = warp * (TM / 8) + q;
-            float h[8], s = 0.f;
+                    for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                h[t] = bf(s_h[row * LDH + lane + 32 * t]);
-                s += h[t] * s_w3[lane + 32 * t];
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-            const float zz = s + b3;
-            if (!TRAIN && r0 + row < n && lane == 0) z[r0 + row] = zz;
-            if constexpr (TRAIN) {
-                float d = 0.f;
-                if (r0 + row < n) {
-                    const float yy = tr.y[r0 + row];
-                    const float w = yy > 0.5f ? tr.pos_weight : 1.f;
-                    const float sg = 1.f / (1.f + __expf(-zz));
-                    d = w * (sg - yy) / (float)n;
-                    const float sp = zz > 0.f ? zz + log1pf(__expf(-zz)) : log1pf(__expf(zz));
-                    if (lane == 0) {
-                        tr.dz[r0 + row] = d;
-                        tr.lrow[r0 + row] = w * (sp - yy * zz) / (float)n;
-                    }
+                        for (int u = 0; u < 2; ++u) {
+                            float c[4] = {0.f, 0.f, 0.f, 0.f};
+                            mma16816(c, a[i], b[2 * u], b[2 * u + 1]);
+                            const int col = nw * 64 + (t + u) * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
+                            const uint32_t lo = bias_relu2(c[0], c[1], s_b1 + col), hi = bias_relu2(c[2], c[3], s_b1 + col);
+                            *reinterpret_cast<uint32_t *>(s_h + row * LDH + col) = lo;
+                            *reinterpret_cast<uint32_t *>(s_h + (row + 8) * LDH + col) = hi;
+                            if constexpr (TRAIN) {           // stored halves are never negative: non-zero is active
+                                const uint32_t m = ((lo & 0x7FFFu) ? 1u : 0u) | ((lo & 0x7FFF0000u) ? 2u : 0u) |
+                                                   ((hi & 0x7FFFu) ? 4u : 0u) | ((hi & 0x7FFF0000u) ? 8u : 0u);
+                                act[i] |= m << (4 * (t + u));
+                            }
+                        }
                 }
+            }
+            sync();
+            if constexpr (TRAIN)
+                for (int i = tid; i < TM * (HID / 8); i += GROUP) {
+                    const int64_t r = r0 + (i >> 5);
+                    if (r < n)
+                        *reinterpret_cast<uint4 *>(tr.h1 + r * HID + (i & 31) * 8) =
+                            *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
+                }
+            float acc[2][8][4];
+            tile_product<false>(acc, u_h, u_w2, mw, nw, lane);
+            sync();                                 // h1 is read: h2 takes its place
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
-                    const bool on = r0 + row < n && h[t] > 0.f;
-                    const __nv_bfloat16 dv = __float2bfloat16(on ? d * s_w3[lane + 32 * t] : 0.f);
-                    s_h[row * LDH + lane + 32 * t] = dv;
-                    gw3[t] += h[t] * d;              // d = 0 past the batch
-                    gb2[t] += bf(dv);
+                    const int col = nw * 64 + t * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
+                    *reinterpret_cast<uint32_t *>(s_h + row * LDH + col) = bias_relu2(acc[i][t][0], acc[i][t][1], s_b2 + col);
+                    *reinterpret_cast<uint32_t *>(s_h + (row + 8) * LDH + col) =
+                        bias_relu2(acc[i][t][2], acc[i][t][3], s_b2 + col);
+                }
+            sync();
+            // the head: a warp takes 16 rows, a lane every 32nd column
+#pragma unroll 2
+            for (int q = 0; q < TM / 8; ++q) {
+                const int row = warp * (TM / 8) + q;
+                float h[8], s = 0.f;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    h[t] = bf(s_h[row * LDH + lane + 32 * t]);
+                    s += h[t] * s_w3[lane + 32 * t];
+                }
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+                const float zz = s + b3;
+                if (!TRAIN && r0 + row < n && lane == 0) z[r0 + row] = zz;
+                if constexpr (TRAIN) {
+                    float d = 0.f;
+                    if (r0 + row < n) {
+                        const float yy = tr.y[r0 + row];
+                        const float w = yy > 0.5f ? tr.pos_weight : 1.f;
+                        const float sg = 1.f / (1.f + __expf(-zz));
+                        d = w * (sg - yy) / (float)n;
+                        const float sp = zz > 0.f ? zz + log1pf(__expf(-zz)) : log1pf(__expf(zz));
+                        if (lane == 0) {
+                            tr.dz[r0 + row] = d;
+                            tr.lrow[r0 + row] = w * (sp - yy * zz) / (float)n;
+                        }
+                    }
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) {
+                        const bool on = r0 + row < n && h[t] > 0.f;
+                        const __nv_bfloat16 dv = __float2bfloat16(on ? d * s_w3[lane + 32 * t] : 0.f);
+                        s_h[row * LDH + lane + 32 * t] = dv;
+                        gw3[t] += h[t] * d;              // d = 0 past the batch
+                        gb2[t] += bf(dv);
+                    }
                 }
             }
+            if constexpr (TRAIN) {
+                sync();
+                for (int i = tid; i < TM * (HID / 8); i += GROUP) {
+                    const int64_t r = r0 + (i >> 5);
+                    if (r < n)
+                        *reinterpret_cast<uint4 *>(tr.dh2 + r * HID + (i & 31) * 8) =
+                            *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
+                }
+                tile_product<true>(acc, u_h, u_w2, mw, nw, lane);
+                sync();                             // dh2 is read: dh1 takes its place
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int col = nw * 64 + t * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
+                        const uint32_t m = act[i] >> (4 * t);
+                        float v[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) v[q] = (m >> q) & 1u ? acc[i][t][q] : 0.f;
+                        gb1[2 * t] += v[0] + v[2];
+                        gb1[2 * t + 1] += v[1] + v[3];
+                        __nv_bfloat162 p0, p1;
+                        p0.x = __float2bfloat16(v[0]); p0.y = __float2bfloat16(v[1]);
+                        p1.x = __float2bfloat16(v[2]); p1.y = __float2bfloat16(v[3]);
+                        *reinterpret_cast<__nv_bfloat162 *>(s_h + row * LDH + col) = p0;
+                        *reinterpret_cast<__nv_bfloat162 *>(s_h + (row + 8) * LDH + col) = p1;
+                    }
+                }
+                sync();
+                for (int i = tid; i < TM * (HID / 8); i += GROUP) {
+                    const int64_t r = r0 + (i >> 5);
+                    if (r < n)
+                        *reinterpret_cast<uint4 *>(tr.dh1 + r * HID + (i & 31) * 8) =
+                            *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
+                }
+            }
+            sync();                                 // s_x and s_h are free
         }
         if constexpr (TRAIN) {
-            sync();
-            for (int i = tid; i < TM * (HID / 8); i += GROUP) {
-                const int64_t r = r0 + (i >> 5);
-                if (r < n)
-                    *reinterpret_cast<uint4 *>(tr.dh2 + r * HID + (i & 31) * 8) =
-                        *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
-            }
-            tile_product<true>(acc, u_h, u_w2, mw, nw, lane);
-            sync();                             // dh2 is read: dh1 takes its place
+            // the slot's partial sums, through shared memory: [16 warps][256] g_b2, the same g_w3,
+            // [2 groups x 2][256] g_b1
+            __syncthreads();
+            constexpr int W = MLP_THREADS / 32;
+            const int aw = threadIdx.x >> 5;
+            float *part = tr.part + (int64_t)slot * PART;
+            float *s_red = reinterpret_cast<float *>(s_w1 + FEAT * LDH);
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int col = nw * 64 + t * 8 + tig * 2, row = mw * 32 + i * 16 + gid;
-                    const uint32_t m = act[i] >> (4 * t);
-                    float v[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) v[q] = (m >> q) & 1u ? acc[i][t][q] : 0.f;
-                    gb1[2 * t] += v[0] + v[2];
-                    gb1[2 * t + 1] += v[1] + v[3];
-                    __nv_bfloat162 p0, p1;
-                    p0.x = __float2bfloat16(v[0]); p0.y = __float2bfloat16(v[1]);
-                    p1.x = __float2bfloat16(v[2]); p1.y = __float2bfloat16(v[3]);
-                    *reinterpret_cast<__nv_bfloat162 *>(s_h + row * LDH + col) = p0;
-                    *reinterpret_cast<__nv_bfloat162 *>(s_h + (row + 8) * LDH + col) = p1;
-                }
+                s_red[aw * HID + lane + 32 * t] = gb2[t];
+                s_red[(W + aw) * HID + lane + 32 * t] = gw3[t];
             }
-            sync();
-            for (int i = tid; i < TM * (HID / 8); i += GROUP) {
-                const int64_t r = r0 + (i >> 5);
-                if (r < n)
-                    *reinterpret_cast<uint4 *>(tr.dh1 + r * HID + (i & 31) * 8) =
-                        *reinterpret_cast<const uint4 *>(s_h + (i >> 5) * LDH + (i & 31) * 8);
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {                   // over the eight rows' lanes of a column
+                float v = gb1[t];
+                v += __shfl_xor_sync(0xffffffffu, v, 4);
+                v += __shfl_xor_sync(0xffffffffu, v, 8);
+                v += __shfl_xor_sync(0xffffffffu, v, 16);
+                if (gid == 0) s_red[(2 * W + group * 2 + mw) * HID + nw * 64 + (t >> 1) * 8 + tig * 2 + (t & 1)] = v;
             }
-        }
-        sync();                                 // s_x and s_h are free
-    }
-    if constexpr (TRAIN) {
-        // the CTA's partial sums, through shared memory: [16 warps][256] g_b2, the same g_w3,
-        // [2 groups x 2][256] g_b1
-        __syncthreads();
-        constexpr int W = MLP_THREADS / 32;
-        const int aw = threadIdx.x >> 5;
-        float *part = tr.part + (int64_t)blockIdx.x * PART;
-        float *s_red = reinterpret_cast<float *>(s_w1 + FEAT * LDH);
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            s_red[aw * HID + lane + 32 * t] = gb2[t];
-            s_red[(W + aw) * HID + lane + 32 * t] = gw3[t];
-        }
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {                   // over the eight rows' lanes of a column
-            float v = gb1[t];
-            v += __shfl_xor_sync(0xffffffffu, v, 4);
-            v += __shfl_xor_sync(0xffffffffu, v, 8);
-            v += __shfl_xor_sync(0xffffffffu, v, 16);
-            if (gid == 0) s_red[(2 * W + group * 2 + mw) * HID + nw * 64 + (t >> 1) * 8 + tig * 2 + (t & 1)] = v;
-        }
-        __syncthreads();
-        if (group == 0) {
-            float a = 0.f, b = 0.f, c = 0.f;
-            for (int w = 0; w < W; ++w) { a += s_red[w * HID + tid]; b += s_red[(W + w) * HID + tid]; }
-            for (int w = 0; w < 2 * MLP_GROUPS; ++w) c += s_red[(2 * W + w) * HID + tid];
-            part[tid] = c;
-            part[HID + tid] = a;
-            part[2 * HID + tid] = b;
+            __syncthreads();
+            if (group == 0) {
+                float a = 0.f, b = 0.f, c = 0.f;
+                for (int w = 0; w < W; ++w) { a += s_red[w * HID + tid]; b += s_red[(W + w) * HID + tid]; }
+                for (int w = 0; w < 2 * MLP_GROUPS; ++w) c += s_red[(2 * W + w) * HID + tid];
+                part[tid] = c;
+                part[HID + tid] = a;
+                part[2 * HID + tid] = b;
+            }
+            __syncthreads();                        // the next slot's tiles take their place
         }
     }
 }
@@ -537,7 +544,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_mlp_wgrad(const __nv_bfloat16
 }
 
 // Every parameter's Adam step on its float32 master, with the gradients of W3 and of the
-// biases of layers 1 and 2 summed here from the CTAs' partial sums (in order); refreshes the
+// biases of layers 1 and 2 summed here from the slots' partial sums (in order); refreshes the
 // bf16 copies.
 struct adam_args {
     float *w1, *b1, *w2, *b2, *w3, *b3;
@@ -656,9 +663,9 @@ extern "C" pastis_status pastis_mlp_train_step(pastis_ctx *ctx, pastis_mlp *net,
     if (!ctx || !net || n <= 0 || n > (1 << 22) || !d_x || !d_y) return PASTIS_ERR_INVALID_ARG;
     cudaStream_t st = ctx->stream;
     // scratch: h1, dh1 and dh2 (bf16 n x 256), dz and the loss terms, the partial sums of the gradients
-    const int grid = (int)std::min<int64_t>(ceil_div64(n, TM), ctx->sm_count);
+    const int slots = (int)std::min<int64_t>(ceil_div64(n, TM), MLP_SLOTS), grid = std::min(slots, ctx->sm_count);
     const size_t act = (size_t)n * HID * 2, zb = ((size_t)n * 4 + 255) & ~(size_t)255;
-    const size_t pb = ((size_t)grid * PART * 4 + 255) & ~(size_t)255;
+    const size_t pb = ((size_t)slots * PART * 4 + 255) & ~(size_t)255;
     char *b;
     PASTIS_WS(b, ctx, WS_MLP, 3 * act + 2 * zb + pb);
     mlp_train_io tr;
@@ -670,6 +677,7 @@ extern "C" pastis_status pastis_mlp_train_step(pastis_ctx *ctx, pastis_mlp *net,
     tr.dz = (float *)(b + 3 * act);
     tr.lrow = (float *)(b + 3 * act + zb);
     tr.part = (float *)(b + 3 * act + 2 * zb);
+    tr.slots = slots;
     prof_begin(ctx, "mlp_train");
     k_mlp<true><<<grid, MLP_THREADS, MLP_SMEM, st>>>(mlp_weights(net), (const __nv_bfloat16 *)d_x, n, nullptr, tr);
     PASTIS_LAUNCHED(ctx);
@@ -690,7 +698,7 @@ extern "C" pastis_status pastis_mlp_train_step(pastis_ctx *ctx, pastis_mlp *net,
     a.c2 = 1.f - powf(a.beta2, (float)net->step);
     const int np = FEAT * HID + HID * HID + 3 * HID + 1;
     prof_begin(ctx, "mlp_adam");
-    k_mlp_adam<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(a, tr.part, grid);
+    k_mlp_adam<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(a, tr.part, slots);
     PASTIS_LAUNCHED(ctx);
     prof_end(ctx);
     return PASTIS_OK;

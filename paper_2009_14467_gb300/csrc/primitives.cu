@@ -428,15 +428,20 @@ __global__ void k_find_col_ptr(const uint32_t *__restrict__ keys, const uint32_t
 pastis_status fill_col_ptr(pastis_ctx *c, const uint32_t *keys, const uint32_t *keep_off, int64_t n, int64_t ncodes,
                            uint32_t *col_ptr) {
     prof_begin(c, "col_ptr");
-    // Too few tiles to fill the SMs (k <= 4), or more entries than codes, so that a tile has a
-    // long stretch of keys: one search per code instead.  7.6 M entries over 24^4 codes: 17 us
-    // so, 1,139 us in 41 tiles; over the 8 M codes of k = 5 the searches take 188 us with 20 M
-    // entries, the tiles 433, and with 7.6 M (tiles) 168 and 196.
-    if (n > ncodes || ceil_div64(ncodes + 1, CP_TILE) < 2 * (int64_t)c->sm_count)
+    // A search per code instead where there are too few tiles to fill the SMs (k <= 4), or where
+    // the tiles' stretches of keys take longer than the searches, which hardly depend on the
+    // keys.  With less than a few waves of tiles (k = 5, 6 tiles an SM) the CTAs of the frequent
+    // residues finish last, and that is so from about one key a code on; where the tiles fill the
+    // SMs many times over (k = 6, 153 an SM) they are read at bandwidth and it takes six.
+    // Measured on residues at their natural frequencies, tiles and searches in us: k = 4, 1 M
+    // keys 110 and 12; k = 5, 8 M codes: 4 M keys 82 and 148, 7.6 M 164 and 167, 20 M 382 and
+    // 188, 300 M 3,129 and 285; k = 6, 191 M codes: 35 M keys 356 and 3,665, 350 M 1,866 and
+    // 4,440, 1 G 4,171 and 4,835, 1.2 G 4,780 and 5,016.
+    const int64_t tiles = ceil_div64(ncodes + 1, CP_TILE), sms = c->sm_count;
+    if (tiles < 2 * sms || n > ncodes * (tiles < 32 * sms ? 1 : 6))
         k_find_col_ptr<<<(unsigned)ceil_div64(ncodes + 1, 256), 256, 0, c->stream>>>(keys, keep_off, n, ncodes, col_ptr);
     else
-        k_fill_col_ptr<<<(unsigned)ceil_div64(ncodes + 1, CP_TILE), CP_THREADS, 0, c->stream>>>(keys, keep_off, n, ncodes,
-                                                                                           col_ptr);
+        k_fill_col_ptr<<<(unsigned)tiles, CP_THREADS, 0, c->stream>>>(keys, keep_off, n, ncodes, col_ptr);
     PASTIS_LAUNCHED(c);
     prof_end(c);
     return PASTIS_OK;

@@ -507,7 +507,10 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
         }
     }
     const int lim = x.best - X;
-    const uint32_t lim2 = xd16_pk(lim), limm2 = __vsub2(lim2, 0x00010001u);
+    // lim - 1 is formed before it is replicated, not as lim2 less a packed one: given that relation,
+    // nvcc 13.0.88 (build 36424714) used lim2 for limm2 in some of the unrolled registers below,
+    // depending on the code around them, and a row past the limit stayed alive there
+    const uint32_t lim2 = xd16_pk(lim), limm2 = xd16_pk(lim - 1);
     const uint32_t rb2 = xd16_pk(a0 - clo), span2 = xd16_pk(chi - clo);
     // the sources on d - 1 that cross a lane boundary
     uint32_t bh, bx, bhc = 0u, bxc = 0u;
@@ -588,8 +591,6 @@ __device__ __forceinline__ void xd16_step(xd16_ext<R, C> &x, int ls, unsigned sm
         // dead halves: H < lim, or the row outside [clo, chi]; the sign of the smallest of
         // row - clo, chi - row and max(H, lim - 1) - lim, replicated
         const uint32_t rr = __vadd2(rb2, (uint32_t)((2 * r) | ((2 * r + 1) << 16)));
-        // (chi - row from row - clo by a subtraction of registers: from chi - a0 less a constant,
-        // this compiler left rows past chi alive with two extensions a warp)
         const uint32_t rs = __vsub2(span2, rr);
         const uint32_t dm = xd16_signs(__vimin3_s16x2(rr, rs, __vsub2(__vmaxs2(hn, limm2), lim2)));
         x.H[P][r] = (__vsub2(hn, o2) & ~dm) | (XD16_NEG2 & dm);

@@ -383,6 +383,7 @@ __global__ void __launch_bounds__(MLP_THREADS, 1) k_mlp(mlp_w net, const __nv_bf
             }
             __syncthreads();                        // the next slot's tiles take their place
         }
+        if constexpr (!TRAIN) break;                // a slot a CTA
     }
 }
 

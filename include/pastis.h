@@ -172,8 +172,8 @@ int32_t pastis_ctx_profile_read(pastis_ctx *ctx, char *buf, int32_t len);
  * roofline of the overlap product: h_out[0] = posting entries visited (products),
  * [1] = left-operand entries of the rows formed (each once per row; of A S those kept: the
  * substitutes that A holds), [2] = candidate records written, [3] = radix-sort element
- * passes of the k-mer matrix builds (A and AS: elements sorted x 8-bit digit passes).  Entries past the fourth are 0.  Synchronises
- * the stream.                                                                             */
+ * passes of the k-mer matrix builds (A and AS: elements sorted x passes, one for every 8
+ * bits of the key or part of them).  Entries past the fourth are 0.  Synchronises the stream. */
 #define PASTIS_STATS 4
 pastis_status pastis_ctx_stats(pastis_ctx *ctx, int64_t *h_out, int32_t n);
 

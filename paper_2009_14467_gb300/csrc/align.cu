@@ -350,8 +350,8 @@ __device__ bool xd_diag_warp(const uint8_t *q, int A, int qs, const uint8_t *t, 
 // What bounds both forms is the integer pipe (ncu: 85% busy, 3.0 instructions a cycle).
 // Measured on 2 M exact candidates of 200,000 proteins: first phase 63.8 ms with separate
 // range and limit masks, dead E and F cleared, and the best score reduced in every step,
-// 53.1 ms so; second phase 14.5 ms with one 32-bit word of statistics per cell, 11.9 ms so;
-// 300,000 family-rich pairs with carries throughout 25.8 -> 20.6 ms.  A window that leaves
+// 51.5 ms so; second phase 14.5 ms with one 32-bit word of statistics per cell, 11.6 ms so;
+// 300,000 family-rich pairs with carries throughout 25.8 -> 20.3 ms.  A window that leaves
 // its range is centred to the nearest lane (16 diagonals with four extensions a warp): the
 // 32-bit kernel's share was 4.1 and 1.2 ms with the shift cut towards zero and is 1.9 and
 // 0.9 ms so.  Shifting by single registers as well leaves 1.1 and 0.6 ms there but takes 3.3

@@ -127,7 +127,7 @@ static inline int64_t ipow24(int k) {
     return v;
 }
 
-// Device radix sort (LSD, 8-bit digits, stable) of (uint32 key, uint64 value) pairs.
+// Device radix sort (LSD, digits of 5 to 8 bits, stable) of (uint32 key, uint64 value) pairs.
 // Sorts keys[0..n) by bits [0, key_bits); the result lands in *keys_out/*vals_out,
 // which point at either the input arrays or the two alternate arrays.
 pastis_status radix_sort_u32_u64(pastis_ctx *c, uint32_t *keys, uint64_t *vals,

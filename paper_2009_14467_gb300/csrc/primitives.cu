@@ -430,9 +430,9 @@ pastis_status fill_col_ptr(pastis_ctx *c, const uint32_t *keys, const uint32_t *
     prof_begin(c, "col_ptr");
     // A search per code instead where there are too few tiles to fill the SMs (k <= 4), or where
     // the tiles' stretches of keys take longer than the searches, which hardly depend on the
-    // keys.  With less than a few waves of tiles (k = 5, 6 tiles an SM) the CTAs of the frequent
-    // residues finish last, and that is so from about one key a code on; where the tiles fill the
-    // SMs many times over (k = 6, 153 an SM) they are read at bandwidth and it takes six.
+    // keys: from one key a code on with a wave or two of tiles (k = 5, 6 tiles an SM), whose
+    // longest, those of the frequent residues, finish late; from six where the tiles fill the SMs
+    // many times over (k = 6, 153 an SM).
     // Measured on residues at their natural frequencies, tiles and searches in us: k = 4, 1 M
     // keys 110 and 12; k = 5, 8 M codes: 4 M keys 82 and 148, 7.6 M 164 and 167, 20 M 382 and
     // 188, 300 M 3,129 and 285; k = 6, 191 M codes: 35 M keys 356 and 3,665, 350 M 1,866 and

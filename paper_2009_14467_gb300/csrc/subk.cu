@@ -97,9 +97,12 @@ __device__ __noinline__ int subk_cut_far(const uint8_t *s_hist, uint32_t digs, i
     return -1;
 }
 
-// One thread per root.  What bounds it is instruction issue: about 700 multiply-adds of
-// phase 1 (16 distances hold the cut of nearly every root with BLOSUM62; the others are
-// counted again over all 64) and a dozen instructions for each step of the walk.  A bit
+// One thread per root: about 700 multiply-adds of phase 1 (16 distances hold the cut of
+// nearly every root with BLOSUM62; the others are counted again over all 64) and a dozen
+// instructions for each step of the walk.  What bounds it is the walks' divergence: 12.5 of 32
+// lanes are active in an instruction and the issue slots are two thirds busy; the rest is
+// branches and dependent steps that 18 warps an SM (their rows in shared memory) do not
+// hide.  A bit
 // mask per (residue, budget) names the replacements that keep a prefix within the cut,
 // so the walk touches only prefixes that lead to a k-mer it keeps or a tie at the cut;
 // its stack, the running slot of each distance and the rows under construction live in

@@ -92,9 +92,11 @@ __global__ void k_seg_flags(const pastis_cand *pairs, int64_t n, uint32_t *flags
 }
 
 // Segments run in order of query length, longest first (bins of 16 residues): the CTAs at
-// work at one time then run the same few of pass 1's sixteen loop bodies, which together
-// exceed the instruction cache (pass 1 of 10^6 pairs 51.2 ms in input order, 46.9 ms so),
-// and the last segments taken are the shortest.
+// work at one time then run the same few of pass 1's loop bodies (16 row counts for each of 8,
+// 16 and 32 lanes, and for 32 lanes in stripes), which together exceed the instruction cache,
+// and the last segments taken are the shortest.  Pass 1 in input order and so: 10^6 pairs of
+// 20,000 proteins 49.0 and 44.1 ms, 10^5 of 1,000 residues 27.6 and 25.2 ms, of 5,000 proteins
+// 56.9 and 54.6 ms.
 constexpr int SEG_BINS = 128;
 __device__ __forceinline__ int seg_bin(int64_t m) { return SEG_BINS - 1 - (int)min((int64_t)SEG_BINS - 1, m >> 4); }
 
@@ -271,8 +273,8 @@ __device__ __forceinline__ uint32_t column2(const uint8_t *__restrict__ pa, cons
 // larger, one less for the holder and the lanes before it, and never less than `none`, what
 // a cell of H = 0 holds.  (A half without a pair has no other cells: one less than those,
 // every later column called for this function, and the last grab of a run of 17 or 18 pairs took
-// a third longer: 10^6 cells a ms 990 at 60 residues and 18 pairs a query, 1,395 so; 1,623 and
-// 2,138 at 120.)
+// a third longer: 990 GCUPS at 60 residues and 18 pairs a query, 1,395 so; 1,623 and 2,138 at
+// 120.)
 template <int G, int LR, bool HI>
 __device__ __forceinline__ int note_best(const uint32_t (&Ho)[LR], bool mine, int row0, int j, int lg, uint32_t sh16,
                                          int none, int &bv, int &brow, int &bcol) {

@@ -15,7 +15,7 @@ MAT = synth.blosum62()
 SLACK = 64 << 20                     # rounding of a dozen allocations, and the call's output
 
 
-def _work(P, n_pairs, q_len, seed):
+def _set(P, n_pairs, q_len, seed):
     rng = np.random.default_rng(seed)
     lens = np.concatenate([np.full(8, q_len), rng.integers(10, 61, 500)])
     offs = np.zeros(len(lens) + 1, np.int64)
@@ -43,7 +43,7 @@ def _with_room(room, call):
 
 def test_bands_never_take_the_room_of_a_needed_buffer():
     import paper_2009_14467_gb300 as P
-    codes, offs, pairs = _work(P, 400_000, 1000, 1)
+    codes, offs, pairs = _set(P, 400_000, 1000, 1)
     need, full = P.Params(matrix=MAT, mode=P.SW_SCORE), P.Params(matrix=MAT, mode=P.SW)
     ctx = P.Context(0)
     P.align_pairs(ctx, codes, offs, pairs, need)
@@ -61,8 +61,8 @@ def test_bands_never_take_the_room_of_a_needed_buffer():
 
 def test_bands_of_an_earlier_call_make_room():
     import paper_2009_14467_gb300 as P
-    codes, offs, pairs = _work(P, 400_000, 1000, 2)
-    big = _work(P, 1000, 3000, 3)
+    codes, offs, pairs = _set(P, 400_000, 1000, 2)
+    big = _set(P, 1000, 3000, 3)
     need, full = P.Params(matrix=MAT, mode=P.SW_SCORE), P.Params(matrix=MAT, mode=P.SW)
     ctx = P.Context(0)
     want = P.align_pairs(ctx, *big, need).cpu()
